@@ -135,16 +135,10 @@ __global__ void __launch_bounds__(Tile<2, (int)sizeof(R)>::THREADS) k_batch_cfl(
             if (gx < I.g.n[0] && gy < I.g.n[1]) {
                 const R *U = reinterpret_cast<const R *>(b.in) + I.off;
                 const long long c = gx + (long long)I.g.n[0] * gy;
-                R q[L::NVAR], wv[L::NVAR];
+                R q[L::NVAR], cs;
 #pragma unroll
                 for (int v = 0; v < L::NVAR; v++) q[v] = U[v * I.g.pitch + c];
-                cons_to_prim<R, 2, NMAT, false>(I.g, q, wv);
-                State<R, 2, NMAT, false> s;
-                state_from_prim<R, 2, NMAT, false>(I.g, wv, s);
-                const R cs = m_sqrt(s.c2);
-                R sum = R(0);
-#pragma unroll
-                for (int d = 0; d < 2; d++) sum += (m_abs(s.u[d]) + cs) / gridc<R>(I.g).dx[d];
+                const R sum = cell_speed<R, 2, NMAT, false>(I.g, q, cs);
                 double sd = (double)sum;
                 if (!(sd == sd)) sd = __longlong_as_double(0x7ff0000000000000LL);
                 red[0] = sd;

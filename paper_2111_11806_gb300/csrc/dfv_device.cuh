@@ -37,6 +37,12 @@ struct MatC {
     T invGam;       // 1 / Gam
     T pref0;        // constant p_ref of the gases (-gamma p_inf, 0)
     T rho0, K0, G0, alpha, beta, sigY;
+    // products of the constants that the closures use, so that they divide by
+    // nothing: 1 + 1/Gam, p_ref/Gam (gases), 1/rho0, K0/(2 alpha^2), K0/alpha,
+    // 1/alpha, beta + 1, beta (beta + 1)
+    T Gam1;         // 1 + Gam
+    T kA, kB, irho0, kE, kP, ialpha, beta1, bb;
+    int n_alpha, n_beta1;   // alpha, beta + 1 where they are whole numbers 1..8, else 0
     int has_rho0;
 };
 
@@ -72,6 +78,12 @@ struct GridP {
     int any_jc;         // some material has a Johnson-Cook flow stress
 };
 
+// an exponent that is one of the whole numbers 1..8, else 0
+__host__ inline int whole_power(double e)
+{
+    return e >= 1.0 && e <= 8.0 && e == std::floor(e) ? (int)e : 0;
+}
+
 template <class T>
 __host__ inline void fill_consts(const GridP &g, MatC<T> *mc, GridC<T> &gc)
 {
@@ -88,6 +100,18 @@ __host__ inline void fill_consts(const GridP &g, MatC<T> *mc, GridC<T> &gc)
         mc[l].beta = (T)m.beta;
         mc[l].sigY = (T)m.sigY;
         mc[l].has_rho0 = m.rho0 > 0.0;
+        const double iG = 1.0 / (m.kind == 2 ? m.Gamma0 : m.gamma - 1.0);
+        mc[l].Gam1 = (T)(1.0 + (m.kind == 2 ? m.Gamma0 : m.gamma - 1.0));
+        mc[l].kA = (T)(1.0 + iG);
+        mc[l].kB = m.kind == 1 ? (T)(-m.gamma * m.pinf * iG) : T(0);
+        mc[l].irho0 = m.rho0 > 0.0 ? (T)(1.0 / m.rho0) : T(0);
+        mc[l].kE = m.alpha != 0.0 ? (T)(m.K0 / (2.0 * m.alpha * m.alpha)) : T(0);
+        mc[l].kP = m.alpha != 0.0 ? (T)(m.K0 / m.alpha) : T(0);
+        mc[l].ialpha = m.alpha != 0.0 ? (T)(1.0 / m.alpha) : T(0);
+        mc[l].beta1 = (T)(m.beta + 1.0);
+        mc[l].bb = (T)(m.beta * (m.beta + 1.0));
+        mc[l].n_alpha = whole_power(m.alpha);
+        mc[l].n_beta1 = whole_power(m.beta + 1.0);
     }
     for (int d = 0; d < 3; d++) {
         gc.lo[d] = (T)g.lo[d];
@@ -305,6 +329,18 @@ struct Lay {
     static constexpr int NF = NVAR + 1 + NB;     // per-face record: fluxes, u*_d, V*_{d.}
 };
 
+// FP32 mixtures of fluids.  Their phasic density (phi rho)_l/phi_l beside an
+// interface, where phi_l is some 1e-6, carries the rounding noise of its two
+// transported factors magnified (1e-3 of the density at single cells), so
+// that any other order of rounding gives another noise; their closures, fluxes
+// and reconstruction keep one fixed order of operations, apart from those of
+// the other forms.
+template <class T, int NMAT, int SOLID>
+__host__ __device__ constexpr bool mix32()
+{
+    return sizeof(T) == 4 && NMAT >= 2 && SOLID == 0;
+}
+
 // stored stretch component c -> tensor indices (a, b)
 __host__ __device__ constexpr int v_row(int dim, int c)
 {
@@ -317,7 +353,6 @@ __host__ __device__ constexpr int v_col(int dim, int c)
 
 // ------------------------------------------------------------------ math
 
-__device__ __forceinline__ double m_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float m_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double m_exp(double x) { return exp(x); }
 __device__ __forceinline__ float m_exp(float x) { return expf(x); }
@@ -334,10 +369,111 @@ __device__ __forceinline__ double m_pow(double x, double y) { return pow(x, y); 
 __device__ __forceinline__ float m_pow(float x, float y) { return powf(x, y); }
 __device__ __forceinline__ double m_abs(double x) { return fabs(x); }
 __device__ __forceinline__ float m_abs(float x) { return fabsf(x); }
-__device__ __forceinline__ double m_min(double a, double b) { return fmin(a, b); }
+__device__ __forceinline__ double m_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float m_fma(float a, float b, float c) { return fmaf(a, b, c); }
+
+// The FP64 pipe is what bounds the FP64 form (two lanes per SM and clock: an
+// FP64 instruction of a warp takes the time of 64 others), so what can be done
+// elsewhere is: reciprocals and roots start from the special-function unit's
+// approximation and take one third-order step (Chebyshev's iteration: the
+// relative error e of the start becomes e^3; e < 2^-19), and comparisons and
+// selections work on the bits.
+
+// 1/x: y (1 + e + e^2), e = 1 - x y
+__device__ __forceinline__ double m_rcp(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float m_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// comparisons on the bits, with those of the ordinary operators: false for a
+// NaN, zero of either sign equal to zero
+__device__ __forceinline__ unsigned long long m_bits(double x) { return (unsigned long long)__double_as_longlong(x); }
+constexpr unsigned long long M_INF = 0x7ff0000000000000ull, M_SIGN = 0x8000000000000000ull;
+__device__ __forceinline__ bool m_pos(double x) { return m_bits(x) - 1ull < M_INF; }                  // x > 0
+__device__ __forceinline__ bool m_pos(float x) { return x > 0.f; }
+__device__ __forceinline__ bool m_neg(double x) { return m_bits(x) - (M_SIGN + 1ull) < M_INF; }       // x < 0
+__device__ __forceinline__ bool m_neg(float x) { return x < 0.f; }
+__device__ __forceinline__ bool m_ge0(double x) { return m_bits(x) <= M_INF || m_bits(x) == M_SIGN; }  // x >= 0
+__device__ __forceinline__ bool m_ge0(float x) { return x >= 0.f; }
+__device__ __forceinline__ bool m_zero(double x) { return (m_bits(x) << 1) == 0ull; }                 // x == 0
+__device__ __forceinline__ bool m_over1(double x)                                                     // x > 1
+{
+    return m_bits(x) - 0x3ff0000000000001ull < M_INF - 0x3ff0000000000000ull;
+}
+__device__ __forceinline__ bool m_over1(float x) { return x > 1.f; }
+__device__ __forceinline__ bool m_nan(double x) { return (__double2hiint(x) & 0x7fffffff) >= 0x7ff80000; }  // quiet NaN
+// whether a < b, neither a NaN; the bits of doubles, negative ones with their magnitude inverted, order like them
+__device__ __forceinline__ long long m_key(double x)
+{
+    const long long k = __double_as_longlong(x);
+    return k ^ ((k >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ bool m_less(double a, double b) { return m_key(a) < m_key(b); }
+__device__ __forceinline__ bool m_less(float a, float b) { return a < b; }
+__device__ __forceinline__ double m_sel(bool c, double a, double b)
+{
+    return __longlong_as_double(c ? __double_as_longlong(a) : __double_as_longlong(b));
+}
+__device__ __forceinline__ float m_sel(bool c, float a, float b) { return c ? a : b; }
+// minimum and maximum that pass over a NaN, as fmin and fmax do: a state of
+// negative c^2 then leaves the wave speeds to the other side of its face
+__device__ __forceinline__ double m_min(double a, double b)
+{
+    return m_sel(m_nan(b) || (!m_nan(a) && m_less(a, b)), a, b);
+}
 __device__ __forceinline__ float m_min(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double m_max(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ double m_max(double a, double b)
+{
+    return m_sel(m_nan(b) || (!m_nan(a) && m_less(b, a)), a, b);
+}
 __device__ __forceinline__ float m_max(float a, float b) { return fmaxf(a, b); }
+
+// sqrt(x): x/sqrt(x), the reciprocal root with the third-order step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2
+__device__ __forceinline__ double m_sqrt(double x)
+{
+    if (m_pos(x) && m_less(x, 1e-290)) return sqrt(x);   // the start flushes subnormals to 0
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double c = x * y;
+    const double e = fma(-c, y, 1.0);
+    const double r = fma(c, e * fma(e, 0.375, 0.5), c);
+    return m_sel(m_zero(x), 0.0, r);
+}
+
+// sqrt(a/b), b > 0: a / sqrt(a b) with the reciprocal root's start y and its
+// third-order step y (1 + e/2 + 3 e^2/8), e = 1 - a b y^2
+__device__ __forceinline__ double m_sqrt_ratio(double a, double b)
+{
+    const double x = a * b;
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    const double c = a * y;
+    const double r = fma(c, e * fma(e, 0.375, 0.5), c);
+    return m_sel(m_zero(x), 0.0, r);
+}
+__device__ __forceinline__ float m_sqrt_ratio(float a, float b) { return sqrtf(a * m_rcp(b)); }
+
+// x^n for a whole number n = 1..8
+template <class T>
+__device__ __forceinline__ T m_whole_pow(T x, int n)
+{
+    const T x2 = x * x, x4 = x2 * x2;
+    T r = n & 1 ? x : T(1);
+    if (n & 2) r *= x2;
+    if (n & 4) r *= x4;
+    if (n & 8) r *= x4 * x4;
+    return r;
+}
 
 __device__ __forceinline__ int map_idx(int i, int n, int periodic)
 {
@@ -366,129 +502,141 @@ __device__ __forceinline__ int halo_idx(const GridP &g, int d, int i, bool *flip
 
 template <class T>
 struct Ref {
-    T Gam, eref, pref, deref, dpref, G;
+    T re, pref, rdp, G;   // rho e_ref, p_ref, rho dp_ref/drho, shear modulus
 };
 
 // Mie-Grueneisen reference curves p = p_ref + rho Gamma (e - e_ref) of one
 // material (Sec. 2.1.2-2.1.3): ideal gas (p_ref = e_ref = 0), stiffened gas
 // (e_ref = 0, p_ref = -gamma p_inf), Romenskii solid (eq:Romenskii, cold term
 // K0/(2 rho alpha^2)(x^alpha - 1)^2 as printed, shear energy G J^2/rho with
-// G = G0 x^(beta+1), x = rho/rho0, and p_ref = rho^2 de_ref/drho).
+// G = G0 x^(beta+1), x = rho/rho0, and p_ref = rho^2 de_ref/drho).  Written
+// for rho e_ref and rho dp_ref/drho, which need no division.  The two powers
+// share one logarithm, and take products where the exponents are whole
+// numbers (copper: 1 and 4); at rho = rho0, where every absent solid is set,
+// both are 1.
 template <class T>
 __device__ __forceinline__ Ref<T> mat_ref(const MatC<T> &m, T rho, T J2)
 {
     Ref<T> r;
     if (m.kind == 2) {
-        const T al = m.alpha, be = m.beta, K0 = m.K0, rho0 = m.rho0;
-        const T x = rho / rho0;
-        const T xa = m_pow(x, al);
-        const T xm1 = xa - T(1);
-        const T ec = K0 / (T(2) * rho * al * al) * xm1 * xm1;
-        const T pc = -K0 / (T(2) * al * al) * xm1 * xm1 + (K0 / al) * xm1 * xa;
-        const T dpc = (K0 / rho0) * (xa / x) * (T(2) * xa - T(1) - xm1 / al);
-        const T G = m.G0 * m_pow(x, be + T(1));
-        const T ps = be * G * J2;
-        r.Gam = m.Gam;
-        r.eref = ec + G * J2 / rho;
-        r.pref = pc + ps;
-        r.deref = (pc + ps) / (rho * rho);
-        r.dpref = dpc + be * (be + T(1)) * G * J2 / rho;
-        r.G = G;
+        T xa = T(1), xg = T(1);
+        if (rho != m.rho0) {
+            const T x = rho * m.irho0;
+            const T lx = (m.n_alpha && m.n_beta1) ? T(0) : m_log(x);
+            xa = m.n_alpha ? m_whole_pow(x, m.n_alpha) : m_exp(m.alpha * lx);
+            xg = m.n_beta1 ? m_whole_pow(x, m.n_beta1) : m_exp(m.beta1 * lx);
+        }
+        const T xm1 = add_rn(xa, T(-1));
+        const T rc = mul_rn(mul_rn(m.kE, xm1), xm1);          // rho e_c
+        r.G = mul_rn(m.G0, xg);
+        const T GJ = mul_rn(r.G, J2);
+        r.re = add_rn(rc, GJ);
+        r.pref = m_fma(m.beta, GJ, m_fma(mul_rn(m.kP, xm1), xa, -rc));
+        r.rdp = m_fma(mul_rn(m.K0, xa), m_fma(-m.ialpha, xm1, m_fma(T(2), xa, T(-1))), mul_rn(m.bb, GJ));
     } else {
-        r.Gam = m.Gam;
-        r.eref = T(0);
+        r.re = T(0);
         r.pref = m.pref0;
-        r.deref = T(0);
-        r.dpref = T(0);
+        r.rdp = T(0);
         r.G = T(0);
     }
     return r;
 }
 
-// ------------------------------------------------- stretch tensor (FP64)
+// ------------------------------------------------------ stretch tensor
 
-// dev(H) = ln V with V^2 = A A^T (Sec. 2.1.2), traceless part, and
-// J^2 = |dev H|^2.  2-D: A A^T is block diagonal, so the in-plane 2x2 block is
-// diagonalised in closed form through the double angle 2 theta of its
-// eigenvectors; 1-D: diagonal.  Also returns the data needed to rebuild a
-// tensor with the same eigenvectors (plastic return).
-struct Eig2 {
-    double d[3];       // deviatoric log-stretches (in-plane 1, 2; out-of-plane)
-    double c2, s2;     // cos 2 theta, sin 2 theta of the in-plane eigenvectors
-};
-
-template <int DIM>
-__device__ __forceinline__ void stretch_log(const double A[3][3], double H[3][3], double &J2, Eig2 &e)
+// artanh(z)/z of z^2 (>= 0): its series to 2^-53 (FP64) or 2^-24 (FP32) below
+// z^2 = 0.01, the closed form above.  An elastic metal's stretches differ by
+// the yield strain, some 0.1 to 1 %, so its cells take the series; a gas may
+// shear without limit.
+__device__ __forceinline__ double artanh_ratio(double z2)
 {
-    double h0, h1, h2;
-    if (DIM == 1) {
-        h0 = 0.5 * log(A[0][0] * A[0][0]);
-        h1 = 0.5 * log(A[1][1] * A[1][1]);
-        h2 = 0.5 * log(A[2][2] * A[2][2]);
-        e.c2 = 1.0;
-        e.s2 = 0.0;
-    } else {
-        const double b00 = A[0][0] * A[0][0] + A[0][1] * A[0][1];
-        const double b01 = A[0][0] * A[1][0] + A[0][1] * A[1][1];
-        const double b11 = A[1][0] * A[1][0] + A[1][1] * A[1][1];
-        const double b22 = A[2][2] * A[2][2];
-        const double mid = 0.5 * (b00 + b11), half = 0.5 * (b00 - b11);
-        const double rad = sqrt(half * half + b01 * b01);
-        h0 = 0.5 * log(mid + rad);
-        h1 = 0.5 * log(mid - rad);
-        h2 = 0.5 * log(b22);
-        e.c2 = rad > 0.0 ? half / rad : 1.0;
-        e.s2 = rad > 0.0 ? b01 / rad : 0.0;
+    if (m_less(z2, 0.01)) {
+        double s = 1.0 / 17.0;
+        s = fma(s, z2, 1.0 / 15.0);
+        s = fma(s, z2, 1.0 / 13.0);
+        s = fma(s, z2, 1.0 / 11.0);
+        s = fma(s, z2, 1.0 / 9.0);
+        s = fma(s, z2, 1.0 / 7.0);
+        s = fma(s, z2, 1.0 / 5.0);
+        s = fma(s, z2, 1.0 / 3.0);
+        return fma(s, z2, 1.0);
     }
-    const double hm = (h0 + h1 + h2) * (1.0 / 3.0);
-    e.d[0] = h0 - hm;
-    e.d[1] = h1 - hm;
-    e.d[2] = h2 - hm;
-    J2 = e.d[0] * e.d[0] + e.d[1] * e.d[1] + e.d[2] * e.d[2];
-    const double av = 0.5 * (e.d[0] + e.d[1]), df = 0.5 * (e.d[0] - e.d[1]);
-    H[0][0] = av + df * e.c2;
-    H[1][1] = av - df * e.c2;
-    H[0][1] = H[1][0] = df * e.s2;
-    H[2][2] = e.d[2];
-    H[0][2] = H[2][0] = H[1][2] = H[2][1] = 0.0;
+    const double z = sqrt(z2);
+    return 0.5 * log((1.0 + z) / (1.0 - z)) / z;
+}
+__device__ __forceinline__ float artanh_ratio(float z2)
+{
+    if (z2 < 0.01f) {
+        float s = 1.f / 9.f;
+        s = fmaf(s, z2, 1.f / 7.f);
+        s = fmaf(s, z2, 1.f / 5.f);
+        s = fmaf(s, z2, 1.f / 3.f);
+        return fmaf(s, z2, 1.f);
+    }
+    const float z = sqrtf(z2);
+    return 0.5f * logf((1.f + z) / (1.f - z)) / z;
 }
 
-// The same in the compute precision T, for the closures (J^2 and dev H at
-// every face side and cell): the FP32 form keeps FP64 for the plastic
-// update's decomposition (plastic_return) only.  For T = double the
-// arithmetic is that of stretch_log.
+// The logarithm of the stretch, dev(H) = dev ln V with V^2 = A A^T (Sec.
+// 2.1.2), in 2-D, where A A^T = B is block diagonal, and 1-D, where it is
+// diagonal.  The in-plane block's log-stretches are mean +- k/2 about a mean
+// that, made traceless, is -d2/2, with
+//   d2 = (1/3) ln(A_zz^2/|det A_2|) = (2/3) artanh(s), s = (A_zz^2 - |det A_2|)/(A_zz^2 + |det A_2|),
+//   k = artanh(z), z = |(half, b01)|/mid of B's mean and deviator,
+// so that in place of three logarithms, a root and two divisions there are
+// two values of artanh(z)/z, an even function; k c_2 and k s_2 (2 theta the
+// doubled angle of the eigenvectors) are then q half and q b01 with
+// q = artanh(z)/(z mid).
+template <class T>
+struct StretchLog {
+    T d2, q, half, b01;   // see above (2-D); 1-D: dev log-stretches d0 = half, d1 = b01, d2
+    T k2, J2;             // k^2; |dev H|^2
+};
+
 template <class T, int DIM>
-__device__ __forceinline__ void stretch_log_ct(const T A[3][3], T H[3][3], T &J2)
+__device__ __forceinline__ void stretch_log(const T A[3][3], StretchLog<T> &e)
 {
-    T h0, h1, h2, c2, s2;
     if (DIM == 1) {
-        h0 = T(0.5) * m_log(A[0][0] * A[0][0]);
-        h1 = T(0.5) * m_log(A[1][1] * A[1][1]);
-        h2 = T(0.5) * m_log(A[2][2] * A[2][2]);
-        c2 = T(1);
-        s2 = T(0);
+        const T h0 = m_log(m_abs(A[0][0])), h1 = m_log(m_abs(A[1][1])), h2 = m_log(m_abs(A[2][2]));
+        const T hm = (h0 + h1 + h2) * (T(1) / T(3));
+        e.half = h0 - hm;
+        e.b01 = h1 - hm;
+        e.d2 = h2 - hm;
+        e.q = e.k2 = T(0);
+        e.J2 = e.half * e.half + e.b01 * e.b01 + e.d2 * e.d2;
     } else {
-        const T b00 = A[0][0] * A[0][0] + A[0][1] * A[0][1];
-        const T b01 = A[0][0] * A[1][0] + A[0][1] * A[1][1];
-        const T b11 = A[1][0] * A[1][0] + A[1][1] * A[1][1];
-        const T b22 = A[2][2] * A[2][2];
-        const T mid = T(0.5) * (b00 + b11), half = T(0.5) * (b00 - b11);
-        const T rad = m_sqrt(half * half + b01 * b01);
-        h0 = T(0.5) * m_log(mid + rad);
-        h1 = T(0.5) * m_log(mid - rad);
-        h2 = T(0.5) * m_log(b22);
-        c2 = rad > T(0) ? half / rad : T(1);
-        s2 = rad > T(0) ? b01 / rad : T(0);
+        const T b00 = m_fma(A[0][0], A[0][0], mul_rn(A[0][1], A[0][1]));
+        const T b11 = m_fma(A[1][1], A[1][1], mul_rn(A[1][0], A[1][0]));
+        e.b01 = m_fma(A[0][0], A[1][0], mul_rn(A[0][1], A[1][1]));
+        e.half = T(0.5) * (b00 - b11);
+        const T imid = m_rcp(T(0.5) * (b00 + b11));
+        const T det = m_abs(m_fma(A[0][0], A[1][1], -mul_rn(A[0][1], A[1][0]))), zz = mul_rn(A[2][2], A[2][2]);
+        const T s = mul_rn(zz - det, m_rcp(add_rn(zz, det)));
+        const T h = e.half * imid, b = e.b01 * imid, z2 = m_fma(h, h, mul_rn(b, b));
+        const T F = artanh_ratio(z2);
+        e.d2 = mul_rn(mul_rn(T(2) / T(3), s), artanh_ratio(s * s));
+        e.q = mul_rn(F, imid);
+        e.k2 = mul_rn(mul_rn(z2, F), F);
+        e.J2 = m_fma(mul_rn(T(1.5), e.d2), e.d2, mul_rn(T(0.5), e.k2));
     }
-    const T hm = (h0 + h1 + h2) * (T(1) / T(3));
-    const T d0 = h0 - hm, d1 = h1 - hm, d2 = h2 - hm;
-    J2 = d0 * d0 + d1 * d1 + d2 * d2;
-    const T av = T(0.5) * (d0 + d1), df = T(0.5) * (d0 - d1);
-    H[0][0] = av + df * c2;
-    H[1][1] = av - df * c2;
-    H[0][1] = H[1][0] = df * s2;
-    H[2][2] = d2;
-    H[0][2] = H[2][0] = H[1][2] = H[2][1] = T(0);
+}
+
+// dev(H), in-plane block (and the other entries a closure reads)
+template <class T, int DIM>
+__device__ __forceinline__ void stretch_dev(const StretchLog<T> &e, T H[DIM][DIM])
+{
+    if constexpr (DIM == 1) {
+        H[0][0] = e.half;
+    } else {
+        const T qh = T(0.5) * e.q, m = T(-0.5) * e.d2;
+#pragma unroll
+        for (int a = 0; a < DIM; a++)
+#pragma unroll
+            for (int b = 0; b < DIM; b++) H[a][b] = T(0);
+        H[0][0] = m_fma(qh, e.half, m);
+        H[1][1] = m_fma(-qh, e.half, m);
+        H[0][1] = H[1][0] = qh * e.b01;
+    }
 }
 
 // ------------------------------------------------------------- thermo
@@ -497,7 +645,7 @@ __device__ __forceinline__ void stretch_log_ct(const T A[3][3], T H[3][3], T &J2
 template <class T>
 __device__ __forceinline__ T phi_clip(T f)
 {
-    return f < T(0) ? T(0) : (f > T(1) ? T(1) : f);
+    return m_sel(m_neg(f), T(0), m_sel(m_over1(f), T(1), f));
 }
 
 // Phasic density (phi rho)_l / phi_l (Sec. 2.2); a material whose clipped
@@ -508,15 +656,72 @@ template <class T>
 __device__ __forceinline__ T phasic_density(const GridP &g, int l, T ar, T phc)
 {
     const MatC<T> &m = matc<T>(g, l);
-    if (phc < T(1e-6) && m.has_rho0) return m.rho0;
+    if (m_less(phc, T(1e-6)) && m.has_rho0) return m.rho0;
     const T guard = gridc<T>(g).phi_guard;
-    return ar / (phc > guard ? phc : guard);
+    const T f = m_less(guard, phc) ? phc : guard;
+    return sizeof(T) == 4 ? ar / f : ar * m_rcp(f);
+}
+
+// Mixture sums over the materials at phasic densities rhol (Sec. 2.2), all
+// with the weights phi_l/Gamma_l: den = sum of the weights, Q such that
+// rho e = p den - Q, Yn = rho c^2 den (one material: rho c^2), and the sums
+// of G and sigma_Y.
+template <class T, int NMAT>
+struct Mix {
+    T phi[NMAT], ar[NMAT];
+    T rho, den, Q, Yn, Gn, Sn;
+};
+
+template <class T, int NMAT, int SOLID>
+__device__ __forceinline__ void mix_sums(const GridP &g, const T *phi, const T *rhol, T p, T J2, Mix<T, NMAT> &x)
+{
+    T fsum = T(0);
+#pragma unroll
+    for (int l = 0; l < NMAT - 1; l++) {
+        x.phi[l] = phi[l];
+        fsum += phi[l];
+    }
+    x.phi[NMAT - 1] = T(1) - fsum;
+    x.rho = x.den = x.Q = x.Yn = x.Gn = x.Sn = T(0);
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) {
+        const MatC<T> &m = matc<T>(g, l);
+        const T f = NMAT == 1 ? T(1) : phi_clip(x.phi[l]);
+        x.phi[l] = f;
+        x.ar[l] = NMAT == 1 ? rhol[l] : mul_rn(f, rhol[l]);
+        x.rho = l == 0 ? x.ar[0] : add_rn(x.rho, x.ar[l]);
+        const T w = mul_rn(f, m.invGam);
+        x.den = l == 0 ? w : add_rn(x.den, w);
+        // a material without mass has no reference energy and no part in the sound speed
+        const bool mass = x.ar[l] != T(0);
+        if (m.kind == 2) {
+            const Ref<T> r = mat_ref<T>(m, rhol[l], J2);
+            x.Q = m_fma(w, r.pref, m_fma(-(mass ? f : T(0)), r.re, x.Q));
+            // (Gam + 1)(p - p_ref) + rho dp_ref/drho + 4/3 G   (rho^2 de_ref/drho = p_ref)
+            const T y = m_fma(m.kA, p - r.pref, mul_rn(m.invGam, m_fma(T(4) / T(3), r.G, r.rdp)));
+            if (NMAT == 1) x.Yn = mul_rn(y, m.Gam);
+            else if (mass) x.Yn = m_fma(f, y, x.Yn);
+            x.Gn = m_fma(w, r.G, x.Gn);
+            x.Sn = m_fma(w, m.sigY, x.Sn);
+        } else {
+            x.Q = m_fma(f, m.kB, x.Q);
+            if (NMAT == 1) {
+                x.Yn = m_fma(p, m.Gam1, -m.pref0);
+            } else {
+                const T y = m_fma(p, m.kA, -m.kB);   // (Gam p + p - p_ref)/Gam
+                if (mass) x.Yn = m_fma(f, y, x.Yn);
+            }
+        }
+    }
 }
 
 template <class T, int DIM, int NMAT, int SOLID>
 struct State {
     T phi[NMAT], ar[NMAT];
-    T rho, u[DIM], p, rhoE, c2, G, sigY;
+    T rho, u[DIM], p, c;   // c: sound speed
+    T den, Q;              // rho E = p den - Q + rho |u|^2/2
+    T c2, rhoE;            // FP32 fluid mixtures: c^2 and rho E in place of c, den, Q
+    T G, sigY;
     T H[DIM][DIM];     // dev(H), in-plane block
     T eps[NMAT];       // equivalent plastic strain (SOLID == 2)
 };
@@ -545,14 +750,11 @@ __device__ __forceinline__ void unpack_A(const T *w, double A[3][3])
     for (int c = 0; c < L::NV; c++) A[v_row(DIM, c)][v_col(DIM, c)] = (double)w[L::IV + c];
 }
 
-// Full state from primitives w (mixture rules of Sec. 2.2): rho = sum phi_l rho_l,
-// rho e = sum [ (phi rho)_l e_ref,l + phi_l (p - p_ref,l)/Gamma_l ],
-// G = sum(phi_l G_l/Gamma_l)/sum(phi_l/Gamma_l) (sigma_Y with the same weights),
-// c^2 = sum(Y_l c_l^2/Gamma_l)/sum(phi_l/Gamma_l) with c_l^2 = a_l^2 + 4/3 G_l/rho_l.
-template <class T, int DIM, int NMAT, int SOLID>
-__device__ __forceinline__ void state_from_prim_ct(const GridP &g, const T *w, State<T, DIM, NMAT, SOLID> &s)
+// The closure of the FP32 fluid mixtures: the same rules, material by material.
+template <class T, int DIM, int NMAT>
+__device__ __forceinline__ void mix32_state(const GridP &g, const T *w, State<T, DIM, NMAT, 0> &s)
 {
-    using L = Lay<DIM, NMAT, SOLID>;
+    using L = Lay<DIM, NMAT, 0>;
     T fsum = T(0);
 #pragma unroll
     for (int l = 0; l < NMAT - 1; l++) {
@@ -572,50 +774,25 @@ __device__ __forceinline__ void state_from_prim_ct(const GridP &g, const T *w, S
 #pragma unroll
     for (int a = 0; a < DIM; a++) s.u[a] = w[L::IMOM + a];
     s.p = w[L::IE];
-#pragma unroll
-    for (int l = 0; l < NMAT; l++) s.eps[l] = T(0);
-    if constexpr (SOLID == 2) {
-#pragma unroll
-        for (int l = 0; l < NMAT; l++) s.eps[l] = w[L::IH + l];
-    }
-    T J2 = T(0);
-    if (SOLID) {
-        T A[3][3], H[3][3];
-        unpack_A_ct<T, DIM, NMAT, SOLID>(w, A);
-        stretch_log_ct<T, DIM>(A, H, J2);
-#pragma unroll
-        for (int a = 0; a < DIM; a++)
-#pragma unroll
-            for (int b = 0; b < DIM; b++) s.H[a][b] = H[a][b];
-    }
-    if constexpr (NMAT == 1) {
-        // single material: the mixture rules reduce to the material's own closure
-        const MatC<T> &m = matc<T>(g, 0);
-        const Ref<T> r = mat_ref<T>(m, rhol[0], J2);
-        const T irl = T(1) / rhol[0];
-        T ke = T(0);
-#pragma unroll
-        for (int a = 0; a < DIM; a++) ke += T(0.5) * s.rho * s.u[a] * s.u[a];
-        s.rhoE = s.ar[0] * r.eref + (s.p - r.pref) * m.invGam + ke;
-        s.G = r.G;
-        s.sigY = m.sigY;
-        s.c2 = (r.Gam * s.p + (s.p - r.pref)) * irl + r.dpref - r.Gam * rhol[0] * r.deref + T(4) / T(3) * r.G * irl;
-        return;
-    }
-    T rhoe = T(0), den = T(0), Gn = T(0), Sn = T(0), Yn = T(0);
+    T rhoe = T(0), den = T(0), Yn = T(0);
 #pragma unroll
     for (int l = 0; l < NMAT; l++) {
         const MatC<T> &m = matc<T>(g, l);
-        const Ref<T> r = mat_ref<T>(m, rhol[l], J2);
         const T iG = m.invGam;
         const T irl = T(1) / rhol[l];
-        if (s.ar[l] != T(0)) rhoe += s.ar[l] * r.eref;
-        rhoe += s.phi[l] * (s.p - r.pref) * iG;
+        if (m.kind == 2) {
+            // a solid's equation of state in a fluid run (no stretch: J^2 = 0)
+            const Ref<T> r = mat_ref<T>(m, rhol[l], T(0));
+            if (s.ar[l] != T(0)) rhoe += s.ar[l] * (r.re * irl);
+            rhoe += s.phi[l] * (s.p - r.pref) * iG;
+            den += s.phi[l] * iG;
+            const T c2l = ((m.Gam + T(1)) * (s.p - r.pref) + r.rdp + T(4) / T(3) * r.G) * irl;
+            if (s.ar[l] != T(0)) Yn += s.ar[l] * c2l * iG;
+            continue;
+        }
+        rhoe += s.phi[l] * (s.p - m.pref0) * iG;
         den += s.phi[l] * iG;
-        Gn += s.phi[l] * r.G * iG;
-        Sn += s.phi[l] * m.sigY * iG;
-        const T a2 = (r.Gam * s.p + (s.p - r.pref)) * irl + r.dpref - r.Gam * rhol[l] * r.deref;
-        const T c2l = a2 + T(4) / T(3) * r.G * irl;
+        const T c2l = (m.Gam * s.p + (s.p - m.pref0)) * irl;
         if (s.ar[l] != T(0)) Yn += s.ar[l] * c2l * iG;
     }
     T ke = T(0);
@@ -623,9 +800,69 @@ __device__ __forceinline__ void state_from_prim_ct(const GridP &g, const T *w, S
     for (int a = 0; a < DIM; a++) ke += T(0.5) * s.rho * s.u[a] * s.u[a];
     const T iden = T(1) / den;
     s.rhoE = rhoe + ke;
-    s.G = Gn * iden;
-    s.sigY = Sn * iden;
     s.c2 = Yn / s.rho * iden;
+    s.c = m_sqrt(s.c2);
+    s.G = s.sigY = T(0);
+}
+
+// Full state from primitives w (mixture rules of Sec. 2.2): rho = sum phi_l rho_l,
+// rho e = sum [ (phi rho)_l e_ref,l + phi_l (p - p_ref,l)/Gamma_l ],
+// G = sum(phi_l G_l/Gamma_l)/sum(phi_l/Gamma_l) (sigma_Y with the same weights),
+// c^2 = sum(Y_l c_l^2/Gamma_l)/sum(phi_l/Gamma_l) with c_l^2 = a_l^2 + 4/3 G_l/rho_l.
+template <class T, int DIM, int NMAT, int SOLID>
+__device__ __forceinline__ void state_from_prim_ct(const GridP &g, const T *w, State<T, DIM, NMAT, SOLID> &s)
+{
+    using L = Lay<DIM, NMAT, SOLID>;
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) s.eps[l] = T(0);
+    if constexpr (mix32<T, NMAT, SOLID>()) {
+        mix32_state<T, DIM, NMAT>(g, w, s);
+        return;
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) s.u[a] = w[L::IMOM + a];
+    s.p = w[L::IE];
+    if constexpr (SOLID == 2) {
+#pragma unroll
+        for (int l = 0; l < NMAT; l++) s.eps[l] = w[L::IH + l];
+    }
+    T J2 = T(0);
+    if (SOLID) {
+        T A[3][3];
+        StretchLog<T> e;
+        unpack_A_ct<T, DIM, NMAT, SOLID>(w, A);
+        stretch_log<T, DIM>(A, e);
+        stretch_dev<T, DIM>(e, s.H);
+        J2 = e.J2;
+    }
+    Mix<T, NMAT> x;
+    mix_sums<T, NMAT, SOLID>(g, w + L::IPHI, w + L::IAR, s.p, J2, x);
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) {
+        s.phi[l] = x.phi[l];
+        s.ar[l] = x.ar[l];
+    }
+    s.rho = x.rho;
+    s.den = x.den;
+    s.Q = x.Q;
+    s.c = m_sqrt_ratio(x.Yn, NMAT == 1 ? x.rho : mul_rn(x.rho, x.den));
+    s.G = s.sigY = T(0);
+    if (SOLID) {
+        const T iden = m_rcp(x.den);
+        s.G = mul_rn(x.Gn, iden);
+        s.sigY = mul_rn(x.Sn, iden);
+    }
+}
+
+// rho E of a state
+template <class T, int DIM, int NMAT, int SOLID>
+__device__ __forceinline__ T state_energy(const State<T, DIM, NMAT, SOLID> &s)
+{
+    if (mix32<T, NMAT, SOLID>()) return s.rhoE;
+    T uu = T(0);
+#pragma unroll
+    for (int a = 0; a < DIM; a++) uu = m_fma(s.u[a], s.u[a], uu);
+    return m_fma(T(0.5) * s.rho, uu, m_fma(s.p, s.den, -s.Q));
 }
 
 // The FP32 form's precision rule: the closure of a mixed cell -- at least two
@@ -672,8 +909,11 @@ __device__ __forceinline__ void state_from_prim(const GridP &g, const T *w, Stat
 #pragma unroll
         for (int a = 0; a < DIM; a++) s.u[a] = (T)sd.u[a];
         s.p = (T)sd.p;
-        s.rhoE = (T)sd.rhoE;
-        s.c2 = (T)sd.c2;
+        s.c = (T)sd.c;
+        s.den = (T)sd.den;
+        s.Q = (T)sd.Q;
+        s.c2 = (T)(sd.c * sd.c);
+        s.rhoE = (T)state_energy<double, DIM, NMAT, SOLID>(sd);
         s.G = (T)sd.G;
         s.sigY = (T)sd.sigY;
 #pragma unroll
@@ -708,44 +948,84 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
         ar[l] = q[L::IAR + l];
         rho += ar[l];
     }
-    T u[DIM];
-    const T irho = T(1) / rho;
+    if constexpr (mix32<T, NMAT, SOLID>()) {
+        T u[DIM];
+        const T irho = T(1) / rho;
 #pragma unroll
-    for (int a = 0; a < DIM; a++) u[a] = q[L::IMOM + a] * irho;
-    T J2 = T(0);
-    if (SOLID) {
-        T A[3][3], H[3][3];
-        unpack_A_ct<T, DIM, NMAT, SOLID>(q, A);
-        stretch_log_ct<T, DIM>(A, H, J2);
-    }
-    T ke = T(0);
+        for (int a = 0; a < DIM; a++) u[a] = q[L::IMOM + a] * irho;
+        T ke = T(0);
 #pragma unroll
-    for (int a = 0; a < DIM; a++) ke += T(0.5) * rho * u[a] * u[a];
-    T num = q[L::IE] - ke, den = T(0);
-    T rhol[NMAT];
-    if constexpr (NMAT == 1) {
-        const MatC<T> &m = matc<T>(g, 0);
-        const Ref<T> r = mat_ref<T>(m, rho, J2);
+        for (int a = 0; a < DIM; a++) ke += T(0.5) * rho * u[a] * u[a];
+        T num = q[L::IE] - ke, den = T(0);
+        T rhol[NMAT];
+#pragma unroll
+        for (int l = 0; l < NMAT; l++) {
+            const T phc = phi_clip(phi[l]);
+            rhol[l] = phasic_density<T>(g, l, ar[l], phc);
+            const MatC<T> &m = matc<T>(g, l);
+            T pref = m.pref0;
+            if (m.kind == 2) {
+                const Ref<T> r = mat_ref<T>(m, rhol[l], T(0));
+                pref = r.pref;
+                if (ar[l] != T(0)) num -= ar[l] * (r.re / rhol[l]);
+            }
+            num += phc * pref * m.invGam;
+            den += phc * m.invGam;
+        }
+#pragma unroll
+        for (int l = 0; l < NMAT - 1; l++) w[L::IPHI + l] = phi[l];
+#pragma unroll
+        for (int l = 0; l < NMAT; l++) w[L::IAR + l] = rhol[l];
 #pragma unroll
         for (int a = 0; a < DIM; a++) w[L::IMOM + a] = u[a];
-        w[L::IAR] = rho;
-        // p = p_ref + Gamma (rho e - rho e_ref)   (eq:MieGruneisenEOS)
-        w[L::IE] = r.pref + r.Gam * (num - rho * r.eref);
-#pragma unroll
-        for (int c = 0; c < L::NV; c++) w[L::IV + c] = q[L::IV + c];
+        w[L::IE] = num / den;
         w[L::IR] = q[L::IR];
-        if constexpr (SOLID == 2) w[L::IH] = rho != T(0) ? q[L::IH] / rho : T(0);
         return;
     }
+    T u[DIM], mu = T(0);
+    const T irho = m_rcp(rho);
 #pragma unroll
-    for (int l = 0; l < NMAT; l++) {
-        const T phc = phi_clip(phi[l]);
-        rhol[l] = (NMAT == 1) ? rho : phasic_density<T>(g, l, ar[l], phc);
-        const MatC<T> &m = matc<T>(g, l);
-        const Ref<T> r = mat_ref<T>(m, rhol[l], J2);
-        if (ar[l] != T(0)) num -= ar[l] * r.eref;
-        num += phc * r.pref * m.invGam;
-        den += phc * m.invGam;
+    for (int a = 0; a < DIM; a++) {
+        u[a] = q[L::IMOM + a] * irho;
+        mu = m_fma(q[L::IMOM + a], u[a], mu);
+    }
+    T J2 = T(0);
+    if (SOLID) {
+        T A[3][3];
+        StretchLog<T> e;
+        unpack_A_ct<T, DIM, NMAT, SOLID>(q, A);
+        stretch_log<T, DIM>(A, e);
+        J2 = e.J2;
+    }
+    T num = m_fma(T(-0.5), mu, q[L::IE]), den = T(0);
+    T rhol[NMAT];
+    if constexpr (NMAT == 1) {
+        // p = p_ref + Gamma (rho e - rho e_ref)   (eq:MieGruneisenEOS)
+        const MatC<T> &m = matc<T>(g, 0);
+        rhol[0] = rho;
+        if (m.kind == 2) {
+            const Ref<T> r = mat_ref<T>(m, rho, J2);
+            w[L::IE] = m_fma(m.Gam, num - r.re, r.pref);
+        } else {
+            w[L::IE] = m_fma(m.Gam, num, m.pref0);
+        }
+    } else {
+#pragma unroll
+        for (int l = 0; l < NMAT; l++) {
+            const T f = phi_clip(phi[l]);
+            rhol[l] = phasic_density<T>(g, l, ar[l], f);
+            const MatC<T> &m = matc<T>(g, l);
+            if (m.kind == 2) {
+                // (phi rho) e_ref is phi (rho e_ref), and for an absent material at rho0 its mass over rho0
+                const Ref<T> r = mat_ref<T>(m, rhol[l], J2);
+                num -= (m_less(f, T(1e-6)) ? ar[l] * m.irho0 : f) * r.re;
+                num += f * m.invGam * r.pref;
+            } else {
+                num = m_fma(f, m.kB, num);
+            }
+            den = m_fma(f, m.invGam, den);
+        }
+        w[L::IE] = num * m_rcp(den);
     }
 #pragma unroll
     for (int l = 0; l < NMAT - 1; l++) w[L::IPHI + l] = phi[l];
@@ -753,15 +1033,37 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
     for (int l = 0; l < NMAT; l++) w[L::IAR + l] = rhol[l];
 #pragma unroll
     for (int a = 0; a < DIM; a++) w[L::IMOM + a] = u[a];
-    w[L::IE] = num / den;
 #pragma unroll
     for (int c = 0; c < L::NV; c++) w[L::IV + c] = q[L::IV + c];
     w[L::IR] = q[L::IR];
     // history: specific eps_l = (phi rho eps)_l / (phi rho)_l, 0 without mass
     if constexpr (SOLID == 2) {
 #pragma unroll
-        for (int l = 0; l < NMAT; l++) w[L::IH + l] = ar[l] != T(0) ? q[L::IH + l] / ar[l] : T(0);
+        for (int l = 0; l < NMAT; l++) w[L::IH + l] = ar[l] != T(0) ? q[L::IH + l] * m_rcp(ar[l]) : T(0);
     }
+}
+
+// Wave speed sum_d (|u_d| + c)/dx_d of one gas cell from its conserved values
+// (FP32; momenta q[1..DIM]); every operation rounded as written, so that
+// the stage kernels and the standalone reduction agree to the bit.  c2: c^2.
+template <int DIM>
+__device__ __forceinline__ float gas_speed(float Gam, float pref0, const float *q, const float *inv_dx, float &c2)
+{
+    const float ir = m_rcp(q[0]), hr = __fmul_rn(0.5f, q[0]);
+    float u[DIM], ke = 0.f;
+#pragma unroll
+    for (int d = 0; d < DIM; d++) {
+        u[d] = __fmul_rn(q[1 + d], ir);
+        const float h = __fmul_rn(hr, u[d]);
+        ke = d == 0 ? __fmul_rn(h, u[d]) : fmaf(h, u[d], ke);
+    }
+    const float p = fmaf(Gam, __fadd_rn(q[1 + DIM], -ke), pref0);
+    c2 = __fmul_rn(fmaf(Gam, p, __fadd_rn(p, -pref0)), ir);
+    const float c = sqrtf(c2);
+    float s = __fmul_rn(__fadd_rn(fabsf(u[DIM - 1]), c), inv_dx[DIM - 1]);
+#pragma unroll
+    for (int d = DIM - 2; d >= 0; d--) s = fmaf(__fadd_rn(fabsf(u[d]), c), inv_dx[d], s);
+    return s;
 }
 
 template <class T, int DIM, int NMAT, int SOLID>
@@ -780,6 +1082,33 @@ __device__ __forceinline__ void cons_to_prim(const GridP &g, const T *q, T *w)
     cons_to_prim_ct<T, DIM, NMAT, SOLID>(g, q, w);
 }
 
+// Wave speed sum_d (|u_d| + c)/dx_d of a cell from its conserved values; c: its
+// sound speed or its square (not positive where c^2 <= 0).
+template <class T, int DIM, int NMAT, int SOLID>
+__device__ __forceinline__ T cell_speed(const GridP &g, const T *q, T &c)
+{
+    using L = Lay<DIM, NMAT, SOLID>;
+    if constexpr (sizeof(T) == 4 && NMAT == 1 && SOLID == 0) {
+        if (g.mc_f[0].kind != 2) {
+            float c2;
+            const T s = gas_speed<DIM>(g.mc_f[0].Gam, g.mc_f[0].pref0, q + L::IAR, g.gc_f.inv_dx, c2);
+            c = c2;
+            return s;
+        }
+    }
+    T w[L::NVAR];
+    cons_to_prim<T, DIM, NMAT, SOLID>(g, q, w);
+    State<T, DIM, NMAT, SOLID> s;
+    state_from_prim<T, DIM, NMAT, SOLID>(g, w, s);
+    T sum = T(0);
+#pragma unroll
+    for (int d = 0; d < DIM; d++)
+        sum += mix32<T, NMAT, SOLID>() ? (m_abs(s.u[d]) + s.c) / gridc<T>(g).dx[d]
+                                       : (m_abs(s.u[d]) + s.c) * gridc<T>(g).inv_dx[d];
+    c = s.c;
+    return sum;
+}
+
 template <class T, int DIM, int NMAT, int SOLID>
 __device__ __forceinline__ void prim_to_cons(const GridP &g, const T *w, T *q)
 {
@@ -792,7 +1121,7 @@ __device__ __forceinline__ void prim_to_cons(const GridP &g, const T *w, T *q)
     for (int l = 0; l < NMAT; l++) q[L::IAR + l] = s.ar[l];
 #pragma unroll
     for (int a = 0; a < DIM; a++) q[L::IMOM + a] = s.rho * s.u[a];
-    q[L::IE] = s.rhoE;
+    q[L::IE] = state_energy<T, DIM, NMAT, SOLID>(s);
 #pragma unroll
     for (int c = 0; c < L::NV; c++) q[L::IV + c] = w[L::IV + c];
     q[L::IR] = w[L::IR];
@@ -804,19 +1133,19 @@ __device__ __forceinline__ void prim_to_cons(const GridP &g, const T *w, T *q)
 
 // ------------------------------------------------------- reconstruction
 
+// The slope, THINC and face reconstruction of the FP32 fluid mixtures, and of
+// the volume fractions and r of every FP32 form (recon_face below says what
+// they do), in one fixed order of operations: where MUSCL's and THINC's
+// boundary variations agree to round-off, the choice between them, and with it
+// the face value, would otherwise change with the order of rounding.
 template <class T>
 __device__ __forceinline__ T vanleer(T a, T b)
 {
     return (a * b <= T(0)) ? T(0) : T(2) * a * b / (a + b);
 }
 
-// THINC face values of a cell (Sec. 3.1, MUSCL-BVD-THINC): the tanh profile
-// q_min + dq/2 (1 + theta tanh(beta (x - x_c))) on [0,1] whose cell average is
-// q0 has tanh(beta x_c) = (cosh beta - exp(theta beta (2C-1)))/sinh beta with
-// C = (q0 - q_min)/dq; its end values are returned.  Only monotone cells with
-// 1e-8 < C < 1 - 1e-8.
 template <class T>
-__device__ __forceinline__ bool thinc(const GridP &g, T qm, T q0, T qp, T &fm, T &fp)
+__device__ __forceinline__ bool mix32_thinc(const GridP &g, T qm, T q0, T qp, T &fm, T &fp)
 {
     if ((qp - q0) * (q0 - qm) <= T(0)) return false;
     const T qmin = m_min(qm, qp), qmax = m_max(qm, qp);
@@ -834,12 +1163,8 @@ __device__ __forceinline__ bool thinc(const GridP &g, T qm, T q0, T qp, T &fm, T
     return true;
 }
 
-// Left and right states at the face between cells f-1 and f of a pencil,
-// s[0..5] = q_{f-3} .. q_{f+2}.  MUSCL (van Leer) for every primitive; for a
-// volume fraction (frac = true) the BVD rule keeps a cell's THINC face values
-// only where its total boundary variation is strictly below MUSCL's.
 template <class T>
-__device__ __forceinline__ void recon_face(const GridP &g, const T *s, bool frac, T &qL, T &qR)
+__device__ __forceinline__ void mix32_recon_face(const GridP &g, const T *s, bool frac, T &qL, T &qR)
 {
     const T slB = vanleer(s[2] - s[1], s[3] - s[2]);
     const T slC = vanleer(s[3] - s[2], s[4] - s[3]);
@@ -852,10 +1177,10 @@ __device__ __forceinline__ void recon_face(const GridP &g, const T *s, bool frac
     const T Ap = s[1] + T(0.5) * slA, Bm = s[2] - T(0.5) * slB;
     const T Cp = s[3] + T(0.5) * slC, Em = s[4] - T(0.5) * slE;
     T tAm = s[1] - T(0.5) * slA, tAp = Ap, tBm = Bm, tBp = Bp, tCm = Cm, tCp = Cp, tEm = Em, tEp = s[4] + T(0.5) * slE;
-    thinc<T>(g, s[0], s[1], s[2], tAm, tAp);
-    thinc<T>(g, s[1], s[2], s[3], tBm, tBp);
-    thinc<T>(g, s[2], s[3], s[4], tCm, tCp);
-    thinc<T>(g, s[3], s[4], s[5], tEm, tEp);
+    mix32_thinc<T>(g, s[0], s[1], s[2], tAm, tAp);
+    mix32_thinc<T>(g, s[1], s[2], s[3], tBm, tBp);
+    mix32_thinc<T>(g, s[2], s[3], s[4], tCm, tCp);
+    mix32_thinc<T>(g, s[3], s[4], s[5], tEm, tEp);
     const T tbvBM = m_abs(Ap - Bm) + m_abs(Bp - Cm);
     const T tbvBT = m_abs(tAp - tBm) + m_abs(tBp - tCm);
     const T tbvCM = m_abs(Bp - Cm) + m_abs(Cp - Em);
@@ -864,14 +1189,88 @@ __device__ __forceinline__ void recon_face(const GridP &g, const T *s, bool frac
     if (tbvCT < tbvCM) qR = tCm;
 }
 
+// half the van Leer slope 2ab/(a+b) of a cell from its backward and forward
+// differences.  (Here and in the closures the products and sums are rounded as
+// written, fused only where fma says so: the two sides of a wall face, mirror
+// images, then go through the same roundings and S* there is exactly 0.)
+template <class T>
+__device__ __forceinline__ T half_slope(T a, T b)
+{
+    const T ab = a * b;
+    return m_pos(ab) ? mul_rn(ab, m_rcp(a + b)) : T(0);
+}
+
+// THINC face values of a cell (Sec. 3.1, MUSCL-BVD-THINC): the tanh profile
+// q_min + dq/2 (1 + theta tanh(beta (x - x_c))) on [0,1] whose cell average is
+// q0 has tanh(beta x_c) = (cosh beta - exp(theta beta (2C-1)))/sinh beta with
+// C = (q0 - q_min)/dq; its end values are returned.  Only monotone cells with
+// 1e-8 < C < 1 - 1e-8.
+template <class T>
+__device__ __forceinline__ bool thinc(const GridP &g, T qm, T q0, T qp, T &fm, T &fp)
+{
+    if (!m_pos((qp - q0) * (q0 - qm))) return false;
+    const bool up = !m_less(qp, qm);
+    const T qmin = m_sel(up, qm, qp);
+    const T d = qp - qm, dq = m_abs(d);
+    const T C = (q0 - qmin) * m_rcp(dq);
+    if (!(m_less(T(1e-8), C) && m_less(C, T(1) - T(1e-8)))) return false;
+    const GridC<T> &gc = gridc<T>(g);
+    const T th = m_sel(up, T(1), T(-1));
+    const T B = m_exp(th * gc.beta * (T(2) * C - T(1)));
+    const T ty = (gc.cosh_b - B) * gc.inv_sinh_b;
+    const T tb = gc.tanh_b;
+    const T t1 = (tb - ty) * m_rcp(T(1) - tb * ty);
+    const T hd = T(0.5) * d;                     // theta dq/2
+    const T mid = m_fma(T(0.5), dq, qmin);
+    fm = m_fma(-hd, ty, mid);
+    fp = m_fma(hd, t1, mid);
+    return true;
+}
+
+// Left and right states at the face between cells f-1 and f of a pencil,
+// s[0..5] = q_{f-3} .. q_{f+2}.  MUSCL (van Leer) for every primitive; for a
+// volume fraction (frac = true) the BVD rule keeps a cell's THINC face values
+// only where its total boundary variation is strictly below MUSCL's.
+template <class T>
+__device__ __forceinline__ void recon_face(const GridP &g, const T *s, bool frac, T &qL, T &qR)
+{
+    if (sizeof(T) == 4 && frac) {
+        mix32_recon_face<T>(g, s, frac, qL, qR);
+        return;
+    }
+    const T hB = half_slope(s[2] - s[1], s[3] - s[2]);
+    const T hC = half_slope(s[3] - s[2], s[4] - s[3]);
+    const T Bp = s[2] + hB, Cm = s[3] - hC;
+    qL = Bp;
+    qR = Cm;
+    if (!frac || !g.use_thinc) return;
+    const T hA = half_slope(s[1] - s[0], s[2] - s[1]);
+    const T hE = half_slope(s[4] - s[3], s[5] - s[4]);
+    const T Ap = s[1] + hA, Bm = s[2] - hB;
+    const T Cp = s[3] + hC, Em = s[4] - hE;
+    T tAm = s[1] - hA, tAp = Ap, tBm = Bm, tBp = Bp, tCm = Cm, tCp = Cp, tEm = Em, tEp = s[4] + hE;
+    thinc<T>(g, s[0], s[1], s[2], tAm, tAp);
+    thinc<T>(g, s[1], s[2], s[3], tBm, tBp);
+    thinc<T>(g, s[2], s[3], s[4], tCm, tCp);
+    thinc<T>(g, s[3], s[4], s[5], tEm, tEp);
+    const T tbvBM = m_abs(Ap - Bm) + m_abs(Bp - Cm);
+    const T tbvBT = m_abs(tAp - tBm) + m_abs(tBp - tCm);
+    const T tbvCM = m_abs(Bp - Cm) + m_abs(Cp - Em);
+    const T tbvCT = m_abs(tBp - tCm) + m_abs(tCp - tEm);
+    if (m_less(tbvBT, tbvBM)) qL = tBp;
+    if (m_less(tbvCT, tbvCM)) qR = tCm;
+}
+
 // ------------------------------------------------------------- Riemann
 
-// Left value for w = 1, right value for w = 0, the mean for w = 1/2 (exactly
-// xl or xr in the first two cases).
+// Left value where the contact moves right (sgn > 0), right value where it
+// moves left, the mean of both where it stands.
 template <class T>
-__device__ __forceinline__ T upwind_mix(T w, T xl, T xr)
+__device__ __forceinline__ T upwind_mix(int sgn, T xl, T xr)
 {
-    return w == T(1) ? xl : (w == T(0) ? xr : T(0.5) * (xl + xr));
+    T v = m_sel(sgn > 0, xl, xr);
+    if (sgn == 0) v = T(0.5) * (xl + xr);
+    return v;
 }
 
 // out += a (U*_K - U_K) on the partial densities, momenta and energy, for the
@@ -880,8 +1279,9 @@ template <class T, int DIM, int NMAT, int SOLID, int D>
 __device__ __forceinline__ void star_jump(const State<T, DIM, NMAT, SOLID> &K, T SK, T TK, T Ss, T a, T *out)
 {
     using L = Lay<DIM, NMAT, SOLID>;
-    const T uK = K.u[D];
-    const T chi = (SK - uK) / (SK - Ss);
+    const T uK = K.u[D], EK = state_energy<T, DIM, NMAT, SOLID>(K);
+    const T iD = m_rcp(SK - Ss);
+    const T chi = (SK - uK) * iD;
 #pragma unroll
     for (int l = 0; l < NMAT; l++) out[L::IAR + l] += a * (K.ar[l] * chi - K.ar[l]);
     if constexpr (SOLID == 2) {
@@ -890,31 +1290,45 @@ __device__ __forceinline__ void star_jump(const State<T, DIM, NMAT, SOLID> &K, T
     }
 #pragma unroll
     for (int b = 0; b < DIM; b++) out[L::IMOM + b] += a * (K.rho * chi * (b == D ? Ss : K.u[b]) - K.rho * K.u[b]);
+    out[L::IE] += a * (chi * EK + (Ss - uK) * (K.rho * chi * Ss + TK * iD) - EK);
+}
+
+template <class T>
+__device__ __forceinline__ T mix32_upwind(T w, T xl, T xr)
+{
+    return w == T(1) ? xl : (w == T(0) ? xr : T(0.5) * (xl + xr));
+}
+
+// out += a (U*_K - U_K) on the partial densities, momenta and energy, for the
+// HLLC star state of side K (wave speed SK, normal traction TK, contact Ss).
+template <class T, int DIM, int NMAT, int D>
+__device__ __forceinline__ void mix32_star_jump(const State<T, DIM, NMAT, 0> &K, T SK, T TK, T Ss, T a, T *out)
+{
+    using L = Lay<DIM, NMAT, 0>;
+    const T uK = K.u[D];
+    const T chi = (SK - uK) / (SK - Ss);
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) out[L::IAR + l] += a * (K.ar[l] * chi - K.ar[l]);
+#pragma unroll
+    for (int b = 0; b < DIM; b++) out[L::IMOM + b] += a * (K.rho * chi * (b == D ? Ss : K.u[b]) - K.rho * K.u[b]);
     const T EK = K.rhoE / K.rho;
     out[L::IE] += a * (K.rho * chi * (EK + (Ss - uK) * (Ss + TK / (K.rho * (SK - uK)))) - K.rhoE);
 }
 
-// HLLC flux across a face normal to direction D (Sec. 3.1: Toro's HLLC; the
-// fluid pressure replaced by the normal traction T = p - 2G devH_DD for solids;
-// Davis wave speeds; partial densities scaled like the mixture density).
-// out[0..NVAR-1]: flux of every plane (r: upwind with the body velocity vr),
-// out[NVAR]: face velocity u*_D, out[NVAR+1+b]: V*_{D b} (upwind by S*).
-template <class T, int DIM, int NMAT, int SOLID, int D>
-__device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR, T vr, T *out)
+// HLLC flux of the FP32 fluid mixtures in their fixed order of operations: the
+// flux of the upwind side plus the jump to its star state.
+template <class T, int DIM, int NMAT, int D>
+__device__ __forceinline__ void mix32_riemann(const GridP &g, const T *wL, const T *wR, T vr, T *out)
 {
-    using L = Lay<DIM, NMAT, SOLID>;
-    State<T, DIM, NMAT, SOLID> sl, sr;
-    state_from_prim<T, DIM, NMAT, SOLID>(g, wL, sl);
-    state_from_prim<T, DIM, NMAT, SOLID>(g, wR, sr);
+    using L = Lay<DIM, NMAT, 0>;
+    State<T, DIM, NMAT, 0> sl, sr;
+    state_from_prim<T, DIM, NMAT, 0>(g, wL, sl);
+    state_from_prim<T, DIM, NMAT, 0>(g, wR, sr);
     const T cL = m_sqrt(sl.c2), cR = m_sqrt(sr.c2);
     const T uL = sl.u[D], uR = sr.u[D];
-    const T TL = SOLID ? sl.p - T(2) * sl.G * sl.H[D][D] : sl.p;
-    const T TR = SOLID ? sr.p - T(2) * sr.G * sr.H[D][D] : sr.p;
+    const T TL = sl.p, TR = sr.p;
     const T SL = m_min(uL - cL, uR - cR);
     const T SR = m_max(uL + cL, uR + cR);
-    // contact speed; the numerator's products are rounded one by one and
-    // summed left to right, so that mirror-image states (a wall face) give
-    // S* = 0 exactly
     const T num = add_rn(add_rn(TR - TL, mul_rn(mul_rn(sl.rho, uL), SL - uL)),
                          -mul_rn(mul_rn(sr.rho, uR), SR - uR));
     const T Ss = num / (sl.rho * (SL - uL) - sr.rho * (SR - uR));
@@ -923,48 +1337,23 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
     else if (Ss >= T(0)) region = 1;
     else if (SR > T(0)) region = 2;
     else region = 3;
-    const State<T, DIM, NMAT, SOLID> &K = (region <= 1) ? sl : sr;
+    const State<T, DIM, NMAT, 0> &K = (region <= 1) ? sl : sr;
     const T SK = (region <= 1) ? SL : SR;
     const T TK = (region <= 1) ? TL : TR;
     const T uK = K.u[D];
     const bool star = (region == 1 || region == 2);
-    // quantities carried by the contact take the left value for S* > 0, the
-    // right one for S* < 0 and the mean of both at S* = 0 (mirror-symmetric
-    // at a wall face)
     const T wlf = Ss > T(0) ? T(1) : (Ss < T(0) ? T(0) : T(0.5));
-    // Tangential traction and velocity at the face: the linear shear-wave
-    // Riemann problem (sigma -/+ Z u constant along the shear characteristics,
-    // Z = sqrt(rho G)); a gas (Z = 0) transmits no shear.  Without shear
-    // stiffness on either side the tangential velocity is upwind by S*.
-    T sig_t[DIM], ut[DIM];
+    T ut[DIM];
 #pragma unroll
-    for (int a = 0; a < DIM; a++) {
-        sig_t[a] = T(0);
-        ut[a] = upwind_mix(wlf, sl.u[a], sr.u[a]);
-    }
-    if (SOLID) {
-        const T ZL = m_sqrt(sl.rho * sl.G), ZR = m_sqrt(sr.rho * sr.G);
-#pragma unroll
-        for (int a = 0; a < DIM; a++) {
-            if (a == D) continue;
-            const T sL = T(2) * sl.G * sl.H[a][D], sR = T(2) * sr.G * sr.H[a][D];
-            if (ZL + ZR > T(0)) {
-                sig_t[a] = (ZR * sL + ZL * sR + ZL * ZR * (sr.u[a] - sl.u[a])) / (ZL + ZR);
-                ut[a] = (ZL * sl.u[a] + ZR * sr.u[a] + sR - sL) / (ZL + ZR);
-            }
-        }
-    }
-    // physical flux of the selected side; in the star regions the tangential
-    // stress is replaced by its face value
+    for (int a = 0; a < DIM; a++) ut[a] = mix32_upwind(wlf, sl.u[a], sr.u[a]);
     T sig[DIM];
 #pragma unroll
-    for (int a = 0; a < DIM; a++) sig[a] = (a == D ? -K.p : T(0)) + (SOLID ? T(2) * K.G * K.H[a][D] : T(0));
-    T work = T(0), work_n = T(0), work_s = T(0);
+    for (int a = 0; a < DIM; a++) sig[a] = (a == D ? -K.p : T(0));
+    T work = T(0), work_n = T(0);
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
         work += K.u[a] * sig[a];
         if (a == D) work_n += K.u[a] * sig[a];
-        else work_s += ut[a] * sig_t[a];
     }
     const T chi = star ? (SK - uK) / (SK - Ss) : T(0);
 #pragma unroll
@@ -972,21 +1361,13 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
         const T F = K.ar[l] * uK;
         out[L::IAR + l] = star ? F + SK * (K.ar[l] * chi - K.ar[l]) : F;
     }
-    if constexpr (SOLID == 2) {
-        // plastic-strain planes: carried like the partial densities
-#pragma unroll
-        for (int l = 0; l < NMAT; l++) {
-            const T m = K.ar[l] * K.eps[l];
-            out[L::IH + l] = star ? m * uK + SK * (m * chi - m) : m * uK;
-        }
-    }
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
         const T m = K.rho * K.u[a];
         const T Us = K.rho * chi * (a == D ? Ss : K.u[a]);
         if (star) {
             const T Fa = m * uK - (a == D ? sig[a] : T(0));
-            out[L::IMOM + a] = Fa + SK * (Us - m) - (a == D ? T(0) : sig_t[a]);
+            out[L::IMOM + a] = Fa + SK * (Us - m);
         } else {
             out[L::IMOM + a] = m * uK - sig[a];
         }
@@ -994,8 +1375,134 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
     {
         const T EK = K.rhoE / K.rho;
         const T Us = K.rho * chi * (EK + (Ss - uK) * (Ss + TK / (K.rho * (SK - uK))));
-        out[L::IE] = star ? (K.rhoE * uK - work_n) + SK * (Us - K.rhoE) - work_s : K.rhoE * uK - work;
+        out[L::IE] = star ? (K.rhoE * uK - work_n) + SK * (Us - K.rhoE) : K.rhoE * uK - work;
     }
+    if (star && g.hllc_lm) {
+        const T Ma = m_max(m_abs(uL) / cL, m_abs(uR) / cR);
+        const T ph = m_sin(m_min(T(1), Ma / T(0.1)) * T(3.14159265358979323846) / T(2));
+        const T k = T(-0.5) * (T(1) - ph);
+        mix32_star_jump<T, DIM, NMAT, D>(sl, SL, TL, Ss, k * SL, out);
+        mix32_star_jump<T, DIM, NMAT, D>(sr, SR, TR, Ss, k * SR, out);
+    }
+    const T us = (region == 0) ? uL : ((region == 3) ? uR : Ss);
+#pragma unroll
+    for (int l = 0; l < NMAT - 1; l++) out[L::IPHI + l] = mix32_upwind(wlf, wL[L::IPHI + l], wR[L::IPHI + l]) * us;
+    out[L::IR] = (vr > T(0)) ? wL[L::IR] * vr : ((vr < T(0)) ? wR[L::IR] * vr : T(0));
+    out[L::NVAR] = us;
+}
+
+// HLLC flux across a face normal to direction D (Sec. 3.1: Toro's HLLC; the
+// fluid pressure replaced by the normal traction T = p - 2G devH_DD for solids;
+// Davis wave speeds; partial densities scaled like the mixture density).
+// out[0..NVAR-1]: flux of every plane (r: upwind with the body velocity vr),
+// out[NVAR]: face velocity u*_D, out[NVAR+1+b]: V*_{D b} (upwind by S*).
+//
+// In the star regions F_K + S_K (U*_K - U_K) is, by the jump conditions across
+// S_K, the flux of the star state itself: with d = S_K - u_K, the mass flux
+// M = rho d S*/(S_K - S*), T* = T_K + rho d (S* - u_K), the normal momentum's
+// M S* + T* and the energy's S* (E* + T*), E* = (d E - T_K u_K + T* S*)/(S_K - S*):
+// half the operations, and no differences of large terms at low Mach numbers.
+// The energy is formed for the upwind side only.
+template <class T, int DIM, int NMAT, int SOLID, int D>
+__device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR, T vr, T *out)
+{
+    using L = Lay<DIM, NMAT, SOLID>;
+    if constexpr (mix32<T, NMAT, SOLID>()) {
+        mix32_riemann<T, DIM, NMAT, D>(g, wL, wR, vr, out);
+        return;
+    }
+    State<T, DIM, NMAT, SOLID> sl, sr;
+    state_from_prim<T, DIM, NMAT, SOLID>(g, wL, sl);
+    state_from_prim<T, DIM, NMAT, SOLID>(g, wR, sr);
+    const T uL = sl.u[D], uR = sr.u[D];
+    const T TL = SOLID ? m_fma(T(-2) * sl.G, sl.H[D][D], sl.p) : sl.p;
+    const T TR = SOLID ? m_fma(T(-2) * sr.G, sr.H[D][D], sr.p) : sr.p;
+    const T SL = m_min(uL - sl.c, uR - sr.c);
+    const T SR = m_max(uL + sl.c, uR + sr.c);
+    // contact speed; the numerator's products are rounded one by one and
+    // summed left to right, so that mirror-image states (a wall face) give
+    // S* = 0 exactly
+    const T dL = SL - uL, dR = SR - uR;
+    const T mL = mul_rn(sl.rho, dL), mR = mul_rn(sr.rho, dR);
+    const T num = add_rn(add_rn(TR - TL, mul_rn(mL, uL)), -mul_rn(mR, uR));
+    const T Ss = num * m_rcp(mL - mR);
+    // regions: left of S_L, left star, right star, right of S_R
+    const bool all_left = m_ge0(SL);
+    const bool left = all_left || m_ge0(Ss);
+    const bool star = !all_left && (left || m_pos(SR));
+    // quantities carried by the contact take the left value for S* > 0, the
+    // right one for S* < 0 and the mean of both at S* = 0 (mirror-symmetric
+    // at a wall face)
+    const int sgn = m_pos(Ss) ? 1 : (m_neg(Ss) ? -1 : 0);
+    State<T, DIM, NMAT, SOLID> K;
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) {
+        K.ar[l] = m_sel(left, sl.ar[l], sr.ar[l]);
+        if (SOLID == 2) K.eps[l] = m_sel(left, sl.eps[l], sr.eps[l]);
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) K.u[a] = m_sel(left, sl.u[a], sr.u[a]);
+    K.rho = m_sel(left, sl.rho, sr.rho);
+    K.p = m_sel(left, sl.p, sr.p);
+    K.den = NMAT == 1 ? sl.den : m_sel(left, sl.den, sr.den);
+    K.Q = (NMAT == 1 && SOLID == 0) && matc<T>(g, 0).kind != 2 ? sl.Q : m_sel(left, sl.Q, sr.Q);
+    const T SK = m_sel(left, SL, SR), TK = m_sel(left, TL, TR), dK = m_sel(left, dL, dR), mK = m_sel(left, mL, mR);
+    const T uK = K.u[D];
+    const T EK = state_energy<T, DIM, NMAT, SOLID>(K);
+    // Tangential traction and velocity at the face: the linear shear-wave
+    // Riemann problem (sigma -/+ Z u constant along the shear characteristics,
+    // Z = sqrt(rho G)); a gas (Z = 0) transmits no shear.  Without shear
+    // stiffness on either side the tangential velocity is upwind by S*.  Right
+    // and left of all waves it is the upwind side's own.
+    T sig_t[DIM], us[DIM];
+    T work_s = T(0);
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+        sig_t[a] = T(0);
+        us[a] = a == D ? (star ? Ss : uK) : (star && sgn == 0 ? T(0.5) * (sl.u[a] + sr.u[a]) : K.u[a]);
+    }
+    if (SOLID) {
+        const T ZL = m_sqrt(sl.rho * sl.G), ZR = m_sqrt(sr.rho * sr.G);
+        const bool stiff = m_pos(ZL + ZR);
+        const T iZ = m_rcp(ZL + ZR);
+#pragma unroll
+        for (int a = 0; a < DIM; a++) {
+            if (a == D) continue;
+            const T sL = T(2) * sl.G * sl.H[a][D], sR = T(2) * sr.G * sr.H[a][D];
+            if (!star) {
+                sig_t[a] = m_sel(left, sL, sR);
+            } else if (stiff) {
+                sig_t[a] = (ZR * sL + ZL * sR + ZL * ZR * (sr.u[a] - sl.u[a])) * iZ;
+                us[a] = (ZL * sl.u[a] + ZR * sr.u[a] + sR - sL) * iZ;
+            }
+            work_s += us[a] * sig_t[a];
+        }
+    }
+    // cS: transport velocity of the upwind side's contents (rho* S*/rho_K, or u_K)
+    T cS, Tf, EF;
+    if (star) {
+        const T iD = m_rcp(SK - Ss);
+        cS = dK * iD * Ss;
+        Tf = m_fma(mK, Ss - uK, TK);
+        const T Es = m_fma(dK, EK, m_fma(Tf, Ss, -(TK * uK))) * iD;
+        EF = Ss * (Es + Tf);
+    } else {
+        cS = uK;
+        Tf = TK;
+        EF = uK * (EK + TK);
+    }
+    const T M = K.rho * cS;
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) out[L::IAR + l] = NMAT == 1 ? M : K.ar[l] * cS;
+    if constexpr (SOLID == 2) {
+        // plastic-strain planes: carried like the partial densities
+#pragma unroll
+        for (int l = 0; l < NMAT; l++) out[L::IH + l] = K.eps[l] * out[L::IAR + l];
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++)
+        out[L::IMOM + a] = a == D ? m_fma(M, us[D], Tf) : (SOLID ? M * K.u[a] - sig_t[a] : M * K.u[a]);
+    out[L::IE] = SOLID ? EF - work_s : EF;
     if (star && g.hllc_lm) {
         // HLLC-LM (the published low-Mach form): the centred flux
         // (F_L + F_R)/2 + [phi S_L (U*_L - U_L) + |S*| (U*_L - U*_R) + phi S_R (U*_R - U_R)]/2
@@ -1003,43 +1510,83 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
         // number.  With the jump conditions across the three waves this is
         // the HLLC flux above minus (1 - phi)/2 [S_L (U*_L - U_L) + S_R (U*_R - U_R)]
         // on the partial densities, momenta and energy.
-        const T Ma = m_max(m_abs(uL) / cL, m_abs(uR) / cR);
+        const T Ma = m_max(m_abs(uL) * m_rcp(sl.c), m_abs(uR) * m_rcp(sr.c));
         const T ph = m_sin(m_min(T(1), Ma / T(0.1)) * T(3.14159265358979323846) / T(2));
         const T k = T(-0.5) * (T(1) - ph);
         star_jump<T, DIM, NMAT, SOLID, D>(sl, SL, TL, Ss, k * SL, out);
         star_jump<T, DIM, NMAT, SOLID, D>(sr, SR, TR, Ss, k * SR, out);
     }
-    // interface state at x/t = 0
-    T us[DIM];
 #pragma unroll
-    for (int a = 0; a < DIM; a++) us[a] = star ? ut[a] : K.u[a];
-    us[D] = (region == 0) ? uL : ((region == 3) ? uR : Ss);
+    for (int l = 0; l < NMAT - 1; l++) out[L::IPHI + l] = upwind_mix(sgn, wL[L::IPHI + l], wR[L::IPHI + l]) * us[D];
+    // V*: upwind by S*; F(V_ab) = V*_ab u*_D - V*_Db u*_a, V*_Db stored whenever b < DIM or (D,b) = (2,2)
+    T vs[L::NV > 0 ? L::NV : 1];
 #pragma unroll
-    for (int l = 0; l < NMAT - 1; l++) out[L::IPHI + l] = upwind_mix(wlf, wL[L::IPHI + l], wR[L::IPHI + l]) * us[D];
+    for (int c = 0; c < L::NV; c++) vs[c] = upwind_mix(sgn, wL[L::IV + c], wR[L::IV + c]);
 #pragma unroll
     for (int c = 0; c < L::NV; c++) {
         const int a = v_row(DIM, c), b = v_col(DIM, c);
-        // F(V_ab) = V*_ab u*_D - V*_Db u*_a ; V*_Db is stored whenever b < DIM or (D,b) = (2,2)
-        T vdb = T(0);
+        T F = vs[c] * us[D];
 #pragma unroll
         for (int cc = 0; cc < L::NV; cc++)
-            if (v_row(DIM, cc) == D && v_col(DIM, cc) == b) vdb = upwind_mix(wlf, wL[L::IV + cc], wR[L::IV + cc]);
-        const T ua = (a < DIM) ? us[a] : T(0);
-        out[L::IV + c] = upwind_mix(wlf, wL[L::IV + c], wR[L::IV + c]) * us[D] - vdb * ua;
+            if (v_row(DIM, cc) == D && v_col(DIM, cc) == b && a < DIM) F -= vs[cc] * us[a];
+        // the row of D itself: V*_Db u*_D - V*_Db u*_D
+        out[L::IV + c] = a == D ? T(0) : F;
     }
-    out[L::IR] = (vr > T(0)) ? wL[L::IR] * vr : ((vr < T(0)) ? wR[L::IR] * vr : T(0));
+    out[L::IR] = m_pos(vr) ? wL[L::IR] * vr : (m_neg(vr) ? wR[L::IR] * vr : T(0));
     out[L::NVAR] = us[D];
 #pragma unroll
     for (int b = 0; b < L::NB; b++) {
         T vdb = T(0);
 #pragma unroll
         for (int cc = 0; cc < L::NV; cc++)
-            if (v_row(DIM, cc) == D && v_col(DIM, cc) == b) vdb = upwind_mix(wlf, wL[L::IV + cc], wR[L::IV + cc]);
+            if (v_row(DIM, cc) == D && v_col(DIM, cc) == b) vdb = vs[cc];
         out[L::NVAR + 1 + b] = vdb;
     }
 }
 
 // -------------------------------------------------------- plastic return
+
+// cosh(y) and sinh(y)/y of y^2 (>= 0), FP64: their series to 2^-53 below
+// y^2 = 0.02 (elastic metals: y is half the yield strain), exp above.
+__device__ __forceinline__ void cosh_sinhc(double y2, double &ch, double &sh)
+{
+    if (m_less(y2, 0.02)) {
+        double c = 1.0 / 3628800.0;                      // 1/10!
+        c = fma(c, y2, 1.0 / 40320.0);
+        c = fma(c, y2, 1.0 / 720.0);
+        c = fma(c, y2, 1.0 / 24.0);
+        c = fma(c, y2, 0.5);
+        ch = fma(c, y2, 1.0);
+        double s = 1.0 / 39916800.0;                     // 1/11!
+        s = fma(s, y2, 1.0 / 362880.0);
+        s = fma(s, y2, 1.0 / 5040.0);
+        s = fma(s, y2, 1.0 / 120.0);
+        s = fma(s, y2, 1.0 / 6.0);
+        sh = fma(s, y2, 1.0);
+        return;
+    }
+    const double y = sqrt(y2), e = exp(y), i = 1.0 / e;
+    ch = 0.5 * (e + i);
+    sh = 0.5 * (e - i) / y;
+}
+
+// exp(x): its series to 2^-53 for |x| < 0.0625, exp otherwise
+__device__ __forceinline__ double exp_near0(double x)
+{
+    if (m_less(m_abs(x), 0.0625)) {
+        double e = 1.0 / 362880.0;                       // 1/9!
+        e = fma(e, x, 1.0 / 40320.0);
+        e = fma(e, x, 1.0 / 5040.0);
+        e = fma(e, x, 1.0 / 720.0);
+        e = fma(e, x, 1.0 / 120.0);
+        e = fma(e, x, 1.0 / 24.0);
+        e = fma(e, x, 1.0 / 6.0);
+        e = fma(e, x, 0.5);
+        e = fma(e, x, 1.0);
+        return fma(e, x, 1.0);
+    }
+    return exp(x);
+}
 
 // Perfect plasticity by instantaneous radial return, in FP64: the stored A is
 // replaced by its symmetric unimodular stretch Q diag(exp(s d_k)) Q^T with d_k
@@ -1050,29 +1597,43 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
 // yield(svm, |d|, J2) gives the yield stress for the trial von Mises stress
 // svm and deviatoric log-stretch norm |d| (Johnson-Cook: plastic strain,
 // temperature and rate); the constant-sigma_Y form ignores its arguments.
+//
+// In 2-D the in-plane log-stretches are -d2/2 +- k/2 (stretch_log), so the new
+// in-plane block is e^{-s d2/2} [cosh(s k/2) I + sinh(s k/2) (c_2, s_2)]: the
+// FP64 pipe does some 75 operations for an elastic or yielding metal cell in
+// place of three logarithms, three exponentials, a root and divisions.
 template <int DIM, class Y>
 __device__ __forceinline__ double plastic_return_y(double A[3][3], double G, Y yield)
 {
-    double H[3][3], J2;
-    Eig2 e;
-    stretch_log<DIM>(A, H, J2, e);
-    const double svm = sqrt(1.5) * 2.0 * G * sqrt(J2);
-    const double sigY = yield(svm, sqrt(J2), J2);
-    const double sc = (svm > sigY) ? sigY / svm : 1.0;
-    // equivalent plastic strain of the removed deviatoric log-strain (1 - s)|d|
-    const double deps = sc < 1.0 ? sqrt(2.0 / 3.0) * (1.0 - sc) * sqrt(J2) : 0.0;
-    const double e0 = exp(sc * e.d[0]), e1 = exp(sc * e.d[1]), e2 = exp(sc * e.d[2]);
-    const double av = 0.5 * (e0 + e1), df = 0.5 * (e0 - e1);
-    A[0][0] = av + df * e.c2;
-    A[1][1] = av - df * e.c2;
-    A[0][1] = A[1][0] = df * e.s2;
-    A[2][2] = e2;
-    A[0][2] = A[2][0] = A[1][2] = A[2][1] = 0.0;
-    if (DIM == 1) {
-        A[0][0] = e0;
-        A[1][1] = e1;
-        A[0][1] = A[1][0] = 0.0;
+    StretchLog<double> e;
+    stretch_log<double, DIM>(A, e);
+    const double nd = m_sqrt(e.J2);
+    const double svm = sqrt(6.0) * G * nd;
+    const double sigY = yield(svm, nd, e.J2);
+    double sc = 1.0, deps = 0.0;
+    if (svm > sigY) {
+        sc = sigY / svm;
+        // equivalent plastic strain of the removed deviatoric log-strain (1 - s)|d|
+        deps = sqrt(2.0 / 3.0) * (1.0 - sc) * nd;
     }
+    if (DIM == 1) {
+        A[0][0] = exp(sc * e.half);
+        A[1][1] = exp(sc * e.b01);
+        A[2][2] = exp(sc * e.d2);
+        A[0][1] = A[1][0] = 0.0;
+    } else {
+        const double h = 0.5 * sc;
+        double ch, sh;
+        cosh_sinhc(h * h * e.k2, ch, sh);
+        const double m = exp_near0(-h * e.d2);
+        const double q = m * sh * (h * e.q);     // sinh(s k/2)/|(half, b01)|, times the mean stretch
+        ch *= m;
+        A[0][0] = fma(q, e.half, ch);
+        A[1][1] = fma(-q, e.half, ch);
+        A[0][1] = A[1][0] = q * e.b01;
+        A[2][2] = m_rcp(m * m);
+    }
+    A[0][2] = A[2][0] = A[1][2] = A[2][1] = 0.0;
     return deps;
 }
 
@@ -1121,10 +1682,10 @@ __device__ __forceinline__ double jc_mixture_yield(const GridP &g, const R *w, d
         if (g.mat[l].jc) {
             double eps = 0.0;
             if constexpr (SOLID == 2) eps = (double)w[L::IH + l];
-            sy = jc_yield(g.mat[l], eps, rate, 298.0 + (p - r.pref) / (rl * r.Gam * g.mat[l].jc_cv));
+            sy = jc_yield(g.mat[l], eps, rate, 298.0 + (p - r.pref) * m_rcp(rl * g.mc_d[l].Gam * g.mat[l].jc_cv));
         }
-        num += ph * sy / r.Gam;
-        den += ph / r.Gam;
+        num += ph * sy * g.mc_d[l].invGam;
+        den += ph * g.mc_d[l].invGam;
     }
     return num / den;
 }

@@ -646,13 +646,10 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
                     zlo = min(zlo, z);
                     zhi = max(zhi, z);
                 }
-                float w[5];
-                gas3_prim(a, o, 0u, w);
-                const float c2 = __fdividef(a.Gam * w[4] + (w[4] - a.pref0), w[0]);
+                const float inv[3] = {a.idx, a.idy, a.idz};
+                float c2;
+                smax_cell = fmaxf(smax_cell, gas_speed<3>(a.Gam, a.pref0, o, inv, c2));
                 if (!(c2 > 0.f)) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
-                const float cs = sqrtf(c2);
-                smax_cell = fmaxf(smax_cell,
-                                  (fabsf(w[1]) + cs) * a.idx + (fabsf(w[2]) + cs) * a.idy + (fabsf(w[3]) + cs) * a.idz);
             }
         }
         if (own) {

@@ -278,12 +278,10 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
                     bx1 = max(bx1, gx);
                     by1 = max(by1, j);
                 }
-                float wv[4];
-                gas_prim(a, o[0], o[1], o[2], o[3], wv);
-                const float c2 = __fmul_rn(fmaf(a.Gam, wv[3], wv[3] - a.pref0), gas_rcp(wv[0]));
+                const float inv[2] = {idx, idy};
+                float c2;
+                smax = fmaxf(smax, gas_speed<2>(a.Gam, a.pref0, o, inv, c2));
                 if (!(c2 > 0.f)) atomicOr(&ctl->err, (unsigned)ERR_SOUND);
-                const float cs = sqrtf(c2);
-                smax = fmaxf(smax, fmaf(fabsf(wv[1]) + cs, idx, __fmul_rn(fabsf(wv[2]) + cs, idy)));
             }
         }
         P0 = P1;

@@ -192,19 +192,23 @@ __device__ __forceinline__ void block_sum3_f32(const float v[3], float *scratch 
     }
 }
 
+// maximum that passes over a NaN
+__device__ __forceinline__ double nan_max(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ float nan_max(float a, float b) { return fmaxf(a, b); }
+
 // Block maximum of one value per thread (fixed order; result in thread 0).
 template <int THREADS, class T>
 __device__ __forceinline__ T block_max(T v, T *scratch /* 32 */)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = m_max(v, __shfl_down_sync(0xffffffffu, v, o));
+    for (int o = 16; o > 0; o >>= 1) v = nan_max(v, __shfl_down_sync(0xffffffffu, v, o));
     if (lane == 0) scratch[warp] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         constexpr int NW = (THREADS + 31) / 32;
         T r = scratch[0];
-        for (int w = 1; w < NW; w++) r = m_max(r, scratch[w]);
+        for (int w = 1; w < NW; w++) r = nan_max(r, scratch[w]);
         v = r;
     }
     return v;
@@ -462,8 +466,7 @@ __device__ __forceinline__ void seed_star(const GridP &g, const R nv[3], const R
     }
     const R TL = SOLID ? sl.p - R(2) * sl.G * HnL : sl.p;
     const R TR = SOLID ? sr.p - R(2) * sr.G * HnR : sr.p;
-    const R cL = m_sqrt(sl.c2), cR = m_sqrt(sr.c2);
-    const R SL = m_min(unL - cL, unR - cR), SR = m_max(unL + cL, unR + cR);
+    const R SL = m_min(unL - sl.c, unR - sr.c), SR = m_max(unL + sl.c, unR + sr.c);
     const R Ss = (TR - TL + sl.rho * unL * (SL - unL) - sr.rho * unR * (SR - unR)) /
                  (sl.rho * (SL - unL) - sr.rho * (SR - unR));
     const R chi = (SR - unR) / (SR - Ss);
@@ -474,7 +477,7 @@ __device__ __forceinline__ void seed_star(const GridP &g, const R nv[3], const R
     const R rs = sr.rho * chi;
 #pragma unroll
     for (int a = 0; a < DIM; a++) q[L::IMOM + a] = rs * (Ss * nv[a] + (sr.u[a] - unR * nv[a]));
-    const R ER = sr.rhoE / sr.rho;
+    const R ER = state_energy<R, DIM, NMAT, SOLID>(sr) / sr.rho;
     q[L::IE] = rs * (ER + (Ss - unR) * (Ss + TR / (sr.rho * (SR - unR))));
 #pragma unroll
     for (int c = 0; c < L::NV; c++) q[L::IV + c] = wr[L::IV + c];
@@ -1010,7 +1013,8 @@ __device__ __forceinline__ void face_pass(const GridP &g, const R *sW, R *sF, R 
 #pragma unroll
             for (int k = 0; k < 6; k++) s[k] = sW[v * B::N + bc + (k - 3) * SD];
             const bool frac = (v >= L::IPHI && v < L::IPHI + NMAT - 1) || v == L::IR;
-            recon_face<R>(g, s, frac, wL[v], wR[v]);
+            if constexpr (mix32<R, NMAT, SOLID>()) mix32_recon_face<R>(g, s, frac, wL[v], wR[v]);
+            else recon_face<R>(g, s, frac, wL[v], wR[v]);
         }
         R F[L::NF];
         riemann<R, DIM, NMAT, SOLID, D>(g, wL, wR, vr, F);
@@ -1236,16 +1240,9 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
         if (STAGE == 3) rigid_new = o[L::IR] > R(0.5);
         if (STAGE == 3) {
             // CFL wave speed of the new state, in the compute precision
-            R w[L::NVAR];
-            cons_to_prim<R, DIM, NMAT, SOLID>(g, o, w);
-            State<R, DIM, NMAT, SOLID> s;
-            state_from_prim<R, DIM, NMAT, SOLID>(g, w, s);
-            if (!(s.c2 > R(0))) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
-            const R cs = m_sqrt(s.c2);
-            R sum = R(0);
-#pragma unroll
-            for (int d = 0; d < DIM; d++) sum += (m_abs(s.u[d]) + cs) / gridc<R>(g).dx[d];
-            smax_cell = sum;
+            R cs;
+            smax_cell = cell_speed<R, DIM, NMAT, SOLID>(g, o, cs);
+            if (!(cs > R(0))) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
         }
     }
     if (STAGE == 3) {
@@ -1336,16 +1333,10 @@ __global__ void __launch_bounds__(256) k_cfl(const void *Uv, double *partials, G
     double red[4] = {0.0, 0.0, 0.0, 0.0};
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < g.ncell;
          c += (long long)gridDim.x * blockDim.x) {
-        R q[L::NVAR], w[L::NVAR];
+        R q[L::NVAR], cs;
 #pragma unroll
         for (int v = 0; v < L::NVAR; v++) q[v] = U[v * P + c];
-        cons_to_prim<R, DIM, NMAT, SOLID>(g, q, w);
-        State<R, DIM, NMAT, SOLID> s;
-        state_from_prim<R, DIM, NMAT, SOLID>(g, w, s);
-        const R cs = m_sqrt(s.c2);
-        R sum = R(0);
-#pragma unroll
-        for (int d = 0; d < DIM; d++) sum += (m_abs(s.u[d]) + cs) / gridc<R>(g).dx[d];
+        const R sum = cell_speed<R, DIM, NMAT, SOLID>(g, q, cs);
         double sd = (double)sum;
         if (!(sd == sd)) sd = __longlong_as_double(0x7ff0000000000000LL);   // NaN -> +inf: dt = 0
         red[0] = fmax(red[0], sd);

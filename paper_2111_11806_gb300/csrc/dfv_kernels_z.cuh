@@ -285,15 +285,9 @@ __global__ void __launch_bounds__(ZGeo::THREADS, 2) k_stage_z(StageArgs a, GridP
                     zlo = min(zlo, z);
                     zhi = max(zhi, z);
                 }
-                R w[L::NVAR];
-                cons_to_prim<R, 3, NMAT, 0>(g, o, w);
-                State<R, 3, NMAT, 0> s;
-                state_from_prim<R, 3, NMAT, 0>(g, w, s);
-                if (!(s.c2 > R(0))) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
-                const R cs = m_sqrt(s.c2);
-                R sum = R(0);
-#pragma unroll
-                for (int d = 0; d < 3; d++) sum += (m_abs(s.u[d]) + cs) / gc.dx[d];
+                R cs;
+                const R sum = cell_speed<R, 3, NMAT, 0>(g, o, cs);
+                if (!(cs > R(0))) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
                 smax_cell = m_max(smax_cell, sum);
             }
 #pragma unroll
