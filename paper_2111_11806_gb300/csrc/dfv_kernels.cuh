@@ -801,15 +801,17 @@ __device__ __forceinline__ long long seed_box_cell(const GridP &g, const int lo[
     return ijk[0] + (long long)g.n[0] * (ijk[1] + (long long)g.n[1] * ijk[2]);
 }
 
-// The box cells, by whole blocks of at most 256 threads: block_first is the
-// block's first cell, stride the cells all blocks cover in one round.  Each
+// The box cells, by blocks blk of nblk, 256 threads each.  A round gives every
+// block at most 256 cells, and as few as 32 where the box is small: the band
+// cells lie together, and seeding one is a long chain of dependent work, so
+// that a box of 80 x 80 cells goes to 200 blocks, not to 25.  Each
 // thread tests one cell; the band cells go to a queue in shared memory and
 // are seeded by groups of SEED_G lanes (seed_compute), lane 0 storing the
 // state (MODE 0: into U, except r; MODE 1: into S with the flag).  MODE 2
 // copies S into U, one cell per thread.
 template <class R, int DIM, int NMAT, int SOLID, int OPT, int MODE>
-__device__ __forceinline__ void seed_box_cells(R *U, R *S, const Ctl *ctl, const GridP &g, long long block_first,
-                                               long long stride, bool next)
+__device__ __forceinline__ void seed_box_cells(R *U, R *S, const Ctl *ctl, const GridP &g, int blk, int nblk,
+                                               bool next)
 {
     using L = Lay<DIM, NMAT, SOLID>;
     const long long P = g.pitch;
@@ -817,9 +819,12 @@ __device__ __forceinline__ void seed_box_cells(R *U, R *S, const Ctl *ctl, const
     if (!seed_box(ctl, g, lo, hi, next)) return;
     const long long w = hi[0] - lo[0] + 1, h = hi[1] - lo[1] + 1;
     const long long total = w * h * (hi[2] - lo[2] + 1);
-    const bool small = total + stride < (1LL << 31);
+    const int spread = min(nblk, 152 * 4);   // CTAs that a small box goes to
+    const int per = (int)min(256LL, max(32LL, ((total + spread - 1) / spread + 31) & ~31LL));
+    const long long stride = (long long)nblk * per;
+    const bool small = total + (long long)nblk * 256 < (1LL << 31);
     if constexpr (MODE == 2) {
-        for (long long t = block_first + threadIdx.x; t < total; t += stride) {
+        for (long long t = blk * 256LL + threadIdx.x; t < total; t += nblk * 256LL) {
             int ijk[3];
             seed_apply<R, DIM, NMAT, SOLID>(U, S, g, seed_box_cell(g, lo, w, h, small, t, ijk));
         }
@@ -831,11 +836,11 @@ __device__ __forceinline__ void seed_box_cells(R *U, R *S, const Ctl *ctl, const
     __shared__ unsigned short s_q[256];
     __shared__ R s_b[5][256];
     const int sub = threadIdx.x & (SEED_G - 1);
-    for (long long b0 = block_first; b0 < total; b0 += stride) {     // the same rounds for the whole block
+    for (long long b0 = (long long)blk * per; b0 < total; b0 += stride) {     // the same rounds for the whole block
         if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
         const long long t = b0 + threadIdx.x;
-        if (t < total) {
+        if ((int)threadIdx.x < per && t < total) {
             int ijk[3];
             const long long c = seed_box_cell(g, lo, w, h, small, t, ijk);
             R rc, gr[3], gn;
@@ -892,8 +897,7 @@ __global__ void __launch_bounds__(256) k_seed(void *Uv, void *Sv, Ctl *ctl, Grid
         return;
     }
     seed_box_cells<R, DIM, NMAT, SOLID, OPT, MODE>(reinterpret_cast<R *>(Uv), reinterpret_cast<R *>(Sv), ctl, g,
-                                                   blockIdx.x * (long long)blockDim.x, (long long)nseed * blockDim.x,
-                                                   fin_mode != 0);
+                                                   (int)blockIdx.x, nseed, fin_mode != 0);
 }
 
 // Launch shape of k_seed: up to 16 CTAs of 256 threads per SM.
