@@ -96,7 +96,7 @@ long long stage_blocks(int dim, const int n[3])
 {
     // the smallest tile of dfv_kernels.cuh per dimension: an upper bound on the
     // number of stage blocks of either precision
-    const int tx = dim == 1 ? 256 : 32, ty = dim == 1 ? 1 : (dim == 2 ? 8 : 4), tz = dim == 3 ? 2 : 1;
+    const int tx = 32, ty = dim == 1 ? 1 : 4, tz = dim == 3 ? 2 : 1;
     const long long bx = (n[0] + tx - 1) / tx;
     const long long by = dim >= 2 ? (n[1] + ty - 1) / ty : 1;
     const long long bz = dim >= 3 ? (n[2] + tz - 1) / tz : 1;

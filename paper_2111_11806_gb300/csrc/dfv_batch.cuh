@@ -55,7 +55,7 @@ __device__ __forceinline__ void load_inst(const BatchInst *src, BatchInst *dst)
 // registers, a few dozen bytes of spills; 1 % faster than four on the
 // 256-ellipse batch), two otherwise.
 template <class R, int NMAT, int STAGE>
-__global__ void __launch_bounds__(Tile<2, (int)sizeof(R)>::THREADS, (sizeof(R) == 4 && NMAT == 1) ? 5 : 2)
+__global__ void __launch_bounds__(Tile<2, 0>::THREADS, (sizeof(R) == 4 && NMAT == 1) ? 5 : 2)
     k_batch_stage(BatchArgs b)
 {
     pdl_enter();
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(Tile<2, (int)sizeof(R)>::THREADS, (sizeof(R) =
         a.want_force = 0;
         a.early = 0;
         a.next = 0;
-        stage_tile<R, 2, NMAT, false, STAGE>(I.g, a, w.y % I.tiles_x, w.y / I.tiles_x, 0, w.y, I.ntiles);
+        stage_tile<R, 2, NMAT, 0, STAGE, 0>(I.g, a, w.y % I.tiles_x, w.y / I.tiles_x, 0, w.y, I.ntiles);
     }
 }
 
@@ -107,9 +107,9 @@ __global__ void __launch_bounds__(256) k_batch_seed(BatchArgs b)
 // CFL wave speed of every instance's stored state; the last tile of each
 // instance reduces its partials and sets its dt (b.final_mode).
 template <class R, int NMAT>
-__global__ void __launch_bounds__(Tile<2, (int)sizeof(R)>::THREADS) k_batch_cfl(BatchArgs b)
+__global__ void __launch_bounds__(Tile<2, 0>::THREADS) k_batch_cfl(BatchArgs b)
 {
-    using TL = Tile<2, (int)sizeof(R)>;
+    using TL = Tile<2, 0>;
     using L = Lay<2, NMAT, false>;
     __shared__ BatchInst s_inst;
     __shared__ long long s_item;
@@ -197,8 +197,8 @@ static __global__ void k_batch_set_run(Ctl *ctl, int count, double cfl, double t
 // Launch table of the batch kernels of one precision.
 template <class R, int NMAT>
 struct BK {
-    static constexpr int threads = Tile<2, (int)sizeof(R)>::THREADS;
-    static constexpr size_t smem = StageSmem<R, 2, NMAT, false>::bytes;
+    static constexpr int threads = Tile<2, 0>::THREADS;
+    static constexpr size_t smem = StageSmem<R, 2, NMAT, 0, 0>::bytes;
     static cudaError_t prepare()
     {
         cudaError_t e = cudaFuncSetAttribute(k_batch_stage<R, NMAT, 1>,

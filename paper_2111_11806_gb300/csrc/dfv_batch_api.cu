@@ -38,8 +38,7 @@ struct Plan {
 };
 
 // the tile of the 2-D stage kernels that the batch items address
-int tile_x(int precision) { return precision == DFV_FP32 ? dfv::Tile<2, 4>::TX : dfv::Tile<2, 8>::TX; }
-int tile_y(int precision) { return precision == DFV_FP32 ? dfv::Tile<2, 4>::TY : dfv::Tile<2, 8>::TY; }
+using BatchTile = dfv::Tile<2, 0>;
 
 int nvar_2d(int nmat) { return (nmat - 1) + nmat + 2 + 1 + 1; }
 
@@ -60,8 +59,8 @@ bool plan_batch(int count, const dfv_instance_desc *desc, int precision, int nma
         const long long pitch = (nc + 63) / 64 * 64;
         P.inst_off[i] = P.elems;
         P.elems += nvar * pitch;
-        P.tiles_x[i] = (desc[i].n[0] + tile_x(precision) - 1) / tile_x(precision);
-        P.tiles_y[i] = (desc[i].n[1] + tile_y(precision) - 1) / tile_y(precision);
+        P.tiles_x[i] = (desc[i].n[0] + BatchTile::TX - 1) / BatchTile::TX;
+        P.tiles_y[i] = (desc[i].n[1] + BatchTile::TY - 1) / BatchTile::TY;
         P.inst_part0[i] = P.nitems;
         P.nitems += (long long)P.tiles_x[i] * P.tiles_y[i];
         P.max_cells = std::max(P.max_cells, nc);

@@ -394,6 +394,11 @@ __device__ __forceinline__ float m_rcp(float x)
     return r;
 }
 
+// a/b (FP32: the product with the approximate reciprocal, rounded on its own --
+// what the fast division gives over the normal range, without its range fix-up)
+__device__ __forceinline__ float m_div(float a, float b) { return __fmul_rn(a, m_rcp(b)); }
+__device__ __forceinline__ double m_div(double a, double b) { return a * m_rcp(b); }
+
 // comparisons on the bits, with those of the ordinary operators: false for a
 // NaN, zero of either sign equal to zero
 __device__ __forceinline__ unsigned long long m_bits(double x) { return (unsigned long long)__double_as_longlong(x); }
@@ -659,7 +664,7 @@ __device__ __forceinline__ T phasic_density(const GridP &g, int l, T ar, T phc)
     if (m_less(phc, T(1e-6)) && m.has_rho0) return m.rho0;
     const T guard = gridc<T>(g).phi_guard;
     const T f = m_less(guard, phc) ? phc : guard;
-    return sizeof(T) == 4 ? ar / f : ar * m_rcp(f);
+    return m_div(ar, f);
 }
 
 // Mixture sums over the materials at phasic densities rhol (Sec. 2.2), all
@@ -779,7 +784,7 @@ __device__ __forceinline__ void mix32_state(const GridP &g, const T *w, State<T,
     for (int l = 0; l < NMAT; l++) {
         const MatC<T> &m = matc<T>(g, l);
         const T iG = m.invGam;
-        const T irl = T(1) / rhol[l];
+        const T irl = m_rcp(rhol[l]);
         if (m.kind == 2) {
             // a solid's equation of state in a fluid run (no stretch: J^2 = 0)
             const Ref<T> r = mat_ref<T>(m, rhol[l], T(0));
@@ -798,9 +803,9 @@ __device__ __forceinline__ void mix32_state(const GridP &g, const T *w, State<T,
     T ke = T(0);
 #pragma unroll
     for (int a = 0; a < DIM; a++) ke += T(0.5) * s.rho * s.u[a] * s.u[a];
-    const T iden = T(1) / den;
+    const T iden = m_rcp(den);
     s.rhoE = rhoe + ke;
-    s.c2 = Yn / s.rho * iden;
+    s.c2 = m_div(Yn, s.rho) * iden;
     s.c = m_sqrt(s.c2);
     s.G = s.sigY = T(0);
 }
@@ -950,7 +955,7 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
     }
     if constexpr (mix32<T, NMAT, SOLID>()) {
         T u[DIM];
-        const T irho = T(1) / rho;
+        const T irho = m_rcp(rho);
 #pragma unroll
         for (int a = 0; a < DIM; a++) u[a] = q[L::IMOM + a] * irho;
         T ke = T(0);
@@ -967,7 +972,7 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
             if (m.kind == 2) {
                 const Ref<T> r = mat_ref<T>(m, rhol[l], T(0));
                 pref = r.pref;
-                if (ar[l] != T(0)) num -= ar[l] * (r.re / rhol[l]);
+                if (ar[l] != T(0)) num -= ar[l] * m_div(r.re, rhol[l]);
             }
             num += phc * pref * m.invGam;
             den += phc * m.invGam;
@@ -978,7 +983,7 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
         for (int l = 0; l < NMAT; l++) w[L::IAR + l] = rhol[l];
 #pragma unroll
         for (int a = 0; a < DIM; a++) w[L::IMOM + a] = u[a];
-        w[L::IE] = num / den;
+        w[L::IE] = m_div(num, den);
         w[L::IR] = q[L::IR];
         return;
     }
@@ -1133,15 +1138,15 @@ __device__ __forceinline__ void prim_to_cons(const GridP &g, const T *w, T *q)
 
 // ------------------------------------------------------- reconstruction
 
-// The slope, THINC and face reconstruction of the FP32 fluid mixtures, and of
-// the volume fractions and r of every FP32 form (recon_face below says what
+// The slope, THINC and reconstruction of the FP32 fluid mixtures, and of
+// the volume fractions and r of every FP32 form (recon_cell below says what
 // they do), in one fixed order of operations: where MUSCL's and THINC's
 // boundary variations agree to round-off, the choice between them, and with it
 // the face value, would otherwise change with the order of rounding.
 template <class T>
 __device__ __forceinline__ T vanleer(T a, T b)
 {
-    return (a * b <= T(0)) ? T(0) : T(2) * a * b / (a + b);
+    return (a * b <= T(0)) ? T(0) : m_div(T(2) * a * b, a + b);
 }
 
 template <class T>
@@ -1163,30 +1168,28 @@ __device__ __forceinline__ bool mix32_thinc(const GridP &g, T qm, T q0, T qp, T 
     return true;
 }
 
+// face values lo (towards i-1) and hi (towards i+1) of cell i, s[0..4] = q_{i-2} .. q_{i+2}
 template <class T>
-__device__ __forceinline__ void mix32_recon_face(const GridP &g, const T *s, bool frac, T &qL, T &qR)
+__device__ __forceinline__ void mix32_recon_cell(const GridP &g, const T *s, bool frac, T &lo, T &hi)
 {
     const T slB = vanleer(s[2] - s[1], s[3] - s[2]);
-    const T slC = vanleer(s[3] - s[2], s[4] - s[3]);
-    const T Bp = s[2] + T(0.5) * slB, Cm = s[3] - T(0.5) * slC;
-    qL = Bp;
-    qR = Cm;
+    const T Bm = s[2] - T(0.5) * slB, Bp = s[2] + T(0.5) * slB;
+    lo = Bm;
+    hi = Bp;
     if (!frac || !g.use_thinc) return;
     const T slA = vanleer(s[1] - s[0], s[2] - s[1]);
-    const T slE = vanleer(s[4] - s[3], s[5] - s[4]);
-    const T Ap = s[1] + T(0.5) * slA, Bm = s[2] - T(0.5) * slB;
-    const T Cp = s[3] + T(0.5) * slC, Em = s[4] - T(0.5) * slE;
-    T tAm = s[1] - T(0.5) * slA, tAp = Ap, tBm = Bm, tBp = Bp, tCm = Cm, tCp = Cp, tEm = Em, tEp = s[4] + T(0.5) * slE;
+    const T slC = vanleer(s[3] - s[2], s[4] - s[3]);
+    const T Ap = s[1] + T(0.5) * slA, Cm = s[3] - T(0.5) * slC;
+    T tAm = s[1] - T(0.5) * slA, tAp = Ap, tBm = Bm, tBp = Bp, tCm = Cm, tCp = s[3] + T(0.5) * slC;
+    if (!mix32_thinc<T>(g, s[1], s[2], s[3], tBm, tBp)) return;   // MUSCL's values either way
     mix32_thinc<T>(g, s[0], s[1], s[2], tAm, tAp);
-    mix32_thinc<T>(g, s[1], s[2], s[3], tBm, tBp);
     mix32_thinc<T>(g, s[2], s[3], s[4], tCm, tCp);
-    mix32_thinc<T>(g, s[3], s[4], s[5], tEm, tEp);
     const T tbvBM = m_abs(Ap - Bm) + m_abs(Bp - Cm);
     const T tbvBT = m_abs(tAp - tBm) + m_abs(tBp - tCm);
-    const T tbvCM = m_abs(Bp - Cm) + m_abs(Cp - Em);
-    const T tbvCT = m_abs(tBp - tCm) + m_abs(tCp - tEm);
-    if (tbvBT < tbvBM) qL = tBp;
-    if (tbvCT < tbvCM) qR = tCm;
+    if (tbvBT < tbvBM) {
+        lo = tBm;
+        hi = tBp;
+    }
 }
 
 // half the van Leer slope 2ab/(a+b) of a cell from its backward and forward
@@ -1227,38 +1230,45 @@ __device__ __forceinline__ bool thinc(const GridP &g, T qm, T q0, T qp, T &fm, T
     return true;
 }
 
-// Left and right states at the face between cells f-1 and f of a pencil,
-// s[0..5] = q_{f-3} .. q_{f+2}.  MUSCL (van Leer) for every primitive; for a
-// volume fraction (frac = true) the BVD rule keeps a cell's THINC face values
-// only where its total boundary variation is strictly below MUSCL's.
+// Face values of cell i of a pencil, s[0..4] = q_{i-2} .. q_{i+2}: lo at its face
+// towards i-1, hi at its face towards i+1.  MUSCL (van Leer) for every
+// primitive (s[1..3] only); for a volume fraction (frac = true) the BVD rule
+// keeps the cell's THINC face values only where its total boundary variation
+// is strictly below MUSCL's (where the cell has none, nothing is to choose).
 template <class T>
-__device__ __forceinline__ void recon_face(const GridP &g, const T *s, bool frac, T &qL, T &qR)
+__device__ __forceinline__ void recon_cell(const GridP &g, const T *s, bool frac, T &lo, T &hi)
 {
     if (sizeof(T) == 4 && frac) {
-        mix32_recon_face<T>(g, s, frac, qL, qR);
+        mix32_recon_cell<T>(g, s, frac, lo, hi);
         return;
     }
     const T hB = half_slope(s[2] - s[1], s[3] - s[2]);
-    const T hC = half_slope(s[3] - s[2], s[4] - s[3]);
-    const T Bp = s[2] + hB, Cm = s[3] - hC;
-    qL = Bp;
-    qR = Cm;
+    const T Bm = s[2] - hB, Bp = s[2] + hB;
+    lo = Bm;
+    hi = Bp;
     if (!frac || !g.use_thinc) return;
+    T tBm, tBp;
+    if (!thinc<T>(g, s[1], s[2], s[3], tBm, tBp)) return;
     const T hA = half_slope(s[1] - s[0], s[2] - s[1]);
-    const T hE = half_slope(s[4] - s[3], s[5] - s[4]);
-    const T Ap = s[1] + hA, Bm = s[2] - hB;
-    const T Cp = s[3] + hC, Em = s[4] - hE;
-    T tAm = s[1] - hA, tAp = Ap, tBm = Bm, tBp = Bp, tCm = Cm, tCp = Cp, tEm = Em, tEp = s[4] + hE;
+    const T hC = half_slope(s[3] - s[2], s[4] - s[3]);
+    const T Ap = s[1] + hA, Cm = s[3] - hC;
+    T tAm = Ap, tAp = Ap, tCm = Cm, tCp = Cm;
     thinc<T>(g, s[0], s[1], s[2], tAm, tAp);
-    thinc<T>(g, s[1], s[2], s[3], tBm, tBp);
     thinc<T>(g, s[2], s[3], s[4], tCm, tCp);
-    thinc<T>(g, s[3], s[4], s[5], tEm, tEp);
     const T tbvBM = m_abs(Ap - Bm) + m_abs(Bp - Cm);
     const T tbvBT = m_abs(tAp - tBm) + m_abs(tBp - tCm);
-    const T tbvCM = m_abs(Bp - Cm) + m_abs(Cp - Em);
-    const T tbvCT = m_abs(tBp - tCm) + m_abs(tCp - tEm);
-    if (m_less(tbvBT, tbvBM)) qL = tBp;
-    if (m_less(tbvCT, tbvCM)) qR = tCm;
+    if (m_less(tbvBT, tbvBM)) {
+        lo = tBm;
+        hi = tBp;
+    }
+}
+
+// the same in the order of operations of a form
+template <class T, int NMAT, int SOLID>
+__device__ __forceinline__ void recon_form(const GridP &g, const T *s, bool frac, T &lo, T &hi)
+{
+    if constexpr (mix32<T, NMAT, SOLID>()) mix32_recon_cell<T>(g, s, frac, lo, hi);
+    else recon_cell<T>(g, s, frac, lo, hi);
 }
 
 // ------------------------------------------------------------- Riemann
@@ -1331,7 +1341,7 @@ __device__ __forceinline__ void mix32_riemann(const GridP &g, const T *wL, const
     const T SR = m_max(uL + cL, uR + cR);
     const T num = add_rn(add_rn(TR - TL, mul_rn(mul_rn(sl.rho, uL), SL - uL)),
                          -mul_rn(mul_rn(sr.rho, uR), SR - uR));
-    const T Ss = num / (sl.rho * (SL - uL) - sr.rho * (SR - uR));
+    const T Ss = m_div(num, sl.rho * (SL - uL) - sr.rho * (SR - uR));
     int region;
     if (SL >= T(0)) region = 0;
     else if (Ss >= T(0)) region = 1;
@@ -1355,7 +1365,7 @@ __device__ __forceinline__ void mix32_riemann(const GridP &g, const T *wL, const
         work += K.u[a] * sig[a];
         if (a == D) work_n += K.u[a] * sig[a];
     }
-    const T chi = star ? (SK - uK) / (SK - Ss) : T(0);
+    const T chi = star ? m_div(SK - uK, SK - Ss) : T(0);
 #pragma unroll
     for (int l = 0; l < NMAT; l++) {
         const T F = K.ar[l] * uK;
@@ -1373,8 +1383,8 @@ __device__ __forceinline__ void mix32_riemann(const GridP &g, const T *wL, const
         }
     }
     {
-        const T EK = K.rhoE / K.rho;
-        const T Us = K.rho * chi * (EK + (Ss - uK) * (Ss + TK / (K.rho * (SK - uK))));
+        const T EK = m_div(K.rhoE, K.rho);
+        const T Us = K.rho * chi * (EK + (Ss - uK) * (Ss + m_div(TK, K.rho * (SK - uK))));
         out[L::IE] = star ? (K.rhoE * uK - work_n) + SK * (Us - K.rhoE) : K.rhoE * uK - work;
     }
     if (star && g.hllc_lm) {

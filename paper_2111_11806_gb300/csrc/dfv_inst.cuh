@@ -11,70 +11,135 @@ namespace dfv {
 template <class R, int DIM, int NMAT, int SOLID>
 struct Impl {
     using L = Lay<DIM, NMAT, SOLID>;
-    using TL = Tile<DIM, (int)sizeof(R)>;
+    // tile sizes that are built: in FP32 the large one only (a CTA's time is
+    // then a chain of dependent work, not the SM's FP64 pipe, and the order of
+    // the pressure-force sum, which goes by tiles, stays)
+    static constexpr int NV = DIM <= 2 && sizeof(R) == 8 ? 2 : 1;
+
+    template <int V>
+    static dim3 tile_grid(const GridP &g)
+    {
+        using TL = Tile<DIM, V>;
+        return dim3((g.n[0] + TL::TX - 1) / TL::TX, (g.n[1] + TL::TY - 1) / TL::TY, (g.n[2] + TL::TZ - 1) / TL::TZ);
+    }
+    template <int V>
+    static long long tiles(const GridP &g)
+    {
+        const dim3 t = tile_grid<V>(g);
+        return (long long)t.x * t.y * t.z;
+    }
+
+    // Whether the stages run on the small tiles.  A stage takes about as long
+    // as the SM with the most tiles, ceil(tiles/SMs) of them; a small tile
+    // costs more per cell (halo cells, closing faces), in warps' work 2/9 of
+    // the large one in 1-D and 9/16 in 2-D.
+    static bool small_tiles(const GridP &g)
+    {
+        if constexpr (NV == 1) {
+            return false;
+        } else {
+            const long long sms = 152, big = (tiles<0>(g) + sms - 1) / sms, sml = (tiles<1>(g) + sms - 1) / sms;
+            return DIM == 1 ? 2 * sml < 9 * big : 9 * sml < 16 * big;
+        }
+    }
 
     static dim3 stage_grid(const GridP &g)
     {
-        return dim3((g.n[0] + TL::TX - 1) / TL::TX, (g.n[1] + TL::TY - 1) / TL::TY, (g.n[2] + TL::TZ - 1) / TL::TZ);
+        if constexpr (NV == 2)
+            if (small_tiles(g)) return tile_grid<1>(g);
+        return tile_grid<0>(g);
     }
 
-    static constexpr size_t smem = StageSmem<R, DIM, NMAT, SOLID>::bytes;
+    template <int V>
+    static constexpr size_t smem = StageSmem<R, DIM, NMAT, SOLID, V>::bytes;
 
-    // 3-D FP32 single-material fluids march along z (k_stage_z); stage 1
-    // with the pressure force keeps the tiled kernel, whose tiles own the
-    // force partials
-    static constexpr bool ZM = DIM == 3 && SOLID == 0 && NMAT == 1 && sizeof(R) == 4;
+    // 3-D single-material fluids march along z (k_stage_z); stage 1 with the
+    // pressure force keeps the tiled kernel, whose tiles own the force partials
+    static constexpr bool ZM = DIM == 3 && SOLID == 0 && NMAT == 1;
     static constexpr size_t zsmem = ZSmem<R, NMAT>::bytes;
-    // planes per CTA: 32 on the 256^3 sphere beats 16, 24, 64 and 256 (the
-    // six-plane prologue of a chunk against the CTA count for the 152 SMs)
-    static constexpr int ZCHUNK = 32;
 
-    static dim3 zgrid(const GridP &g)
+    // Planes per CTA: the chunk count that gives the SM with the most CTAs the
+    // fewest planes, a chunk's prologue (two more planes of conversions, one
+    // more z slope and face) counted as a plane and a half; among equals the fewest.
+    static int zchunk(const GridP &g)
     {
-        return dim3((g.n[0] + ZGeo::TX - 1) / ZGeo::TX, (g.n[1] + ZGeo::TY - 1) / ZGeo::TY,
-                    (g.n[2] + ZCHUNK - 1) / ZCHUNK);
+        using Z = ZGeo<R>;
+        const long long cols = (long long)((g.n[0] + Z::TX - 1) / Z::TX) * ((g.n[1] + Z::TY - 1) / Z::TY);
+        long long best = -1;
+        int zbest = g.n[2];
+        for (int k = 1; k <= g.n[2] && k <= 64; k++) {
+            const int zc = (g.n[2] + k - 1) / k;
+            const long long ctas = cols * ((g.n[2] + zc - 1) / zc), per = (ctas + 151) / 152;
+            const long long cost = per * (2 * zc + 3);
+            if (best < 0 || cost < best) {
+                best = cost;
+                zbest = zc;
+            }
+        }
+        return zbest;
+    }
+
+    static dim3 zgrid(const GridP &g, int zc)
+    {
+        using Z = ZGeo<R>;
+        return dim3((g.n[0] + Z::TX - 1) / Z::TX, (g.n[1] + Z::TY - 1) / Z::TY, (g.n[2] + zc - 1) / zc);
     }
 
     // Opt the stage kernels in to their dynamic shared memory on the current
     // device (called at grid creation, outside any stream capture).
+    template <class K>
+    static cudaError_t opt_in(K *k, size_t bytes)
+    {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    }
+    template <int V>
+    static cudaError_t prepare_v()
+    {
+        cudaError_t e = opt_in(k_stage<R, DIM, NMAT, SOLID, 1, V>, smem<V>);
+        if (e == cudaSuccess) e = opt_in(k_stage<R, DIM, NMAT, SOLID, 2, V>, smem<V>);
+        if (e == cudaSuccess) e = opt_in(k_stage<R, DIM, NMAT, SOLID, 3, V>, smem<V>);
+        // the first-wave size is looked up here, outside any stream capture
+        if (e == cudaSuccess) (void)first_wave<V>();
+        return e;
+    }
     static cudaError_t prepare()
     {
-        cudaError_t e = cudaFuncSetAttribute(k_stage<R, DIM, NMAT, SOLID, 1>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_stage<R, DIM, NMAT, SOLID, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_stage<R, DIM, NMAT, SOLID, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
-        // the first-wave size is looked up here, outside any stream capture
-        if (e == cudaSuccess) (void)first_wave();
+        cudaError_t e = prepare_v<0>();
+        if constexpr (NV == 2)
+            if (e == cudaSuccess) e = prepare_v<1>();
         if constexpr (ZM) {
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_stage_z<R, NMAT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)zsmem);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_stage_z<R, NMAT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)zsmem);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_stage_z<R, NMAT, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 1>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 2>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 3>, zsmem);
         }
         return e;
+    }
+
+    template <int S, int V>
+    static cudaError_t stage_v(const GridP &g, StageArgs a, cudaStream_t st)
+    {
+        a.early = S == 1 ? first_wave<V>() : 0;
+        return launch_pdl(k_stage<R, DIM, NMAT, SOLID, S, V>, tile_grid<V>(g), dim3(Tile<DIM, V>::THREADS), smem<V>, st,
+                          a, g);
     }
 
     template <int S>
     static cudaError_t stage_s(const GridP &g, const StageArgs &a, cudaStream_t st)
     {
         if constexpr (ZM) {
-            if (!(S == 1 && a.want_force))
-                return launch_pdl(k_stage_z<R, NMAT, S>, zgrid(g), dim3(ZGeo::THREADS), zsmem, st, a, g, ZCHUNK);
+            if (!(S == 1 && a.want_force)) {
+                const int zc = zchunk(g);
+                return launch_pdl(k_stage_z<R, NMAT, S>, zgrid(g, zc), dim3(ZGeo<R>::THREADS), zsmem, st, a, g, zc);
+            }
         }
-        return launch_pdl(k_stage<R, DIM, NMAT, SOLID, S>, stage_grid(g), dim3(TL::THREADS), smem, st, a, g);
+        if constexpr (NV == 2)
+            if (small_tiles(g)) return stage_v<S, 1>(g, a, st);
+        return stage_v<S, 0>(g, a, st);
     }
 
     // CTAs of the stage-1 kernel resident at once on the device (the first
     // wave), looked up once
+    template <int V>
     static int first_wave()
     {
         static int n = -1;
@@ -82,8 +147,8 @@ struct Impl {
             int dev = 0, sms = 0, per = 0;
             if (cudaGetDevice(&dev) != cudaSuccess ||
                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage<R, DIM, NMAT, SOLID, 1>, TL::THREADS,
-                                                              smem) != cudaSuccess) {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_stage<R, DIM, NMAT, SOLID, 1, V>,
+                                                              Tile<DIM, V>::THREADS, smem<V>) != cudaSuccess) {
                 (void)cudaGetLastError();
                 return 0;
             }
@@ -103,7 +168,7 @@ struct Impl {
         a.ctl = ctl;
         a.partials = partials;
         a.want_force = want_force;
-        a.early = s == 1 ? first_wave() : 0;
+        a.early = 0;   // set with the tile size
         a.next = next;
         if (s == 1) return stage_s<1>(g, a, st);
         if (s == 2) return stage_s<2>(g, a, st);
@@ -163,7 +228,7 @@ struct Impl {
 
     static const Ops *ops()
     {
-        static const Ops o = {L::NVAR, TL::THREADS, (int)sizeof(R), &prepare, &stage_grid, &seed, &stage, &cfl,
+        static const Ops o = {L::NVAR, Tile<DIM, 0>::THREADS, (int)sizeof(R), &prepare, &stage_grid, &seed, &stage, &cfl,
                               &p2c, &c2p, &c2f};
         return &o;
     }
@@ -177,13 +242,13 @@ const Ops *select_ops_nmat(int solid)
     // a stage tile must fit the 227 KB of shared memory a CTA may have (the
     // 3-D FP64 three-material fluid does not: not built)
     constexpr size_t lim = 227u * 1024u;
-    if constexpr (StageSmem<R, DIM, NMAT, 0>::bytes <= lim) {
+    if constexpr (StageSmem<R, DIM, NMAT, 0, 0>::bytes <= lim) {
         if (!solid) return Impl<R, DIM, NMAT, 0>::ops();
     }
     if constexpr (DIM <= 2) {
-        if constexpr (StageSmem<R, DIM, NMAT, 1>::bytes <= lim)
+        if constexpr (StageSmem<R, DIM, NMAT, 1, 0>::bytes <= lim)
             if (solid == 1) return Impl<R, DIM, NMAT, 1>::ops();
-        if constexpr (StageSmem<R, DIM, NMAT, 2>::bytes <= lim)
+        if constexpr (StageSmem<R, DIM, NMAT, 2, 0>::bytes <= lim)
             if (solid == 2) return Impl<R, DIM, NMAT, 2>::ops();
     }
     return nullptr;

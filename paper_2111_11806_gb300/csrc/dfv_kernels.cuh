@@ -3,7 +3,7 @@
 //               (queued per block, seeded by groups of 8 lanes); optionally
 //               with the previous step's finalize in one extra block
 //   k_stage<S>  one SSP-RK3 stage (Sec. 3.1): halo-3 tile of primitives in
-//               shared memory, per-face MUSCL-BVD-THINC + HLLC, divergence,
+//               shared memory, per-cell MUSCL-BVD-THINC, per-face HLLC, divergence,
 //               non-conservative terms, rigid mask, RK combination; stage 1
 //               also sums the pressure force, stage 3 applies the plastic
 //               return and reduces the CFL wave speed of the new state
@@ -20,48 +20,54 @@ namespace dfv {
 
 // ------------------------------------------------------------ tiling
 
-// Tile of one CTA: TX x TY x TZ cells, with one thread per face of the
-// largest face sweep (the extra warp covers the tile's closing faces).  2-D
-// tiles are 32 x 8 in both precisions: measured on the cylinder at 512^2 to
-// 2048^2, FP32 steps are 6-8 % shorter than with 32 x 16 tiles (more, smaller
-// CTAs balance better over the SMs than the taller tile saves in halo).
-template <int DIM, int W>
+// Tile of one CTA: TX x TY x TZ cells, one thread each, and as many extra
+// threads as a sweep has pencils at most, which do their closing faces.  V
+// selects the size: 0 the large one, whose halo costs least, 1 the small one,
+// for FP64 grids of few large tiles (small_tiles says when).
+template <int DIM, int V>
 struct Tile;
-template <int W>
-struct Tile<1, W> {
+template <>
+struct Tile<1, 0> {
     static constexpr int TX = 256, TY = 1, TZ = 1, THREADS = 288;
 };
-template <int W>
-struct Tile<2, W> {
+template <>
+struct Tile<1, 1> {
+    static constexpr int TX = 32, TY = 1, TZ = 1, THREADS = 64;
+};
+template <>
+struct Tile<2, 0> {
     static constexpr int TX = 32, TY = 8, TZ = 1, THREADS = 288;
 };
-template <int W>
-struct Tile<3, W> {
+template <>
+struct Tile<2, 1> {
+    static constexpr int TX = 32, TY = 4, TZ = 1, THREADS = 160;
+};
+template <>
+struct Tile<3, 0> {
     static constexpr int TX = 32, TY = 4, TZ = 2, THREADS = 384;
 };
 
-template <int DIM, int W>
+template <int DIM, int V>
 struct Box {
-    using TL = Tile<DIM, W>;
+    using TL = Tile<DIM, V>;
     static constexpr int HX = 3, HY = DIM >= 2 ? 3 : 0, HZ = DIM >= 3 ? 3 : 0;
     static constexpr int BX = TL::TX + 2 * HX, BY = TL::TY + 2 * HY, BZ = TL::TZ + 2 * HZ;
     static constexpr int N = BX * BY * BZ;
     static constexpr int CELLS = TL::TX * TL::TY * TL::TZ;
     static constexpr int FX = (TL::TX + 1) * TL::TY * TL::TZ;
-    static constexpr int FY = TL::TX * (TL::TY + 1) * TL::TZ;
-    static constexpr int FZ = TL::TX * TL::TY * (TL::TZ + 1);
+    static constexpr int FY = DIM >= 2 ? TL::TX * (TL::TY + 1) * TL::TZ : 0;
+    static constexpr int FZ = DIM >= 3 ? TL::TX * TL::TY * (TL::TZ + 1) : 0;
     static constexpr int MAXF = FX > FY ? (FX > FZ ? FX : FZ) : (FY > FZ ? FY : FZ);
     __host__ __device__ static constexpr int stride(int d) { return d == 0 ? 1 : (d == 1 ? BX : BX * BY); }
 };
 
-template <class R, int DIM, int NMAT, int SOLID>
+template <class R, int DIM, int NMAT, int SOLID, int V>
 struct StageSmem {
     using L = Lay<DIM, NMAT, SOLID>;
-    using B = Box<DIM, (int)sizeof(R)>;
-    // 2-D fluid tiles compute the faces of both directions before one
-    // barrier, so they keep one face array per direction (solids keep one:
-    // their larger face records would cost occupancy)
-    static constexpr int NSF = (DIM == 2 && SOLID == 0) ? 2 : 1;
+    using B = Box<DIM, V>;
+    // fluids keep one face array per direction or two in turn, which saves
+    // barriers (solids one: their larger face records would cost occupancy)
+    static constexpr int NSF = (DIM >= 2 && SOLID == 0) ? 2 : 1;
     static constexpr size_t floats = (size_t)L::NVAR * B::N + (size_t)NSF * L::NF * B::MAXF;
     static constexpr size_t bytes = ((sizeof(R) * floats + 7) & ~(size_t)7) + 4 * 32 * sizeof(double);
 };
@@ -935,11 +941,11 @@ struct StageArgs {
 // mirrored (wall) counts as touching; a clamped (outflow) halo is clamped.
 // Read before the seeding launch has finished: the box words come from L2
 // (written by an earlier launch, complete before this one started).
-template <int DIM, int W>
+template <int DIM, int V>
 __device__ __forceinline__ bool tile_touches_box(const GridP &g, const Ctl *ctl, int ox, int oy, int oz, bool next)
 {
-    using TL = Tile<DIM, W>;
-    using B = Box<DIM, W>;
+    using TL = Tile<DIM, V>;
+    using B = Box<DIM, V>;
     const bool valid = next || __ldcg(&ctl->rbox_valid) != 0;
     if (!valid) return true;
     const int *box = next ? ctl->rnext : ctl->rbox;
@@ -961,81 +967,120 @@ __device__ __forceinline__ bool tile_touches_box(const GridP &g, const Ctl *ctl,
     return true;
 }
 
-// Fluxes of every face of direction D of the tile into sF (no barrier).
-template <class R, int DIM, int NMAT, int SOLID, int D>
-__device__ __forceinline__ void face_pass(const GridP &g, const R *sW, R *sF, R vr)
+// Where a thread stands in the sweep of direction D: its own cell and the
+// face below it, or (extra threads) the pencil whose closing face it does.
+template <int DIM, int V, int D>
+struct Sweep {
+    using TL = Tile<DIM, V>;
+    using B = Box<DIM, V>;
+    static constexpr int T = D == 0 ? TL::TX : (D == 1 ? TL::TY : TL::TZ);
+    static constexpr int EX = TL::TX + (D == 0), EY = TL::TY + (D == 1);
+    static constexpr int SF = D == 0 ? 1 : (D == 1 ? EX : EX * EY);   // from a face to the next of its pencil
+    static constexpr int SB = B::stride(D);
+    static constexpr int LINES = B::CELLS / T;                        // pencils
+    static_assert(LINES <= TL::THREADS - B::CELLS, "one extra thread per pencil");
+    int box, face;    // box index of the cell, index of its lower face (extra threads: of cell 0 and face 0)
+    bool own, extra;
+
+    __device__ __forceinline__ Sweep()
+    {
+        const int t = threadIdx.x;
+        own = t < B::CELLS;
+        extra = !own && t - B::CELLS < LINES;
+        int lx, ly, lz;
+        if (own) {
+            lx = t % TL::TX;
+            ly = (t / TL::TX) % TL::TY;
+            lz = t / (TL::TX * TL::TY);
+        } else {
+            const int e = t - B::CELLS;
+            lx = D == 0 ? 0 : e % TL::TX;
+            ly = D == 0 ? e % TL::TY : (D == 1 ? 0 : e / TL::TX);
+            lz = D == 0 ? e / TL::TY : (D == 1 ? e / TL::TX : 0);
+        }
+        box = ((lz + B::HZ) * B::BY + (ly + B::HY)) * B::BX + (lx + B::HX);
+        face = (lz * EY + ly) * EX + lx;
+    }
+};
+
+// Reconstruction of direction D, each cell once: a thread forms both face
+// values of its own cell, leaves the upper one as the left state of the next
+// face in sQ and keeps the lower one, the right state of its own face, in
+// lo.  The extra threads do the same for the cells beyond the two ends of
+// their pencils (upper value of cell -1, lower value of cell T).  No barrier.
+template <class R, int DIM, int NMAT, int SOLID, int V, int D>
+__device__ __forceinline__ void slope_pass(const GridP &g, const R *sW, R *sQ, R vr, R *lo)
 {
     using L = Lay<DIM, NMAT, SOLID>;
-    using B = Box<DIM, (int)sizeof(R)>;
-    using TL = Tile<DIM, (int)sizeof(R)>;
-    constexpr int EX = TL::TX + (D == 0), EY = TL::TY + (D == 1), EZ = TL::TZ + (D == 2);
-    constexpr int NFACE = EX * EY * EZ;
-    constexpr int SD = B::stride(D);
-    // Faces to threads: with 32-wide tiles every warp takes one row of 32
-    // faces (lane = x), and in the x sweep the warps past the last row take
-    // the rows' closing faces (x = 32); otherwise a flat index.
-    constexpr bool ROWS = TL::TX == 32 && DIM >= 2;
-    constexpr int NROW = TL::TY * TL::TZ;                   // rows of the tile
-    // warps of work: one per face row, plus (x sweep) the closing faces
-    constexpr int WROWS = D == 0 ? NROW + (NROW + 31) / 32 : EY * EZ;
-    constexpr int ITEMS = ROWS ? WROWS * 32 : NFACE;
-    for (int t = threadIdx.x; t < ITEMS; t += TL::THREADS) {
-        int fx, fy, fz;
-        if constexpr (ROWS) {
-            const int lane = t & 31, warp = t >> 5;
-            int row;
-            if (D == 0 && warp >= NROW) {
-                row = (warp - NROW) * 32 + lane;
-                fx = TL::TX;
-                if (row >= NROW) continue;
-            } else {
-                row = warp;
-                fx = lane;
-                if (row >= EY * EZ) continue;
+    using B = Box<DIM, V>;
+    using S = Sweep<DIM, V, D>;
+    const S p;
+    if (!p.own && !p.extra) return;
+#pragma unroll
+    for (int v = 0; v < L::NVAR; v++) {
+        const bool frac = (v >= L::IPHI && v < L::IPHI + NMAT - 1) || v == L::IR;
+        // the upwind r flux (Sec. 3.1) vanishes for a body at rest in this
+        // direction, whatever the face values of r
+        if (v == L::IR && vr == R(0)) {
+            lo[v] = R(0);
+            continue;
+        }
+        R s[5], hi;
+        if (p.own || frac) {
+            // (one copy of the fractions' code, large with the BVD choice: the extra threads go through it twice)
+            const R *w = sW + v * B::N + p.box - (p.own ? 0 : S::SB);
+            R *q = sQ + v * B::MAXF + p.face + (p.own ? S::SF : 0);
+#pragma unroll 1
+            for (int pass = p.own ? 1 : 0; pass < 2; pass++) {
+#pragma unroll
+                for (int k = 0; k < 5; k++) s[k] = (frac || (k > 0 && k < 4)) ? w[(k - 2) * S::SB] : R(0);
+                recon_form<R, NMAT, SOLID>(g, s, frac, lo[v], hi);
+                if (p.own || pass == 0) *q = hi;
+                w += (S::T + 1) * S::SB;
             }
-            fy = row % EY;
-            fz = row / EY;
         } else {
-            if (t >= NFACE) continue;
-            fx = t % EX;
-            fy = (t / EX) % EY;
-            fz = t / (EX * EY);
+            const R *w = sW + v * B::N + p.box;
+            R dummy;
+#pragma unroll
+            for (int k = 1; k < 4; k++) s[k] = w[(k - 3) * S::SB];
+            recon_form<R, NMAT, SOLID>(g, s, frac, dummy, hi);
+            sQ[v * B::MAXF + p.face] = hi;
+#pragma unroll
+            for (int k = 1; k < 4; k++) s[k] = w[(k - 2 + S::T) * S::SB];
+            recon_form<R, NMAT, SOLID>(g, s, frac, lo[v], dummy);
         }
-        const int item = (fz * EY + fy) * EX + fx;
-        // box index of the cell on the right of the face
-        const int bc = ((fz + B::HZ) * B::BY + (fy + B::HY)) * B::BX + (fx + B::HX);
-        R wL[L::NVAR], wR[L::NVAR];
-#pragma unroll
-        for (int v = 0; v < L::NVAR; v++) {
-            if (v == L::IR && vr == R(0)) {
-                // the upwind r flux (Sec. 3.1) vanishes for a body at rest in
-                // this direction, whatever the face values of r
-                wL[v] = wR[v] = R(0);
-                continue;
-            }
-            R s[6];
-#pragma unroll
-            for (int k = 0; k < 6; k++) s[k] = sW[v * B::N + bc + (k - 3) * SD];
-            const bool frac = (v >= L::IPHI && v < L::IPHI + NMAT - 1) || v == L::IR;
-            if constexpr (mix32<R, NMAT, SOLID>()) mix32_recon_face<R>(g, s, frac, wL[v], wR[v]);
-            else recon_face<R>(g, s, frac, wL[v], wR[v]);
-        }
-        R F[L::NF];
-        riemann<R, DIM, NMAT, SOLID, D>(g, wL, wR, vr, F);
-#pragma unroll
-        for (int k = 0; k < L::NF; k++) sF[k * B::MAXF + item] = F[k];
     }
+}
+
+// Fluxes of direction D, each face by the thread that holds its right state:
+// the record takes the place of the left state it was made from (no other
+// thread reads that).  No barrier.
+template <class R, int DIM, int NMAT, int SOLID, int V, int D>
+__device__ __forceinline__ void face_pass(const GridP &g, R *sQ, R vr, const R *lo)
+{
+    using L = Lay<DIM, NMAT, SOLID>;
+    using B = Box<DIM, V>;
+    using S = Sweep<DIM, V, D>;
+    const S p;
+    if (!p.own && !p.extra) return;
+    R *q = sQ + (p.own ? p.face : p.face + S::T * S::SF);
+    R wL[L::NVAR], F[L::NF];
+#pragma unroll
+    for (int v = 0; v < L::NVAR; v++) wL[v] = (v == L::IR && vr == R(0)) ? R(0) : q[v * B::MAXF];
+    riemann<R, DIM, NMAT, SOLID, D>(g, wL, lo, vr, F);
+#pragma unroll
+    for (int k = 0; k < L::NF; k++) q[k * B::MAXF] = F[k];
 }
 
 // Divergence and non-conservative terms of direction D for the thread's own
 // cell, from the face fluxes in sF (no barrier).
-template <class R, int DIM, int NMAT, int SOLID, int D>
+template <class R, int DIM, int NMAT, int SOLID, int V, int D>
 __device__ __forceinline__ void accum_pass(const GridP &g, const R *sW, const R *sF, bool own, int lx, int ly, int lz,
                                            Acc<R> *Dacc)
 {
     using L = Lay<DIM, NMAT, SOLID>;
-    using B = Box<DIM, (int)sizeof(R)>;
-    using TL = Tile<DIM, (int)sizeof(R)>;
+    using B = Box<DIM, V>;
+    using TL = Tile<DIM, V>;
     constexpr int EX = TL::TX + (D == 0), EY = TL::TY + (D == 1);
     if (own) {
         const int fl = (lz * EY + ly) * EX + lx;
@@ -1062,18 +1107,28 @@ __device__ __forceinline__ void accum_pass(const GridP &g, const R *sW, const R 
     }
 }
 
+// whether the body rests (read from L2 before the seeding launch is waited for)
+template <class R, int DIM>
+__device__ __forceinline__ bool ctl_rest(const Ctl *c, bool early)
+{
+    bool rest = true;
+#pragma unroll
+    for (int d = 0; d < DIM; d++) rest = rest && (early ? ctl_v_cg<R>(c, d) : ctl_v<R>(c, d)) == R(0);
+    return rest;
+}
+
 // One tile of one SSP-RK3 stage, executed by a whole CTA: (tbx, tby, tbz) is
 // the tile position in tile units, tile_id its index among the ntiles tiles of
 // the grid (partials slot; the last of them to finish runs the finalize).
-template <class R, int DIM, int NMAT, int SOLID, int STAGE>
+template <class R, int DIM, int NMAT, int SOLID, int STAGE, int V>
 __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, int tbx, int tby, int tbz,
                                            long long tile_id, long long ntiles)
 {
     using L = Lay<DIM, NMAT, SOLID>;
-    using B = Box<DIM, (int)sizeof(R)>;
-    using TL = Tile<DIM, (int)sizeof(R)>;
+    using B = Box<DIM, V>;
+    using TL = Tile<DIM, V>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using SM = StageSmem<R, DIM, NMAT, SOLID>;
+    using SM = StageSmem<R, DIM, NMAT, SOLID, V>;
     R *sW = reinterpret_cast<R *>(smem_raw);
     R *sF = sW + (size_t)L::NVAR * B::N;
     double *sred = reinterpret_cast<double *>(smem_raw + ((sizeof(R) * SM::floats + 7) & ~(size_t)7));
@@ -1089,7 +1144,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
     // (only the first wave: later tiles start after the seeding anyway, and
     // their loads keep the L1 hits of the halo shared with earlier tiles)
     const bool early = STAGE == 1 && tile_id < a.early &&
-                       !tile_touches_box<DIM, (int)sizeof(R)>(g, a.ctl, ox, oy, oz, a.next);
+                       !tile_touches_box<DIM, V>(g, a.ctl, ox, oy, oz, a.next);
     if (STAGE == 1 && a.early > 0 && !early) pdl_wait();
 
     // 1. primitives of the tile and its halo (the corner regions are unused);
@@ -1097,11 +1152,32 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
     const bool interior = ox >= B::HX && ox + TL::TX + B::HX <= g.n[0] &&
                           (DIM < 2 || (oy >= B::HY && oy + TL::TY + B::HY <= g.n[1])) &&
                           (DIM < 3 || (oz >= B::HZ && oz + TL::TZ + B::HZ <= g.n[2]));
-    for (int i = threadIdx.x; i < B::N; i += TL::THREADS) {
-        const int bx = i % B::BX, by = (i / B::BX) % B::BY, bz = i / (B::BX * B::BY);
-        const int lx = bx - B::HX, ly = by - B::HY, lz = bz - B::HZ;
-        const int outside = (lx < 0 || lx >= TL::TX) + (ly < 0 || ly >= TL::TY) + (lz < 0 || lz >= TL::TZ);
-        if (outside > 1) continue;
+    // without a fraction to reconstruct (one material, the body at rest) the
+    // outermost halo cells are read by nobody
+    const bool h2 = NMAT == 1 && ctl_rest<R, DIM>(a.ctl, early);
+    const int hw = h2 ? 2 : 3, px = TL::TX + 2 * hw;
+    const int n1 = px * TL::TY * TL::TZ, n2 = n1 + (DIM >= 2 ? 2 * hw * TL::TX * TL::TZ : 0),
+              n3 = n2 + (DIM >= 3 ? 2 * hw * TL::TX * TL::TY : 0);
+    for (int i = threadIdx.x; i < n3; i += TL::THREADS) {
+        // rows with their x halo, then the y halo's, then the z halo's
+        int lx, ly, lz;
+        if (i < n1) {
+            const int row = h2 ? i / (TL::TX + 4) : i / (TL::TX + 6);
+            lx = i - row * px - hw;
+            ly = row % TL::TY;
+            lz = row / TL::TY;
+        } else if (DIM < 3 || i < n2) {
+            const int k = i - n1, row = k / TL::TX, h = row / TL::TZ;
+            lx = k % TL::TX;
+            ly = h < hw ? h - hw : TL::TY + h - hw;
+            lz = row % TL::TZ;
+        } else {
+            const int k = i - n2, row = k / TL::TX, h = row / TL::TY;
+            lx = k % TL::TX;
+            ly = row % TL::TY;
+            lz = h < hw ? h - hw : TL::TZ + h - hw;
+        }
+        const int ib = ((lz + B::HZ) * B::BY + (ly + B::HY)) * B::BX + (lx + B::HX);
         bool fl[3] = {false, false, false};
         int gx = ox + lx, gy = DIM >= 2 ? oy + ly : 0, gz = DIM >= 3 ? oz + lz : 0;
         if (!interior) {
@@ -1130,7 +1206,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
                 if ((v_row(DIM, cc) == d) != (v_col(DIM, cc) == d)) w[L::IV + cc] = -w[L::IV + cc];
         }
 #pragma unroll
-        for (int v = 0; v < L::NVAR; v++) sW[v * B::N + i] = w[v];
+        for (int v = 0; v < L::NVAR; v++) sW[v * B::N + ib] = w[v];
     }
     __syncthreads();
 
@@ -1151,26 +1227,42 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
 #pragma unroll
     for (int v = 0; v < L::NVAR; v++) Dacc[v].zero();
 
-    if constexpr (SM::NSF == 2) {
-        // 2-D fluids: the faces of both directions, one barrier, both divergences
-        R *sF1 = sF + (size_t)L::NF * B::MAXF;
-        face_pass<R, DIM, NMAT, SOLID, 0>(g, sW, sF, vr[0]);
-        face_pass<R, DIM, NMAT, SOLID, 1>(g, sW, sF1, vr[1]);
+    if constexpr (DIM == 2 && SM::NSF == 2) {
+        // 2-D fluids: both directions between the same barriers
+        R *sQ = sF + (size_t)L::NF * B::MAXF;
+        R lo0[L::NVAR], lo1[L::NVAR];
+        slope_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, vr[0], lo0);
+        slope_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, vr[1], lo1);
         __syncthreads();
-        accum_pass<R, DIM, NMAT, SOLID, 0>(g, sW, sF, own, lx, ly, lz, Dacc);
-        accum_pass<R, DIM, NMAT, SOLID, 1>(g, sW, sF1, own, lx, ly, lz, Dacc);
+        face_pass<R, DIM, NMAT, SOLID, V, 0>(g, sF, vr[0], lo0);
+        face_pass<R, DIM, NMAT, SOLID, V, 1>(g, sQ, vr[1], lo1);
         __syncthreads();
+        accum_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, own, lx, ly, lz, Dacc);
+        accum_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, own, lx, ly, lz, Dacc);
     } else {
-#pragma unroll
-        for (int d = 0; d < DIM; d++) {
-            if (d == 0) face_pass<R, DIM, NMAT, SOLID, 0>(g, sW, sF, vr[0]);
-            if constexpr (DIM >= 2) if (d == 1) face_pass<R, DIM, NMAT, SOLID, 1>(g, sW, sF, vr[1]);
-            if constexpr (DIM >= 3) if (d == 2) face_pass<R, DIM, NMAT, SOLID, 2>(g, sW, sF, vr[2]);
+        R lo[L::NVAR];
+        slope_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, vr[0], lo);
+        __syncthreads();
+        face_pass<R, DIM, NMAT, SOLID, V, 0>(g, sF, vr[0], lo);
+        __syncthreads();
+        accum_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, own, lx, ly, lz, Dacc);
+        if constexpr (DIM >= 2) {
+            // the other face array, or this one once its divergence is formed
+            R *sQ = sF + (SM::NSF - 1) * (size_t)L::NF * B::MAXF;
+            if (SM::NSF == 1) __syncthreads();
+            slope_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, vr[1], lo);
             __syncthreads();
-            if (d == 0) accum_pass<R, DIM, NMAT, SOLID, 0>(g, sW, sF, own, lx, ly, lz, Dacc);
-            if constexpr (DIM >= 2) if (d == 1) accum_pass<R, DIM, NMAT, SOLID, 1>(g, sW, sF, own, lx, ly, lz, Dacc);
-            if constexpr (DIM >= 3) if (d == 2) accum_pass<R, DIM, NMAT, SOLID, 2>(g, sW, sF, own, lx, ly, lz, Dacc);
+            face_pass<R, DIM, NMAT, SOLID, V, 1>(g, sQ, vr[1], lo);
             __syncthreads();
+            accum_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, own, lx, ly, lz, Dacc);
+        }
+        if constexpr (DIM >= 3) {
+            if (SM::NSF == 1) __syncthreads();
+            slope_pass<R, DIM, NMAT, SOLID, V, 2>(g, sW, sF, vr[2], lo);
+            __syncthreads();
+            face_pass<R, DIM, NMAT, SOLID, V, 2>(g, sF, vr[2], lo);
+            __syncthreads();
+            accum_pass<R, DIM, NMAT, SOLID, V, 2>(g, sW, sF, own, lx, ly, lz, Dacc);
         }
     }
 
@@ -1303,18 +1395,20 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
     }
 }
 
-// Register bound: four CTAs per SM for the 2-D FP32 single-material fluid
-// (56 registers without spills; stage 3 would otherwise take 62 and three),
-// two for the other 2-D forms (which would otherwise take up to 138
-// registers and run one 9-warp CTA per SM).
-template <class R, int DIM, int NMAT, int SOLID>
-constexpr int stage_min_ctas()
+// Register bound of the 2-D forms: four CTAs per SM for the FP32
+// single-material fluid, three for the other FP32 forms (two for solids of
+// three materials, which would spill), two for the FP64 ones
+// (which would otherwise take up to 138 registers and run one 9-warp CTA per
+// SM); twice as many small tiles.
+template <class R, int DIM, int NMAT, int SOLID, int V>
+__host__ __device__ constexpr int stage_min_ctas()
 {
-    return DIM != 2 ? 1 : ((sizeof(R) == 4 && NMAT == 1 && SOLID == 0) ? 4 : 2);
+    return DIM != 2 ? 1
+                    : (sizeof(R) == 4 ? (NMAT == 1 && SOLID == 0 ? 4 : (NMAT == 3 && SOLID ? 2 : 3)) : 2) * (V ? 2 : 1);
 }
 
-template <class R, int DIM, int NMAT, int SOLID, int STAGE>
-__global__ void __launch_bounds__(Tile<DIM, (int)sizeof(R)>::THREADS, stage_min_ctas<R, DIM, NMAT, SOLID>())
+template <class R, int DIM, int NMAT, int SOLID, int STAGE, int V>
+__global__ void __launch_bounds__(Tile<DIM, V>::THREADS, stage_min_ctas<R, DIM, NMAT, SOLID, V>())
     k_stage(StageArgs a, GridP g)
 {
     // stage 1 after the seeding waits inside stage_tile (early tiles late)
@@ -1322,7 +1416,7 @@ __global__ void __launch_bounds__(Tile<DIM, (int)sizeof(R)>::THREADS, stage_min_
     else pdl_enter();
     const long long tile = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
     const long long nt = (long long)gridDim.x * gridDim.y * gridDim.z;
-    stage_tile<R, DIM, NMAT, SOLID, STAGE>(g, a, blockIdx.x, blockIdx.y, blockIdx.z, tile, nt);
+    stage_tile<R, DIM, NMAT, SOLID, STAGE, V>(g, a, blockIdx.x, blockIdx.y, blockIdx.z, tile, nt);
 }
 
 // ------------------------------------------------------------------ CFL
