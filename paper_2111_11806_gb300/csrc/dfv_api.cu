@@ -329,6 +329,7 @@ dfv_status launch_stage(dfv_grid *g, int s, const void *in, const void *un, void
         a.Gam = g->g.mc_f[0].Gam;
         a.invGam = g->g.mc_f[0].invGam;
         a.pref0 = g->g.mc_f[0].pref0;
+        a.wide = (unsigned long long)g->g.pitch * 5u * 4u >= (1ull << 32);
         DFV_CU(g, dfv::gasw_stage(s, a, g->gas_grid, g->stream), "k_gasw_stage");
         return DFV_OK;
     }

@@ -223,6 +223,7 @@ dfv_status phase(dfv_batch *b, int ph, const void *in, const void *un, void *out
         ga.Gam = m.Gam;
         ga.invGam = m.invGam;
         ga.pref0 = m.pref0;
+        ga.wide = (unsigned long long)b->plan.elems * 4u >= (1ull << 32);
         // CTAs of independent warps, one warp per item at a time
         const long long n = (b->plan.gas_nitems + dfv::GaswT::WARPS - 1) / dfv::GaswT::WARPS;
         const long long persistent = (long long)b->sm_count * std::min(std::max(b->ctas_per_sm, 1), b->gas_max_ctas);

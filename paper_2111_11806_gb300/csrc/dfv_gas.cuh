@@ -54,20 +54,28 @@ __device__ __forceinline__ float2 gas_sub2(float2 p, float2 q)
     return __ffma2_rn(q, make_float2(-1.f, -1.f), p);
 }
 
-// van Leer limited slope of a cell from its backward and forward differences
-__device__ __forceinline__ float gas_vanleer(float a, float b)
+// half the van Leer slope 2ab/(a+b) of a cell from its backward and forward differences
+__device__ __forceinline__ float gas_half_slope(float a, float b)
 {
     const float ab = __fmul_rn(a, b);
-    return ab <= 0.f ? 0.f : __fmul_rn(ab + ab, gas_rcp(a + b));
+    return ab <= 0.f ? 0.f : __fmul_rn(ab, gas_rcp(__fadd_rn(a, b)));
 }
 
 // the same for two pairs of differences at once
-__device__ __forceinline__ float2 gas_vanleer2(float2 a, float2 b)
+__device__ __forceinline__ float2 gas_half_slope2(float2 a, float2 b)
 {
     const float2 ab = __fmul2_rn(a, b);
     const float2 s = __fadd2_rn(a, b);
-    const float2 q = __fmul2_rn(__fadd2_rn(ab, ab), gas_f2(gas_rcp(s.x), gas_rcp(s.y)));
+    const float2 q = __fmul2_rn(ab, gas_f2(gas_rcp(s.x), gas_rcp(s.y)));
     return gas_f2(ab.x <= 0.f ? 0.f : q.x, ab.y <= 0.f ? 0.f : q.y);
+}
+
+// approximate reciprocal square root: one instruction
+__device__ __forceinline__ float gas_rsqrt(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // Conserved (rho, rho u, rho v, rho E) -> primitive (rho, u, v, p) of the gas
@@ -86,57 +94,63 @@ __device__ __forceinline__ void gas_prim(const A &a, float r, float mu, float mv
     w[3] = fmaf(a.Gam, E - ke, a.pref0);
 }
 
+// The wave speeds of a face between (rL, unL, pL) and (rR, unR, pR): Davis'
+// S_L, S_R, the contact S*, and of each side d = S_K - u_K and rho d.  The
+// sound speed is k/sqrt(k rho) with k = rho c^2 = (Gam + 1) p - p_ref: one
+// special function a side.  The contact numerator's products are rounded one
+// by one (a wall face between mirror-image states gets S* = 0 exactly).
+template <class A>
+__device__ __forceinline__ void gas_waves(const A &a, float rL, float unL, float pL, float rR, float unR, float pR,
+                                          float &SL, float &SR, float &Ss, float2 &d2, float2 &m2)
+{
+    const float2 r2 = gas_f2(rL, rR), un2 = gas_f2(unL, unR);
+    const float2 k2 = __ffma2_rn(gas_f2(a.Gam, a.Gam), gas_f2(pL, pR), gas_sub2(gas_f2(pL, pR), gas_f2(a.pref0, a.pref0)));
+    const float2 x2 = __fmul2_rn(k2, r2);
+    const float2 c2 = __fmul2_rn(k2, gas_f2(gas_rsqrt(x2.x), gas_rsqrt(x2.y)));
+    const float2 lo = gas_sub2(un2, c2), hi = __fadd2_rn(un2, c2);
+    SL = fminf(lo.x, lo.y);
+    SR = fmaxf(hi.x, hi.y);
+    d2 = gas_sub2(gas_f2(SL, SR), un2);
+    m2 = __fmul2_rn(r2, d2);
+    const float2 mm = __fmul2_rn(m2, un2);
+    const float num = __fadd_rn(__fadd_rn(__fadd_rn(pR, -pL), mm.x), -mm.y);
+    Ss = __fmul_rn(num, gas_rcp(__fadd_rn(m2.x, -m2.y)));
+}
+
 // HLLC flux of the gas across a face (Sec. 3.1: Toro's HLLC with Davis wave
 // speeds), normal velocity un, tangential ut; F = (rho, normal momentum,
-// tangential momentum, energy).  The left and right states' sound speeds,
-// wave-speed bounds and contact-speed terms are formed pairwise.
+// tangential momentum, energy).  In the star regions the flux of the star
+// state itself, which the jump conditions make F_K + S_K (U*_K - U_K): mass
+// M = rho d S*/(S_K - S*), p* = p + rho d (S* - u_K), energy
+// S* (E* + p*) with E* = (d E - p u_K + p* S*)/(S_K - S*).
 template <class A>
 __device__ __forceinline__ void gas_hllc(const A &a, float rL, float unL, float utL, float pL, float rR,
                                          float unR, float utR, float pR, float F[4])
 {
-    const float2 r2 = gas_f2(rL, rR), un2 = gas_f2(unL, unR), p2 = gas_f2(pL, pR);
-    const float2 ir2 = gas_f2(gas_rcp(rL), gas_rcp(rR));
-    const float2 cc = __fmul2_rn(__ffma2_rn(gas_f2(a.Gam, a.Gam), p2, gas_sub2(p2, gas_f2(a.pref0, a.pref0))), ir2);
-    const float2 c2 = gas_f2(sqrtf(cc.x), sqrtf(cc.y));
-    const float2 lo = gas_sub2(un2, c2), hi = __fadd2_rn(un2, c2);
-    const float SL = fminf(lo.x, lo.y);
-    const float SR = fmaxf(hi.x, hi.y);
-    // contact speed, the numerator's products rounded one by one (a wall face
-    // between mirror-image states gets S* = 0 exactly)
-    const float2 d2 = gas_sub2(gas_f2(SL, SR), un2);                  // S_K - u_K
-    const float2 mm = __fmul2_rn(__fmul2_rn(r2, un2), d2);
-    const float num = __fadd_rn(__fadd_rn(pR - pL, mm.x), -mm.y);
-    const float Ss = __fmul_rn(num, gas_rcp(fmaf(rL, d2.x, -__fmul_rn(rR, d2.y))));
+    float SL, SR, Ss;
+    float2 d2, m2;
+    gas_waves(a, rL, unL, pL, rR, unR, pR, SL, SR, Ss, d2, m2);
     // regions: left of S_L, left star, right star, right of S_R
     const int region = SL >= 0.f ? 0 : (Ss >= 0.f ? 1 : (SR > 0.f ? 2 : 3));
     const bool left = region <= 1;
     const float r = left ? rL : rR, un = left ? unL : unR, ut = left ? utL : utR, p = left ? pL : pR;
-    const float S = left ? SL : SR;
-    const float hr = __fmul_rn(0.5f, r);
-    const float2 h = __fmul2_rn(gas_f2(hr, hr), gas_f2(ut, un));       // (hr ut, hr un)
-    const float E = fmaf(h.x, ut, fmaf(p - a.pref0, a.invGam, __fmul_rn(h.y, un)));
-    const float m = __fmul_rn(r, un);
-    // physical flux of the upwind side: (rho, normal momentum), (tangential momentum, energy)
-    float2 Fa = gas_f2(m, fmaf(m, un, p));
-    float2 Fb = __fmul2_rn(gas_f2(m, E + p), gas_f2(ut, un));
-    const bool star = region == 1 || region == 2;
-    if (star) {
-        // star state U*_K = rho_K chi [1, S*, u_t, E_K/rho_K + (S* - u_K)(S* + p_K/(rho_K (S_K - u_K)))],
-        // chi = (S_K - u_K)/(S_K - S*); with iD = 1/(S_K - S*) its energy is
-        // chi E_K + (S* - u_K)(rho_K chi S* + p_K iD): one reciprocal
-        const float2 dd = gas_sub2(gas_f2(S, S), gas_f2(Ss, un));   // (S_K - S*, S_K - u_K)
+    const float S = left ? SL : SR, d = left ? d2.x : d2.y, m = left ? m2.x : m2.y;
+    const float E = fmaf(__fmul_rn(0.5f, r), fmaf(ut, ut, __fmul_rn(un, un)), __fmul_rn(__fadd_rn(p, -a.pref0), a.invGam));
+    float us = un, ps = p, cS = un, FE = __fmul_rn(__fadd_rn(E, p), un);
+    if (region == 1 || region == 2) {
+        const float2 dd = gas_sub2(gas_f2(S, Ss), gas_f2(Ss, un));   // (S_K - S*, S* - u_K)
         const float iD = gas_rcp(dd.x);
-        const float chi = __fmul_rn(dd.y, iD);
-        const float rs = __fmul_rn(r, chi);
-        const float Es = fmaf(chi, E, __fmul_rn(Ss - un, fmaf(rs, Ss, __fmul_rn(p, iD))));
-        // F + S_K (U*_K - U_K)
-        Fa = __ffma2_rn(gas_f2(S, S), gas_f2(rs - r, fmaf(rs, Ss, -m)), Fa);
-        Fb = __ffma2_rn(gas_f2(S, S), gas_f2(fmaf(rs, ut, -__fmul_rn(r, ut)), Es - E), Fb);
+        us = Ss;
+        cS = __fmul_rn(__fmul_rn(d, iD), Ss);
+        ps = fmaf(m, dd.y, p);
+        const float Es = __fmul_rn(fmaf(d, E, fmaf(ps, Ss, -__fmul_rn(p, un))), iD);
+        FE = __fmul_rn(__fadd_rn(Es, ps), Ss);
     }
-    F[0] = Fa.x;
-    F[1] = Fa.y;
-    F[2] = Fb.x;
-    F[3] = Fb.y;
+    const float M = __fmul_rn(r, cS);
+    F[0] = M;
+    F[1] = fmaf(M, us, ps);
+    F[2] = __fmul_rn(M, ut);
+    F[3] = FE;
 }
 
 // Whether a 2-D grid can take the gas stage kernel: FP32, one ideal or

@@ -16,7 +16,7 @@
 //   3. faces: every thread the HLLC fluxes of its cell's left x face, bottom
 //      y face and top z face; the bottom z face and the top z-face value of
 //      plane z were carried in shared memory from the previous plane;
-//   4. update of plane z: divergence with a compensated (TwoSum) sum, rigid
+//   4. update of plane z: divergence, rigid
 //      mask, RK combination; in stage 3 the CFL maximum and the rigid box.
 // Each primitive is converted once per chunk and each slope computed once;
 // the arithmetic per face is that of the 2-D gas kernel (dfv_gas.cuh) with
@@ -133,42 +133,32 @@ struct Gas3Args {
 __device__ __forceinline__ void gas_hllc3(const Gas3Args &a, const float L[5], const float R[5], float F[5])
 {
     // L, R: (rho, un, ut1, ut2, p)
-    const float rL = L[0], unL = L[1], pL = L[4], rR = R[0], unR = R[1], pR = R[4];
-    const float irL = __fdividef(1.f, rL), irR = __fdividef(1.f, rR);
-    const float cL = sqrtf((a.Gam * pL + (pL - a.pref0)) * irL);
-    const float cR = sqrtf((a.Gam * pR + (pR - a.pref0)) * irR);
-    const float SL = fminf(unL - cL, unR - cR);
-    const float SR = fmaxf(unL + cL, unR + cR);
-    // contact speed, the numerator's products rounded one by one (a wall face
-    // between mirror-image states gets S* = 0 exactly)
-    const float num = __fadd_rn(__fadd_rn(pR - pL, __fmul_rn(__fmul_rn(rL, unL), SL - unL)),
-                                -__fmul_rn(__fmul_rn(rR, unR), SR - unR));
-    const float Ss = __fdividef(num, rL * (SL - unL) - rR * (SR - unR));
+    float SL, SR, Ss;
+    float2 d2, m2;
+    gas_waves(a, L[0], L[1], L[4], R[0], R[1], R[4], SL, SR, Ss, d2, m2);
     const int region = SL >= 0.f ? 0 : (Ss >= 0.f ? 1 : (SR > 0.f ? 2 : 3));
-    const bool left = region <= 1, star = region == 1 || region == 2;
+    const bool left = region <= 1;
     // the upwind side's state, element by element (a pointer choice would
     // put both arrays in local memory)
     const float r = left ? L[0] : R[0], un = left ? L[1] : R[1], u1 = left ? L[2] : R[2];
     const float u2 = left ? L[3] : R[3], p = left ? L[4] : R[4];
-    const float S = left ? SL : SR;
-    const float E = (p - a.pref0) * a.invGam + 0.5f * r * un * un + 0.5f * r * u1 * u1 + 0.5f * r * u2 * u2;
-    const float m = r * un;
-    float Fr = m, Fn = m * un + p, F1 = m * u1, F2 = m * u2, FE = (E + p) * un;
-    if (star) {
-        const float iD = __fdividef(1.f, S - Ss);
-        const float chi = (S - un) * iD;
-        const float rs = r * chi;
-        const float Es = chi * E + (Ss - un) * (rs * Ss + p * iD);
-        Fr += S * (rs - r);
-        Fn += S * (rs * Ss - m);
-        F1 += S * (rs * u1 - r * u1);
-        F2 += S * (rs * u2 - r * u2);
-        FE += S * (Es - E);
+    const float S = left ? SL : SR, d = left ? d2.x : d2.y, m = left ? m2.x : m2.y;
+    const float E = fmaf(0.5f * r, fmaf(u2, u2, fmaf(u1, u1, un * un)), (p - a.pref0) * a.invGam);
+    float us = un, ps = p, cS = un, FE = (E + p) * un;
+    if (region == 1 || region == 2) {
+        // the star state's own flux (gas_hllc)
+        const float2 dd = gas_sub2(gas_f2(S, Ss), gas_f2(Ss, un));   // (S_K - S*, S* - u_K)
+        const float iD = gas_rcp(dd.x);
+        us = Ss;
+        cS = __fmul_rn(__fmul_rn(d, iD), Ss);
+        ps = fmaf(m, dd.y, p);
+        FE = (fmaf(d, E, fmaf(ps, Ss, -__fmul_rn(p, un))) * iD + ps) * Ss;
     }
-    F[0] = Fr;
-    F[1] = Fn;
-    F[2] = F1;
-    F[3] = F2;
+    const float M = __fmul_rn(r, cS);
+    F[0] = M;
+    F[1] = fmaf(M, us, ps);
+    F[2] = M * u1;
+    F[3] = M * u2;
     F[4] = FE;
 }
 
@@ -180,6 +170,11 @@ struct Gas3Plane {
     unsigned flip;
     int gz;           // plane read
     unsigned phase;   // tensor copies issued so far (TMA path)
+    // of each cell that the thread converts: its place in the fetch slot's box
+    // (low half) and in a ring plane (high half), the same for every plane, and
+    // its x and y mirror flags (2 bits a cell; TMA path)
+    unsigned at[Gas3T::K];
+    unsigned mirror;
 };
 
 __device__ __forceinline__ void gas3_cp4(float *dst, const float *src)
@@ -290,8 +285,7 @@ __device__ __forceinline__ void gas3_prim(const Gas3Args &a, const float q[5], u
 // Convert the fetched plane into ring slot `slot`; false when a tensor copy
 // never completed (bounded wait).
 template <bool TMA>
-__device__ __forceinline__ bool gas3_commit(const Gas3Args &a, Gas3Plane &f, Gas3Smem &S, int slot, int ox, int oy,
-                                            bool interior)
+__device__ __forceinline__ bool gas3_commit(const Gas3Args &a, Gas3Plane &f, Gas3Smem &S, int slot)
 {
     using T = Gas3T;
     if constexpr (TMA) {
@@ -301,38 +295,55 @@ __device__ __forceinline__ bool gas3_commit(const Gas3Args &a, Gas3Plane &f, Gas
     } else {
         asm volatile("cp.async.wait_group 0;" ::: "memory");   // this thread's copies have landed
     }
+    float4 *pa = &S.pa[slot][0][0];
+    float *pp = &S.pp[slot][0][0];
 #pragma unroll
     for (int k = 0; k < T::K; k++) {
-        const int q = threadIdx.x + k * T::THREADS;
-        if (q >= T::NCONV) continue;
-        int lx, ly;
-        gas3_cell(q, lx, ly);
+        if (threadIdx.x + k * T::THREADS >= T::NCONV) continue;
+        const unsigned at = f.at[k] & 0xffffu, to = f.at[k] >> 16;
         float c5[5], w[5];
         unsigned flip;
         if constexpr (TMA) {
-            // the cell's place in the box: the halo beyond a side is the
-            // nearest cell or the mirror image (flip), clamped into the box
-            // (cells far outside a small grid feed only faces outside it)
-            bool fx = false, fy = false;
-            int gx = ox + lx, gy = oy + ly;
-            if (!interior) {
-                gx = gas3_map(gx, a.n0, a.wall[0][0], a.wall[0][1], &fx);
-                gy = gas3_map(gy, a.n1, a.wall[1][0], a.wall[1][1], &fy);
-            }
-            const int bx = min(max(gx - (ox - 4), 0), T::BX - 1), by = min(max(gy - (oy - T::H), 0), T::BY - 1);
 #pragma unroll
-            for (int v = 0; v < 5; v++) c5[v] = S.xfer[(v * T::BY + by) * T::BX + bx];
-            flip = (fx ? 1u : 0u) | (fy ? 2u : 0u) | f.flip;
+            for (int v = 0; v < 5; v++) c5[v] = S.xfer[v * T::BY * T::BX + at];
+            flip = (f.mirror >> (2 * k) & 3u) | f.flip;
         } else {
 #pragma unroll
             for (int v = 0; v < 5; v++) c5[v] = S.xfer[(k * 5 + v) * T::THREADS + threadIdx.x];
             flip = (f.flip >> (3 * k)) & 7u;
         }
         gas3_prim(a, c5, flip, w);
-        S.pa[slot][ly + T::H][lx + T::H] = make_float4(w[0], w[1], w[2], w[3]);
-        S.pp[slot][ly + T::H][lx + T::H] = w[4];
+        pa[to] = make_float4(w[0], w[1], w[2], w[3]);
+        pp[to] = w[4];
     }
     return true;
+}
+
+// The places of the thread's cells (Gas3Plane::at, mirror).
+__device__ __forceinline__ void gas3_places(const Gas3Args &a, Gas3Plane &f, int ox, int oy, bool interior)
+{
+    using T = Gas3T;
+    f.mirror = 0u;
+#pragma unroll
+    for (int k = 0; k < T::K; k++) {
+        const int q = threadIdx.x + k * T::THREADS;
+        f.at[k] = 0u;
+        if (q >= T::NCONV) continue;
+        int lx, ly;
+        gas3_cell(q, lx, ly);
+        // the cell's place in the box: the halo beyond a side is the
+        // nearest cell or the mirror image (flip), clamped into the box
+        // (cells far outside a small grid feed only faces outside it)
+        bool fx = false, fy = false;
+        int gx = ox + lx, gy = oy + ly;
+        if (!interior) {
+            gx = gas3_map(gx, a.n0, a.wall[0][0], a.wall[0][1], &fx);
+            gy = gas3_map(gy, a.n1, a.wall[1][0], a.wall[1][1], &fy);
+        }
+        const int bx = min(max(gx - (ox - 4), 0), T::BX - 1), by = min(max(gy - (oy - T::H), 0), T::BY - 1);
+        f.at[k] = (unsigned)(by * T::BX + bx) | (unsigned)((ly + T::H) * (T::PX + 1) + lx + T::H) << 16;
+        f.mirror |= ((fx ? 1u : 0u) | (fy ? 2u : 0u)) << (2 * k);
+    }
 }
 
 // primitives of the column's own cell in a ring slot
@@ -365,9 +376,9 @@ __device__ __forceinline__ void gas3_slope(const float m[5], const float c[5], c
 {
 #pragma unroll
     for (int v = 0; v < 5; v++) {
-        const float s = gas_vanleer(c[v] - m[v], p[v] - c[v]);
-        lo[v] = c[v] - 0.5f * s;
-        hi[v] = c[v] + 0.5f * s;
+        const float h = gas_half_slope(c[v] - m[v], p[v] - c[v]);
+        lo[v] = c[v] - h;
+        hi[v] = c[v] + h;
     }
 }
 
@@ -443,13 +454,14 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
     // the column's planes z0-2, z0-1 for its first z slopes
     Gas3Plane fp;
     fp.phase = 0u;
+    gas3_places(a, fp, ox, oy, interior);
     gas3_fetch<TMA>(a, &map, S, fp, ox, oy, z0, interior);
-    if (__syncthreads_or(!gas3_commit<TMA>(a, fp, S, z0 % T::RING, ox, oy, interior))) {
+    if (__syncthreads_or(!gas3_commit<TMA>(a, fp, S, z0 % T::RING))) {
         gas3_fail(a, S, fp);
         return;
     }
     gas3_fetch<TMA>(a, &map, S, fp, ox, oy, z0 + 1, interior);
-    if (__syncthreads_or(!gas3_commit<TMA>(a, fp, S, (z0 + 1) % T::RING, ox, oy, interior))) {
+    if (__syncthreads_or(!gas3_commit<TMA>(a, fp, S, (z0 + 1) % T::RING))) {
         gas3_fail(a, S, fp);
         return;
     }
@@ -481,7 +493,7 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
         // 1. plane z+2 into the ring (its slot held plane z-1, whose last
         // readers are behind the previous plane's barriers); then, with the
         // fetch slot read by every thread, plane z+3 fetched into it
-        if (__syncthreads_or(!gas3_commit<TMA>(a, fp, S, s2, ox, oy, interior))) {
+        if (__syncthreads_or(!gas3_commit<TMA>(a, fp, S, s2))) {
             gas3_fail(a, S, fp);
             return;
         }
@@ -489,11 +501,11 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
         if (col && z + 1 < z1) {
             // the cell's stage input and U^n at the next plane into L1 (read
             // at that plane's update; no register or shared slot holds them)
-            const long long cn = gx + (long long)a.n0 * (gy + (long long)a.n1 * (z + 1));
+            const unsigned cn = gx + (unsigned)a.n0 * (gy + (unsigned)a.n1 * (z + 1));
 #pragma unroll
             for (int v = 0; v < 6; v++) {
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(a.in + cn + v * a.pitch));
-                if (STAGE > 1) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.un + cn + v * a.pitch));
+                asm volatile("prefetch.global.L1 [%0];" ::"l"((a.in + v * a.pitch) + cn));
+                if (STAGE > 1) asm volatile("prefetch.global.L1 [%0];" ::"l"((a.un + v * a.pitch) + cn));
             }
         }
 
@@ -609,13 +621,14 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
 
         // 4. update of plane z: the cell's stage input and step-start values
         // (loaded here, not held through the faces: three CTAs fit an SM)
-        const long long c = gx + (long long)a.n0 * (gy + (long long)a.n1 * z);
+        // (a 32-bit index from each plane's address: cells are fewer than 2^32)
+        const unsigned c = gx + (unsigned)a.n0 * (gy + (unsigned)a.n1 * z);
         if (col) {
             float cin[6], cun[6];
 #pragma unroll
             for (int v = 0; v < 6; v++) {
-                cin[v] = a.in[c + v * a.pitch];
-                cun[v] = a.un[c + v * a.pitch];
+                cin[v] = (a.in + v * a.pitch)[c];
+                cun[v] = (a.un + v * a.pitch)[c];
             }
             const float4 e4 = S.fxa[cj][ci + 1], n4 = S.fya[cj + 1][ci];
             const float Fxr[5] = {e4.x, e4.y, e4.z, e4.w, S.fxe[cj][ci + 1]};
@@ -624,22 +637,15 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
             float o[6];
 #pragma unroll
             for (int v = 0; v < 5; v++) {
-                Acc<float> D;
-                D.set((Fxr[v] - Fxl[v]) * a.idx);
-                D.add((Fyr[v] - Fyl[v]) * a.idy);
-                D.add((Fzhi[v] - S.zcarry[5 + v][tid]) * a.idz);
-                o[v] = masked ? cun[v] : rk_combine<float>(STAGE, cun[v], cin[v], D, dt, ca, cb);
+                const float D = fmaf(Fzhi[v] - S.zcarry[5 + v][tid], a.idz,
+                                     fmaf(Fyr[v] - Fyl[v], a.idy, (Fxr[v] - Fxl[v]) * a.idx));
+                const float y = fmaf(-dt, D, cin[v]);
+                o[v] = masked ? cun[v] : (STAGE == 1 ? y : fmaf(cb, y, __fmul_rn(ca, cun[v])));
             }
-            {
-                // r: no flux without a moving body
-                Acc<float> D;
-                D.set(0.f);
-                D.add(0.f);
-                D.add(0.f);
-                o[5] = rk_combine<float>(STAGE, cun[5], cin[5], D, dt, ca, cb);
-            }
+            // r: no flux without a moving body
+            o[5] = STAGE == 1 ? cin[5] : fmaf(cb, cin[5], __fmul_rn(ca, cun[5]));
 #pragma unroll
-            for (int v = 0; v < 6; v++) a.out[c + v * a.pitch] = o[v];
+            for (int v = 0; v < 6; v++) (a.out + v * a.pitch)[c] = o[v];
             if (!(o[0] > 0.f) || !(o[4] == o[4])) atomicOr(&a.ctl->err, (unsigned)ERR_STATE);
             if (STAGE == 3) {
                 if (o[5] > 0.5f) {

@@ -36,7 +36,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 int gasw_max_ctas_per_sm()
 {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gasw_stage<3>, GaswT::THREADS, 0) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gasw_stage<3, unsigned>, GaswT::THREADS, 0) != cudaSuccess) {
         (void)cudaGetLastError();
         return 1;
     }
@@ -46,9 +46,14 @@ int gasw_max_ctas_per_sm()
 cudaError_t gasw_stage(int stage, const GaswArgs &a, int grid, cudaStream_t st)
 {
     const dim3 g(grid < 1 ? 1 : grid), b(GaswT::THREADS);
-    if (stage == 1) return launch_pdl(k_gasw_stage<1>, g, b, 0, st, a);
-    if (stage == 2) return launch_pdl(k_gasw_stage<2>, g, b, 0, st, a);
-    return launch_pdl(k_gasw_stage<3>, g, b, 0, st, a);
+    if (a.wide) {
+        if (stage == 1) return launch_pdl(k_gasw_stage<1, unsigned long long>, g, b, 0, st, a);
+        if (stage == 2) return launch_pdl(k_gasw_stage<2, unsigned long long>, g, b, 0, st, a);
+        return launch_pdl(k_gasw_stage<3, unsigned long long>, g, b, 0, st, a);
+    }
+    if (stage == 1) return launch_pdl(k_gasw_stage<1, unsigned>, g, b, 0, st, a);
+    if (stage == 2) return launch_pdl(k_gasw_stage<2, unsigned>, g, b, 0, st, a);
+    return launch_pdl(k_gasw_stage<3, unsigned>, g, b, 0, st, a);
 }
 
 int gasw_rows(long long cells)

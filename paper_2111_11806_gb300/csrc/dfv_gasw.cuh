@@ -16,7 +16,7 @@
 // Per row j: the van Leer slope of row j+1 in y gives the y face j+1/2
 // (HLLC); the slope of row j in x (the neighbours' primitives by warp
 // shuffle) gives each lane the flux of its left x face, and its right one by
-// a shuffle from the next lane; then the compensated (TwoSum) divergence, the
+// a shuffle from the next lane; then the divergence, the
 // rigid mask and the RK combination of the owned cells, and in stage 3 the
 // CFL maximum and the box of the new rigid cells.  Each cell of a strip is
 // converted and given its slopes once (plus four rows and two rows of y
@@ -49,6 +49,7 @@ struct GaswArgs {
     const float *un;       // U^n
     float *out;            // stage output (U^n itself in stage 3)
     float Gam, invGam, pref0;
+    int wide;              // the planes of all instances take 4 GiB or more: 64-bit offsets
 };
 
 // Cell index of halo cell g of a line of n cells: the nearest cell beyond a
@@ -67,13 +68,24 @@ __device__ __forceinline__ int gasw_map(int g, int n, int wall0, int wall1, bool
     return g < 0 ? 0 : (g > n - 1 ? n - 1 : g);
 }
 
-// rho, rho u, rho v, rho E of one cell (planes P apart)
-__device__ __forceinline__ void gasw_load4(const float *p, long long P, float c[4])
+// Cells are addressed by byte offsets from the kernel's three state pointers, O
+// = unsigned (below 4 GiB) or unsigned long long: a 32-bit offset from an
+// address that all threads share is one operand of a load, where 64-bit
+// pointers take two or three instructions for each of the 19 accesses of a row.
+template <class O>
+__device__ __forceinline__ float gasw_ld(const float *p, O off)
 {
-    c[0] = __ldg(p);
-    c[1] = __ldg(p + P);
-    c[2] = __ldg(p + 2 * P);
-    c[3] = __ldg(p + 3 * P);
+    return __ldg(reinterpret_cast<const float *>(reinterpret_cast<const char *>(p) + off));
+}
+
+// rho, rho u, rho v, rho E of one cell (planes P bytes apart)
+template <class O>
+__device__ __forceinline__ void gasw_load4(const float *p, O off, O P, float c[4])
+{
+    c[0] = gasw_ld<O>(p, off);
+    c[1] = gasw_ld<O>(p, off + P);
+    c[2] = gasw_ld<O>(p, off + 2 * P);
+    c[3] = gasw_ld<O>(p, off + 3 * P);
 }
 
 // primitives of a loaded cell, the velocity mirrored across a reflective side
@@ -96,10 +108,9 @@ __device__ __forceinline__ float4 gasw_cat(const float2 &l, const float2 &h) { r
 __device__ __forceinline__ void gasw_faces_d(const float4 &c, const float4 &db, const float4 &df, float4 &lo,
                                              float4 &hi)
 {
-    const float2 s0 = gas_vanleer2(gasw_lo(db), gasw_lo(df)), s1 = gas_vanleer2(gasw_hi(db), gasw_hi(df));
-    const float2 mh = make_float2(-0.5f, -0.5f), ph = make_float2(0.5f, 0.5f);
-    lo = gasw_cat(__ffma2_rn(mh, s0, gasw_lo(c)), __ffma2_rn(mh, s1, gasw_hi(c)));
-    hi = gasw_cat(__ffma2_rn(ph, s0, gasw_lo(c)), __ffma2_rn(ph, s1, gasw_hi(c)));
+    const float2 h0 = gas_half_slope2(gasw_lo(db), gasw_lo(df)), h1 = gas_half_slope2(gasw_hi(db), gasw_hi(df));
+    lo = gasw_cat(gas_sub2(gasw_lo(c), h0), gas_sub2(gasw_hi(c), h1));
+    hi = gasw_cat(__fadd2_rn(gasw_lo(c), h0), __fadd2_rn(gasw_hi(c), h1));
 }
 
 __device__ __forceinline__ float4 gasw_sub(const float4 &p, const float4 &q)
@@ -140,20 +151,16 @@ __device__ __forceinline__ float4 gasw_shfl_down(const float4 &v)
                        __shfl_down_sync(0xffffffffu, v.z, 1), __shfl_down_sync(0xffffffffu, v.w, 1));
 }
 
-// two conserved variables of an owned cell: flux divergence (the x and y
-// terms summed by TwoSum, the error kept as the low part), rigid mask, RK
-// combination out = ca un + cb (in - dt (hi + lo)), the low part first
+// two conserved variables of an owned cell: flux divergence, rigid mask, RK
+// combination out = ca un + cb (in - dt D).  D rounds one product and, fused,
+// the sum (the two products and their compensated sum before it rounded one
+// more and took eight more instructions; the errors of the result agree).
 template <int STAGE>
 __device__ __forceinline__ float2 gasw_update2(float2 unv, float2 inv, float2 fxl, float2 fxr, float2 fyl, float2 fyr,
                                               float2 idx, float2 idy, float2 mdt, float2 ca, float2 cb, bool masked)
 {
-    const float2 div = __fmul2_rn(gas_sub2(fxr, fxl), idx);
-    const float2 dvy = __fmul2_rn(gas_sub2(fyr, fyl), idy);
-    const float2 hi = __fadd2_rn(div, dvy);
-    const float2 bp = gas_sub2(hi, div);
-    const float2 err = __fadd2_rn(gas_sub2(div, gas_sub2(hi, bp)), gas_sub2(dvy, bp));
-    const float2 lo = __fadd2_rn(make_float2(0.f, 0.f), err);
-    const float2 y = __ffma2_rn(mdt, hi, __ffma2_rn(mdt, lo, inv));
+    const float2 D = __ffma2_rn(gas_sub2(fyr, fyl), idy, __fmul2_rn(gas_sub2(fxr, fxl), idx));
+    const float2 y = __ffma2_rn(mdt, D, inv);
     if (masked) return unv;
     return STAGE == 1 ? y : __ffma2_rn(cb, y, __fmul2_rn(ca, unv));
 }
@@ -166,7 +173,7 @@ __device__ __forceinline__ long long gasw_take(unsigned int *queue, int lane)
     return (long long)__shfl_sync(0xffffffffu, v, 0);
 }
 
-template <int STAGE>
+template <int STAGE, class O>
 __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, int tile, int lane, float ca,
                                           float cb)
 {
@@ -179,10 +186,7 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
     bool fx;
     const int cx = gasw_map(gx, n0, I.wall_x0, I.wall_x1, fx);
     const bool owned = lane >= T::H && lane < 32 - T::H && gx < n0;   // then cx == gx
-    const long long P = I.pitch, n0l = n0;
-    const float *in = a.in + I.off + cx;
-    const float *unp = a.un + I.off + cx;
-    float *out = a.out + I.off + cx;
+    const O P = (O)I.pitch * 4u, row = (O)n0 * 4u, base = ((O)I.off + (O)cx) * 4u;
     Ctl *ctl = I.ctl;
     const float dt = ctl_dt<float>(ctl);
     const float idx = I.idx, idy = I.idy;
@@ -194,7 +198,7 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
         float c[4][4];
         bool f[4];
 #pragma unroll
-        for (int r = 0; r < 4; r++) gasw_load4(in + n0l * gasw_map(y0 - 2 + r, n1, wy0, wy1, f[r]), P, c[r]);
+        for (int r = 0; r < 4; r++) gasw_load4<O>(a.in, base + row * (O)gasw_map(y0 - 2 + r, n1, wy0, wy1, f[r]), P, c[r]);
         Pa = gasw_prim(a, c[0], fx, f[0]);
         Pb = gasw_prim(a, c[1], fx, f[1]);
         P0 = gasw_prim(a, c[2], fx, f[2]);
@@ -202,11 +206,12 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
     }
     float ld[4];
     bool fld;
-    gasw_load4(in + n0l * gasw_map(y0 + 2, n1, wy0, wy1, fld), P, ld);
+    gasw_load4<O>(a.in, base + row * (O)gasw_map(y0 + 2, n1, wy0, wy1, fld), P, ld);
+    O oj = base + row * (O)y0;   // the lane's cell of row j
     float unx[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // U^n of the next row to update (stages 2, 3)
     if (STAGE > 1 && owned)
 #pragma unroll
-        for (int v = 0; v < 5; v++) unx[v] = unp[n0l * y0 + v * P];
+        for (int v = 0; v < 5; v++) unx[v] = *reinterpret_cast<const float *>(reinterpret_cast<const char *>(a.un) + (oj + v * P));
 
     float4 qT, FyB;
     {
@@ -219,19 +224,20 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
 
     float smax = 0.f;
     int bx0 = 0x7fffffff, by0 = 0x7fffffff, bx1 = -1, by1 = -1;
-    for (int j = y0; j < yend; j++) {
+    for (int j = y0; j < yend; j++, oj += row) {
         const float4 P2 = gasw_prim(a, ld, fx, fld);   // row j+2
-        if (j + 3 <= yend + 1) gasw_load4(in + n0l * gasw_map(j + 3, n1, wy0, wy1, fld), P, ld);
+        if (j + 3 <= yend + 1) gasw_load4<O>(a.in, base + row * (O)gasw_map(j + 3, n1, wy0, wy1, fld), P, ld);
         float cin[5], u5[5];
         if (owned) {
 #pragma unroll
-            for (int v = 0; v < 5; v++) cin[v] = __ldg(in + n0l * j + v * P);
+            for (int v = 0; v < 5; v++) cin[v] = gasw_ld<O>(a.in, oj + v * P);
         }
 #pragma unroll
         for (int v = 0; v < 5; v++) u5[v] = STAGE == 1 ? cin[v] : unx[v];
         if (STAGE > 1 && owned && j + 1 < yend)
 #pragma unroll
-            for (int v = 0; v < 5; v++) unx[v] = unp[n0l * (j + 1) + v * P];
+            for (int v = 0; v < 5; v++)
+                unx[v] = *reinterpret_cast<const float *>(reinterpret_cast<const char *>(a.un) + (oj + row + v * P));
 
         // y face j + 1/2 from the slopes of row j+1
         float4 qB1, qT1;
@@ -260,16 +266,10 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
             o[1] = o01.y;
             o[2] = o23.x;
             o[3] = o23.y;
-            {
-                // r: no flux without a moving body
-                Acc<float> D;
-                D.set(0.f);
-                D.add(0.f);
-                o[4] = rk_combine<float>(STAGE, u5[4], cin[4], D, dt, ca, cb);
-            }
-            float *op = out + n0l * j;
+            // r: no flux without a moving body
+            o[4] = STAGE == 1 ? cin[4] : fmaf(cb, cin[4], __fmul_rn(ca, u5[4]));
 #pragma unroll
-            for (int v = 0; v < 5; v++) op[v * P] = o[v];
+            for (int v = 0; v < 5; v++) *reinterpret_cast<float *>(reinterpret_cast<char *>(a.out) + (oj + v * P)) = o[v];
             if (!(o[0] > 0.f) || !(o[3] == o[3])) atomicOr(&ctl->err, (unsigned)ERR_STATE);
             if (STAGE == 3) {
                 if (o[4] > 0.5f) {
@@ -315,7 +315,7 @@ __device__ __forceinline__ void gasw_item(const GaswArgs &a, const GasInst &I, i
     }
 }
 
-template <int STAGE>
+template <int STAGE, class O>
 // stage 1 (no U^n stream of its own) fits in 80 registers: six CTAs per SM
 __global__ void __launch_bounds__(GaswT::THREADS, STAGE == 1 ? 6 : GaswT::MIN_CTAS) k_gasw_stage(GaswArgs a)
 {
@@ -325,13 +325,30 @@ __global__ void __launch_bounds__(GaswT::THREADS, STAGE == 1 ? 6 : GaswT::MIN_CT
     long long it = (long long)blockIdx.x * T::WARPS + (threadIdx.x >> 5);
     const float ca = STAGE == 2 ? 0.75f : (STAGE == 3 ? 1.f / 3.f : 0.f);
     const float cb = STAGE == 2 ? 0.25f : (STAGE == 3 ? 2.f / 3.f : 1.f);
-    pdl_enter();   // the previous kernel (its writes of the stage input) is complete
-    if (a.queue) it = gasw_take(a.queue, lane);
+    if (!a.queue) {
+        // the first item's record does not change: read while the previous
+        // kernel still runs (static schedules; one item a warp unless persistent)
+        if (it < a.nitems) {
+            const int2 w = a.items ? a.items[it] : make_int2(0, (int)it);
+            const GasInst I = a.inst[w.x];
+            pdl_enter();   // the previous kernel (its writes of the stage input) is complete
+            gasw_item<STAGE, O>(a, I, w.y, lane, ca, cb);
+        } else {
+            pdl_enter();
+        }
+        for (it += nw; it < a.nitems; it += nw) {
+            const int2 w = a.items ? a.items[it] : make_int2(0, (int)it);
+            gasw_item<STAGE, O>(a, a.inst[w.x], w.y, lane, ca, cb);
+        }
+        return;
+    }
+    pdl_enter();
+    it = gasw_take(a.queue, lane);
     while (it < a.nitems) {
         // the next item is taken before this one runs (the queue's latency overlaps it)
-        const long long next = a.queue ? gasw_take(a.queue, lane) : it + nw;
+        const long long next = gasw_take(a.queue, lane);
         const int2 w = a.items ? a.items[it] : make_int2(0, (int)it);
-        gasw_item<STAGE>(a, a.inst[w.x], w.y, lane, ca, cb);
+        gasw_item<STAGE, O>(a, a.inst[w.x], w.y, lane, ca, cb);
         it = next;
     }
 }
