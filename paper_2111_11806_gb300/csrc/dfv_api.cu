@@ -224,7 +224,7 @@ dfv_status finalize(dfv_grid *g, int mode, long long nb_max)
                "k_finalize_lite");
         return DFV_OK;
     }
-    DFV_CU(g, dfv::launch_pdl(dfv::k_finalize, dim3(1), dim3(1024), 0, g->stream, g->ctl, (const double *)g->partials,
+    DFV_CU(g, dfv::launch_pdl(dfv::k_finalize, dim3(1), dim3(dfv::FINALIZE_THREADS), 0, g->stream, g->ctl, (const double *)g->partials,
                               nb_max, g->nb_stage, mode, g->dim, g->g.dx[0], g->g.dx[1], g->g.dx[2]),
            "k_finalize");
     return DFV_OK;
@@ -333,7 +333,9 @@ dfv_status launch_stage(dfv_grid *g, int s, const void *in, const void *un, void
         DFV_CU(g, dfv::gasw_stage(s, a, g->gas_grid, g->stream), "k_gasw_stage");
         return DFV_OK;
     }
-    DFV_CU(g, g->ops->stage(s, g->g, in, un, out, g->ctl, g->partials, want_force, next, g->stream), "k_stage");
+    const int rest = g->dynamic || g->body_moving ? 0 : 2;
+    DFV_CU(g, g->ops->stage(s, g->g, in, un, out, g->ctl, g->partials, (want_force ? 1 : 0) | rest, next, g->stream),
+           "k_stage");
     return DFV_OK;
 }
 
@@ -727,11 +729,14 @@ dfv_status dfv_set_body(dfv_grid *g, const double v[3], const double x[3], doubl
     k_set_body<<<1, 1, 0, g->stream>>>(g->ctl, vv[0], vv[1], vv[2], xx[0], xx[1], xx[2], mass, dynamic ? 1 : 0);
     g->launches++;
     DFV_CU(g, cudaGetLastError(), "k_set_body");
+    // the captured step reads velocity, position and mass from the control
+    // block; which kernels it launches depends on whether the body moves
+    const bool moving = vv[0] != 0.0 || vv[1] != 0.0 || vv[2] != 0.0;
+    if (g->dynamic != (dynamic != 0) || g->body_moving != moving) g->graph_ready = false;
     g->dynamic = dynamic != 0;
-    g->body_moving = vv[0] != 0.0 || vv[1] != 0.0 || vv[2] != 0.0;
+    g->body_moving = moving;
     g->smax_valid = false;   // the body speed enters the CFL bound
     g->dt_valid = false;
-    g->graph_ready = false;
     return DFV_OK;
 }
 

@@ -14,7 +14,7 @@ struct BatchInst {
     GridP g;            // the instance's grid and materials (pitch: its own)
     long long off;      // element offset of its planes in the state arrays
     long long part0;    // its first slot in the partials array (4 doubles each)
-    int tiles_x, tiles_y, ntiles, pad;
+    int tiles_x, tiles_y, ntiles, rest;   // rest: its body does not move
     Ctl *ctl;           // its control block (dt, t, smax, ticket, error word)
 };
 
@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(Tile<2, 0>::THREADS, (sizeof(R) == 4 && NMAT =
         a.ctl = I.ctl;
         a.partials = b.partials + 4 * I.part0;
         a.want_force = 0;
+        a.rest = I.rest;
         a.early = 0;
         a.next = 0;
         stage_tile<R, 2, NMAT, 0, STAGE, 0>(I.g, a, w.y % I.tiles_x, w.y / I.tiles_x, 0, w.y, I.ntiles);
@@ -104,60 +105,50 @@ __global__ void __launch_bounds__(256) k_batch_seed(BatchArgs b)
                                                  (int)(blockIdx.x % SEED_CTAS), SEED_CTAS, false);
 }
 
-// CFL wave speed of every instance's stored state; the last tile of each
-// instance reduces its partials and sets its dt (b.final_mode).
+// CFL wave speed of every instance's stored state: blockIdx.y the instance,
+// blockIdx.x its CFL_CELLS cells, the block's maximum folded into the
+// instance's running maximum as stage 3 does; the finalize launch that follows
+// sets its dt.  (One CTA for each 256 cells with a ticket for the last of an
+// instance, which reduced their partials, took 826 us on 26 million cells;
+// read once they are 525 MB.)
+constexpr int CFL_CELLS = 4096;
+
 template <class R, int NMAT>
-__global__ void __launch_bounds__(Tile<2, 0>::THREADS) k_batch_cfl(BatchArgs b)
+__global__ void __launch_bounds__(256) k_batch_cfl(const BatchInst *inst, const void *Uv)
 {
-    using TL = Tile<2, 0>;
-    using L = Lay<2, NMAT, false>;
-    __shared__ BatchInst s_inst;
-    __shared__ long long s_item;
-    __shared__ int s_cur;
-    __shared__ double sred[4 * 32];
-    __shared__ unsigned int s_last;
-    if (threadIdx.x == 0) s_cur = -1;
-    for (long long it = next_item(b, -1, &s_item); it < b.nitems; it = next_item(b, it, &s_item)) {
-        const int2 w = b.items[it];
-        __syncthreads();
-        if (s_cur != w.x) {
-            load_inst(&b.inst[w.x], &s_inst);
-            __syncthreads();
-            if (threadIdx.x == 0) s_cur = w.x;
-        }
-        __syncthreads();
-        const BatchInst &I = s_inst;
-        double red[4] = {0.0, 0.0, 0.0, 0.0};
-        if (threadIdx.x < TL::TX * TL::TY) {
-            const int gx = (w.y % I.tiles_x) * TL::TX + threadIdx.x % TL::TX;
-            const int gy = (w.y / I.tiles_x) * TL::TY + threadIdx.x / TL::TX;
-            if (gx < I.g.n[0] && gy < I.g.n[1]) {
-                const R *U = reinterpret_cast<const R *>(b.in) + I.off;
-                const long long c = gx + (long long)I.g.n[0] * gy;
-                R q[L::NVAR], cs;
+    using L = Lay<2, NMAT, 0>;
+    __shared__ R sred[32];
+    const BatchInst &I = inst[blockIdx.y];
+    const long long n = I.g.ncell, P = I.g.pitch, c0 = (long long)blockIdx.x * CFL_CELLS;
+    if (c0 >= n) return;
+    const R *U = reinterpret_cast<const R *>(Uv) + I.off;
+    const long long c1 = min(n, c0 + CFL_CELLS);
+    R top = R(0);
+    bool bad = false;
+    for (long long c = c0 + threadIdx.x; c < c1; c += 256) {
+        R q[L::NVAR], cs;
 #pragma unroll
-                for (int v = 0; v < L::NVAR; v++) q[v] = U[v * I.g.pitch + c];
-                const R sum = cell_speed<R, 2, NMAT, false>(I.g, q, cs);
-                double sd = (double)sum;
-                if (!(sd == sd)) sd = __longlong_as_double(0x7ff0000000000000LL);
-                red[0] = sd;
-            }
-        }
-        block_reduce4<TL::THREADS>(red, sred);
-        if (threadIdx.x == 0) {
-            b.partials[4 * (I.part0 + w.y)] = red[0];
-            __threadfence();
-            const unsigned int t = atomicAdd(&I.ctl->ticket, 1u);
-            s_last = (t == (unsigned int)(I.ntiles - 1)) ? 1u : 0u;
-        }
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            finalize_block<TL::THREADS>(I.ctl, b.partials + 4 * I.part0, I.ntiles, I.ntiles, b.final_mode, 2,
-                                        I.g.dx[0], I.g.dx[1], I.g.dx[2], sred);
-            if (threadIdx.x == 0) I.ctl->ticket = 0u;
-        }
+        for (int v = 0; v < L::NVAR; v++) q[v] = U[v * P + c];
+        const R s = cell_speed<R, 2, NMAT, 0>(I.g, q, cs);
+        bad = bad || !(s == s);
+        top = nan_max(top, s);
     }
+    top = block_max<256, R>(top, sred);
+    const int nan = __syncthreads_or(bad);
+    if (threadIdx.x == 0) {
+        double m = (double)top;
+        if (nan || !(m >= 0.0)) m = __longlong_as_double(0x7ff0000000000000LL);   // NaN -> +inf: dt = 0
+        atomicMax(&I.ctl->smax_acc, (unsigned long long)__double_as_longlong(m));
+    }
+}
+
+template <class R, int NMAT>
+cudaError_t batch_cfl(int count, long long max_cells, const BatchInst *inst, const void *U, cudaStream_t st)
+{
+    const unsigned bx = (unsigned)((max_cells + CFL_CELLS - 1) / CFL_CELLS);
+    for (int i0 = 0; i0 < count; i0 += 65535)
+        k_batch_cfl<R, NMAT><<<dim3(bx, (unsigned)std::min(count - i0, 65535)), 256, 0, st>>>(inst + i0, U);
+    return cudaGetLastError();
 }
 
 // Finalize of every instance after stage 3, one block per instance: its CFL
@@ -191,6 +182,48 @@ static __global__ void k_batch_set_run(Ctl *ctl, int count, double cfl, double t
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
         ctl[i].cfl = cfl;
         ctl[i].t_end = t_end;
+    }
+}
+
+// Field conversion of every instance in one launch: blockIdx.y the instance,
+// blockIdx.x its FIELD_CELLS cells (blocks past its end return).  ptr: the
+// caller's FP64 planes of each instance, in memory the device can address,
+// passed with the launch (nothing of the host is read later).  One
+// launch for FIELD_INST instances instead of one for each (256 of them left the
+// chip idle between and at the end of each).  MODE 0: primitives in (and the rigid box
+// unknown), 1: conserved out, 2: primitives out.
+constexpr int FIELD_CELLS = 2048, FIELD_INST = 256;
+
+struct FieldPtrs {
+    double *p[FIELD_INST];
+};
+
+template <class R, int NMAT, int MODE>
+__global__ void __launch_bounds__(256) k_batch_fields(const BatchInst *inst, const __grid_constant__ FieldPtrs ptr, void *Uv)
+{
+    using L = Lay<2, NMAT, 0>;
+    const BatchInst &I = inst[blockIdx.y];
+    const long long n = I.g.ncell, P = I.g.pitch, c0 = (long long)blockIdx.x * FIELD_CELLS;
+    if (MODE == 0 && blockIdx.x == 0 && threadIdx.x == 0) I.ctl->rbox_valid = 0;
+    if (c0 >= n) return;
+    R *U = reinterpret_cast<R *>(Uv) + I.off;
+    double *f = ptr.p[blockIdx.y];
+    const long long c1 = min(n, c0 + FIELD_CELLS);
+    for (long long c = c0 + threadIdx.x; c < c1; c += 256) {
+        double a[L::NVAR], b[L::NVAR];
+        if constexpr (MODE == 0) {
+#pragma unroll
+            for (int v = 0; v < L::NVAR; v++) a[v] = f[v * n + c];
+            prim_to_cons<double, 2, NMAT, 0>(I.g, a, b);
+#pragma unroll
+            for (int v = 0; v < L::NVAR; v++) U[v * P + c] = m_store<R>(b[v]);
+        } else {
+#pragma unroll
+            for (int v = 0; v < L::NVAR; v++) a[v] = m_widen(U[v * P + c]);
+            if constexpr (MODE == 2) cons_to_prim_ct<double, 2, NMAT, 0>(I.g, a, b);
+#pragma unroll
+            for (int v = 0; v < L::NVAR; v++) f[v * n + c] = MODE == 2 ? b[v] : a[v];
+        }
     }
 }
 
@@ -228,7 +261,7 @@ struct BK {
         default: launch_pdl(k_batch_seed<R, NMAT, MODE, 3>, dim3(grid * SEED_CTAS), dim3(256), 0, st, a); break;
         }
     }
-    // phase: 0 seed in place, 1..3 stages, 4 CFL, 5 / 6 seed to scratch / apply,
+    // phase: 0 seed in place, 1..3 stages, 5 / 6 seed to scratch / apply,
     // 7 finalize after stage 3;
     // opt: the seeding option set (seed_opt)
     static cudaError_t launch(int phase, int grid, const BatchArgs &a, int opt, cudaStream_t st)
@@ -240,25 +273,45 @@ struct BK {
         case 7: launch_pdl(k_batch_finalize<32>, dim3(grid), dim3(32), 0, st, a); break;
         case 1: launch_pdl(k_batch_stage<R, NMAT, 1>, dim3(grid), dim3(threads), smem, st, a); break;
         case 2: launch_pdl(k_batch_stage<R, NMAT, 2>, dim3(grid), dim3(threads), smem, st, a); break;
-        case 3: launch_pdl(k_batch_stage<R, NMAT, 3>, dim3(grid), dim3(threads), smem, st, a); break;
-        default: k_batch_cfl<R, NMAT><<<grid, threads, 0, st>>>(a); break;
+        default: launch_pdl(k_batch_stage<R, NMAT, 3>, dim3(grid), dim3(threads), smem, st, a); break;
         }
         return cudaGetLastError();
     }
 };
 
+// Field conversion of every instance (mode as k_batch_fields); max_cells: of
+// the largest instance.
+template <class R, int NMAT>
+cudaError_t batch_fields(int mode, int count, long long max_cells, const BatchInst *inst, double *const *ptr, void *U,
+                         cudaStream_t st)
+{
+    const unsigned bx = (unsigned)((max_cells + FIELD_CELLS - 1) / FIELD_CELLS);
+    for (int i0 = 0; i0 < count; i0 += FIELD_INST) {
+        const int n = std::min(count - i0, FIELD_INST);
+        FieldPtrs p;
+        for (int i = 0; i < FIELD_INST; i++) p.p[i] = i < n ? ptr[i0 + i] : nullptr;
+        const dim3 g(bx, (unsigned)n);
+        if (mode == 0) k_batch_fields<R, NMAT, 0><<<g, 256, 0, st>>>(inst + i0, p, U);
+        else if (mode == 1) k_batch_fields<R, NMAT, 1><<<g, 256, 0, st>>>(inst + i0, p, U);
+        else k_batch_fields<R, NMAT, 2><<<g, 256, 0, st>>>(inst + i0, p, U);
+    }
+    return cudaGetLastError();
+}
+
 struct Kern {
     cudaError_t (*prepare)();
     int (*max_ctas_per_sm)();
     cudaError_t (*launch)(int, int, const BatchArgs &, int, cudaStream_t);
+    cudaError_t (*fields)(int, int, long long, const BatchInst *, double *const *, void *, cudaStream_t);
+    cudaError_t (*cfl)(int, long long, const BatchInst *, const void *, cudaStream_t);
 };
 
 template <class R>
 Kern batch_kernels(int nmat)
 {
-    return nmat == 1   ? Kern{BK<R, 1>::prepare, BK<R, 1>::max_ctas_per_sm, BK<R, 1>::launch}
-           : nmat == 2 ? Kern{BK<R, 2>::prepare, BK<R, 2>::max_ctas_per_sm, BK<R, 2>::launch}
-                       : Kern{BK<R, 3>::prepare, BK<R, 3>::max_ctas_per_sm, BK<R, 3>::launch};
+    return nmat == 1   ? Kern{BK<R, 1>::prepare, BK<R, 1>::max_ctas_per_sm, BK<R, 1>::launch, batch_fields<R, 1>, batch_cfl<R, 1>}
+           : nmat == 2 ? Kern{BK<R, 2>::prepare, BK<R, 2>::max_ctas_per_sm, BK<R, 2>::launch, batch_fields<R, 2>, batch_cfl<R, 2>}
+                       : Kern{BK<R, 3>::prepare, BK<R, 3>::max_ctas_per_sm, BK<R, 3>::launch, batch_fields<R, 3>, batch_cfl<R, 3>};
 }
 
 // One translation unit per precision (the FP32 one is built with the fast

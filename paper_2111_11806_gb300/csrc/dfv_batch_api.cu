@@ -197,19 +197,15 @@ int grid_size(dfv_batch *b)
 
 // one launch of a phase.  The dynamic schedule's counters (slots 1-3, one
 // per stage) start at 0 and the finalize phase puts them back to 0 at the end
-// of every step, so no memset sits between the step's kernels.  Seeding
-// (phase 0) and the CFL reduction (phase 4) do little work per item, so they
-// always run one CTA per item and let the hardware overlap the items' memory
-// latency.
+// of every step, so no memset sits between the step's kernels.
 dfv_status phase(dfv_batch *b, int ph, const void *in, const void *un, void *out, int final_mode, int slot)
 {
     BatchArgs a = args(b, in, un, out, final_mode);
-    const bool light = (ph == 0 || ph == 4 || ph == 5 || ph == 6 || ph == 7);
-    if (b->schedule == 2 && !light) a.queue = b->d_queue + slot;
-    if (ph == 7) a.queue = b->d_queue;
     // seeding: SEED_CTAS per instance (the launcher multiplies); finalize: one
-    // per instance; CFL: one CTA per work item
+    // per instance
     const bool per_inst = (ph == 0 || ph == 5 || ph == 6 || ph == 7);
+    if (b->schedule == 2 && !per_inst) a.queue = b->d_queue + slot;
+    if (ph == 7) a.queue = b->d_queue;
     if (b->gas && ph >= 1 && ph <= 3) {
         const dfv::MatC<float> &m = b->hinst[0].g.mc_f[0];
         dfv::GaswArgs ga;
@@ -232,7 +228,7 @@ dfv_status phase(dfv_batch *b, int ph, const void *in, const void *un, void *out
         b->launches++;
         return DFV_OK;
     }
-    const int grid = per_inst ? b->count : (light ? (int)std::max(1LL, b->plan.nitems) : grid_size(b));
+    const int grid = per_inst ? b->count : grid_size(b);
     B_CU(b, b->kern.launch(ph, grid, a, b->seed_opt, b->stream), "batch kernel");
     b->launches++;
     return DFV_OK;
@@ -293,7 +289,9 @@ dfv_status ensure_dt(dfv_batch *b, double cfl, double t_end)
         b->dt_valid = false;
     }
     if (!b->dt_valid) {
-        dfv_status s = phase(b, 4, b->U, b->U, b->U, 1 | 8, 4);
+        B_CU(b, b->kern.cfl(b->count, b->plan.max_cells, b->d_inst, b->U, b->stream), "k_batch_cfl");
+        b->launches++;
+        dfv_status s = phase(b, 7, b->U, b->U, b->U, 1 | 8, 0);
         if (s != DFV_OK) return s;
         b->dt_valid = true;
     }
@@ -407,6 +405,7 @@ dfv_status dfv_batch_create(int dim, int count, const dfv_instance_desc *desc, i
         I.tiles_x = P.tiles_x[i];
         I.tiles_y = P.tiles_y[i];
         I.ntiles = P.tiles_x[i] * P.tiles_y[i];
+        I.rest = desc[i].v_body[0] == 0.0 && desc[i].v_body[1] == 0.0;
         I.ctl = b->d_ctl + i;
     }
     // work lists: instance order, and largest instances first
@@ -594,6 +593,23 @@ dfv_status get_one(dfv_batch *b, int i, double *outp, int which, int on_device)
     return DFV_OK;
 }
 
+// The conversion of every instance's fields in one launch, when all of the
+// caller's buffers are memory that the device can address (done is then
+// set); mode as k_batch_fields.
+dfv_status all_fields(dfv_batch *b, const double *const *ptrs, int mode, int on_device, bool &done)
+{
+    done = false;
+    std::vector<double *> p(b->count);
+    for (int i = 0; i < b->count; i++) {
+        p[i] = const_cast<double *>(on_device ? ptrs[i] : static_cast<const double *>(mapped_host(ptrs[i])));
+        if (!p[i]) return DFV_OK;
+    }
+    B_CU(b, b->kern.fields(mode, b->count, b->plan.max_cells, b->d_inst, p.data(), b->U, b->stream), "k_batch_fields");
+    b->launches += (b->count + dfv::FIELD_INST - 1) / dfv::FIELD_INST;
+    done = true;
+    return DFV_OK;
+}
+
 dfv_status set_ready(dfv_batch *b)
 {
     if (b->nmat != b->nmat_opt) return bfail(b, DFV_ERR_ARG, "dfv_batch_set_fields: materials missing");
@@ -622,7 +638,13 @@ dfv_status dfv_batch_set_all_fields(dfv_batch *b, const double *const *prim, int
     for (int i = 0; i < b->count; i++)
         if (!prim[i]) return bfail(b, DFV_ERR_ARG, "dfv_batch_set_all_fields: bad arguments");
     dfv_status s = set_ready(b);
-    for (int i = 0; i < b->count && s == DFV_OK; i++) s = set_one(b, i, prim[i], on_device);
+    bool done = false;
+    if (s == DFV_OK) s = all_fields(b, prim, 0, on_device, done);
+    if (s == DFV_OK && done) {
+        b->fields_set.assign(b->count, 1);
+        b->dt_valid = false;
+    }
+    for (int i = 0; i < b->count && s == DFV_OK && !done; i++) s = set_one(b, i, prim[i], on_device);
     if (s != DFV_OK) return s;
     if (!on_device) B_CU(b, cudaStreamSynchronize(b->stream), "set_all_fields sync");
     return DFV_OK;
@@ -645,10 +667,10 @@ dfv_status dfv_batch_get_all_fields(dfv_batch *b, double *const *out, int which,
     if (!out) return bfail(b, DFV_ERR_ARG, "dfv_batch_get_all_fields: bad arguments");
     for (int i = 0; i < b->count; i++)
         if (!out[i] || !b->fields_set[i]) return bfail(b, DFV_ERR_ARG, "dfv_batch_get_all_fields: bad arguments");
-    for (int i = 0; i < b->count; i++) {
-        dfv_status s = get_one(b, i, out[i], which, on_device);
-        if (s != DFV_OK) return s;
-    }
+    bool done = false;
+    dfv_status s = all_fields(b, out, which == DFV_FIELDS_PRIMITIVE ? 2 : 1, on_device, done);
+    for (int i = 0; i < b->count && s == DFV_OK && !done; i++) s = get_one(b, i, out[i], which, on_device);
+    if (s != DFV_OK) return s;
     if (!on_device) B_CU(b, cudaStreamSynchronize(b->stream), "get_all_fields sync");
     return DFV_OK;
 }

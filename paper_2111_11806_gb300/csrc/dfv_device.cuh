@@ -379,6 +379,45 @@ __device__ __forceinline__ float m_fma(float a, float b, float c) { return fmaf(
 // relative error e of the start becomes e^3; e < 2^-19), and comparisons and
 // selections work on the bits.
 
+// Conversions between the precisions by integer arithmetic, the same values as
+// the conversion instructions, which go through the FP64 pipe: exact to FP64,
+// to nearest (ties to even) to FP32.  Subnormals, infinities, NaNs and
+// overflows take the instruction (volatile: else it is executed for all and its
+// result selected).
+__device__ __forceinline__ double m_widen(float x)
+{
+    const unsigned u = __float_as_uint(x);
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    if ((((u >> 23) + 1u) & 0xffu) <= 1u) {   // exponent 0 or 255
+        double r;
+        asm volatile("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(x));
+        return r;
+    }
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double m_widen(double x) { return x; }
+__device__ __forceinline__ float m_narrow(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    const unsigned e = (unsigned)(b >> 52);
+    if (b == 0ull) return __uint_as_float((unsigned)__double2hiint(x));
+    if (e - 897u > 252u) {   // outside the normal range below the last binade
+        float r;
+        asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(x));
+        return r;
+    }
+    const unsigned q = (unsigned)(b >> 29), rem = (unsigned)b & 0x1fffffffu;
+    const unsigned r = q - 0xc0000000u + ((rem + 0x0fffffffu + (q & 1u)) >> 29);
+    return __uint_as_float(r | ((unsigned)__double2hiint(x) & 0x80000000u));
+}
+// to the storage type
+template <class R>
+__device__ __forceinline__ R m_store(double x);
+template <>
+__device__ __forceinline__ double m_store<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float m_store<float>(double x) { return m_narrow(x); }
+
 // 1/x: y (1 + e + e^2), e = 1 - x y
 __device__ __forceinline__ double m_rcp(double x)
 {
@@ -752,7 +791,7 @@ __device__ __forceinline__ void unpack_A(const T *w, double A[3][3])
 #pragma unroll
         for (int b = 0; b < 3; b++) A[a][b] = 0.0;
 #pragma unroll
-    for (int c = 0; c < L::NV; c++) A[v_row(DIM, c)][v_col(DIM, c)] = (double)w[L::IV + c];
+    for (int c = 0; c < L::NV; c++) A[v_row(DIM, c)][v_col(DIM, c)] = m_widen(w[L::IV + c]);
 }
 
 // The closure of the FP32 fluid mixtures: the same rules, material by material.
@@ -891,6 +930,12 @@ __device__ __forceinline__ bool needs_fp64(const T *phi_first)
     mn = m_min(mn, last);
     present += last >= T(1e-6);
     return present >= 2 && mn < T(1e-6);
+}
+
+template <class T, int NMAT>
+__device__ __forceinline__ bool fp64_closure(const T *phi_first)
+{
+    return sizeof(T) == 4 && needs_fp64<T, NMAT>(phi_first);
 }
 
 // State from primitives in the compute type T; the FP32 form switches to FP64
@@ -1469,7 +1514,9 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
         sig_t[a] = T(0);
-        us[a] = a == D ? (star ? Ss : uK) : (star && sgn == 0 ? T(0.5) * (sl.u[a] + sr.u[a]) : K.u[a]);
+        us[a] = a == D ? m_sel(star, Ss, uK) : K.u[a];
+        // (a solid's stretch flux alone reads the tangential velocity of a standing contact)
+        if (SOLID && a != D && star && sgn == 0) us[a] = T(0.5) * (sl.u[a] + sr.u[a]);
     }
     if (SOLID) {
         const T ZL = m_sqrt(sl.rho * sl.G), ZR = m_sqrt(sr.rho * sr.G);
@@ -1612,15 +1659,16 @@ __device__ __forceinline__ double exp_near0(double x)
 // in-plane block is e^{-s d2/2} [cosh(s k/2) I + sinh(s k/2) (c_2, s_2)]: the
 // FP64 pipe does some 75 operations for an elastic or yielding metal cell in
 // place of three logarithms, three exponentials, a root and divisions.
+// e: the stretch logarithm of A; sc: the scale s.
 template <int DIM, class Y>
-__device__ __forceinline__ double plastic_return_y(double A[3][3], double G, Y yield)
+__device__ __forceinline__ double plastic_return_y(const StretchLog<double> &e, double A[3][3], double G, Y yield,
+                                                   double &sc)
 {
-    StretchLog<double> e;
-    stretch_log<double, DIM>(A, e);
     const double nd = m_sqrt(e.J2);
     const double svm = sqrt(6.0) * G * nd;
     const double sigY = yield(svm, nd, e.J2);
-    double sc = 1.0, deps = 0.0;
+    double deps = 0.0;
+    sc = 1.0;
     if (svm > sigY) {
         sc = sigY / svm;
         // equivalent plastic strain of the removed deviatoric log-strain (1 - s)|d|
@@ -1647,31 +1695,26 @@ __device__ __forceinline__ double plastic_return_y(double A[3][3], double G, Y y
     return deps;
 }
 
-template <int DIM>
-__device__ __forceinline__ double plastic_return(double A[3][3], double G, double sigY)
-{
-    return plastic_return_y<DIM>(A, G, [sigY](double, double, double) { return sigY; });
-}
-
 // Johnson-Cook flow stress of material m (the law, the reference temperature
 // 298 K and rate 1/s are readings of Table 2, which lists the constants only):
 // (c1 + c2 eps^n)(1 + c3 ln max(rate, 1))(1 - T*^m), T* = (T - 298)/(T_melt - 298)
-// clipped to [0, 1].
-__device__ __forceinline__ double jc_yield(const MatP &m, double eps, double rate, double T)
+// clipped to [0, 1]: its first and last factors.
+__device__ __forceinline__ double jc_yield0(const MatP &m, double eps, double T)
 {
     double ts = (T - 298.0) / (m.jc_tmelt - 298.0);
     ts = ts < 0.0 ? 0.0 : (ts > 1.0 ? 1.0 : ts);
     const double e = eps > 0.0 ? eps : 0.0;
-    return (m.jc_c1 + m.jc_c2 * pow(e, m.jc_n)) * (1.0 + m.jc_c3 * log(rate > 1.0 ? rate : 1.0)) *
-           (1.0 - pow(ts, m.jc_m));
+    return (m.jc_c1 + m.jc_c2 * pow(e, m.jc_n)) * (1.0 - pow(ts, m.jc_m));
 }
 
 // Mixture yield stress of a cell with Johnson-Cook materials (weights
 // phi_l/Gamma_l, Sec. 2.2), each at its plastic strain and at the temperature
 // of its Mie-Grueneisen thermal energy, 298 K + (p - p_ref)/(rho_l Gamma_l C_V);
-// w: the cell's primitives, J2: its |dev ln V|^2.
+// w: the cell's primitives, J2: its |dev ln V|^2.  The rate enters through its
+// logarithm only: the yield stress is y0 + y1 ln max(rate, 1), one evaluation
+// of the powers for the rate-free and the final stress.
 template <class R, int DIM, int NMAT, int SOLID>
-__device__ __forceinline__ double jc_mixture_yield(const GridP &g, const R *w, double J2, double rate)
+__device__ __forceinline__ void jc_mixture_yield(const GridP &g, const R *w, double J2, double &y0, double &y1)
 {
     using L = Lay<DIM, NMAT, SOLID>;
     double fsum = 0.0, phi[NMAT];
@@ -1681,23 +1724,140 @@ __device__ __forceinline__ double jc_mixture_yield(const GridP &g, const R *w, d
         fsum += phi[l];
     }
     phi[NMAT - 1] = 1.0 - fsum;
-    double num = 0.0, den = 0.0;
+    double n0 = 0.0, n1 = 0.0, den = 0.0;
     const double p = (double)w[L::IE];
 #pragma unroll
     for (int l = 0; l < NMAT; l++) {
-        const double ph = phi_clip(phi[l]);
-        const double rl = (double)w[L::IAR + l];
-        const Ref<double> r = mat_ref<double>(g.mc_d[l], rl, J2);
+        const double f = phi_clip(phi[l]) * g.mc_d[l].invGam;
         double sy = g.mat[l].sigY;
         if (g.mat[l].jc) {
+            const double rl = (double)w[L::IAR + l];
+            const Ref<double> r = mat_ref<double>(g.mc_d[l], rl, J2);
             double eps = 0.0;
             if constexpr (SOLID == 2) eps = (double)w[L::IH + l];
-            sy = jc_yield(g.mat[l], eps, rate, 298.0 + (p - r.pref) * m_rcp(rl * g.mc_d[l].Gam * g.mat[l].jc_cv));
+            sy = jc_yield0(g.mat[l], eps, 298.0 + (p - r.pref) * m_rcp(rl * g.mc_d[l].Gam * g.mat[l].jc_cv));
+            n1 += f * sy * g.mat[l].jc_c3;
         }
-        num += ph * sy * g.mc_d[l].invGam;
-        den += ph * g.mc_d[l].invGam;
+        n0 += f * sy;
+        den += f;
     }
-    return num / den;
+    const double i = m_rcp(den);
+    y0 = n0 * i;
+    y1 = n1 * i;
+}
+
+// End of a step for a cell of a solid's grid (Sec. 2.1.1): the plastic return
+// of the new conserved state o, and the wave speed of the state it leaves
+// (cell_speed).  The reference curves are linear in J^2 (p_ref and rho e_ref
+// by G J^2), and the return scales J^2 by s^2, so that pressure, shear modulus
+// and sound speed before and after it come from one stretch logarithm and one
+// evaluation of the curves (FP64 form: five and four before).  The
+// decomposition and the return are FP64 in both forms.
+template <class R, int DIM, int NMAT, int SOLID>
+__device__ __forceinline__ R solid_finish(const GridP &g, double dt, R *o, R &c)
+{
+    using L = Lay<DIM, NMAT, SOLID>;
+    R A[3][3];
+    unpack_A_ct<R, DIM, NMAT, SOLID>(o, A);
+    StretchLog<R> e;
+    stretch_log<R, DIM>(A, e);
+    // sums over the materials: num = num0 + J^2 numJ (over den, the pressure),
+    // Yn = p K1 - K0 + J^2 KJ (mix_sums), G and sigma_Y
+    R phi[NMAT], rhol[NMAT], rho = R(0), rhos = R(0), fsum = R(0);
+#pragma unroll
+    for (int l = 0; l < NMAT - 1; l++) {
+        phi[l] = o[L::IPHI + l];
+        fsum += phi[l];
+    }
+    phi[NMAT - 1] = R(1) - fsum;
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) rho += o[L::IAR + l];
+    const R irho = m_rcp(rho);
+    R u[DIM], mu = R(0);
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+        u[a] = o[L::IMOM + a] * irho;
+        mu = m_fma(o[L::IMOM + a], u[a], mu);
+    }
+    R num0 = m_fma(R(-0.5), mu, o[L::IE]), numJ = R(0), den = R(0), K1 = R(0), K0 = R(0), KJ = R(0), Gn = R(0), Sn = R(0);
+#pragma unroll
+    for (int l = 0; l < NMAT; l++) {
+        const MatC<R> &m = matc<R>(g, l);
+        const R ar = o[L::IAR + l], f = NMAT == 1 ? R(1) : phi_clip(phi[l]);
+        rhol[l] = NMAT == 1 ? rho : phasic_density<R>(g, l, ar, f);
+        const R w = f * m.invGam, as = f * rhol[l];
+        rhos += as;
+        den += w;
+        const R fy = as != R(0) ? f : R(0);   // a material without mass has no part in the sound speed
+        K1 = m_fma(fy, m.kA, K1);
+        if (m.kind == 2) {
+            const Ref<R> r = mat_ref<R>(m, rhol[l], R(0));
+            const R fe = NMAT > 1 && m_less(f, R(1e-6)) ? ar * m.irho0 : f;
+            num0 += w * r.pref - fe * r.re;
+            numJ += (w * m.beta - fe) * r.G;
+            const R ky = fy * m.kA, wy = fy * m.invGam;
+            K0 += ky * r.pref - wy * m_fma(R(4) / R(3), r.G, r.rdp);
+            KJ += (wy * m.bb - ky * m.beta) * r.G;
+            Gn = m_fma(w, r.G, Gn);
+            Sn = m_fma(w, m.sigY, Sn);
+        } else {
+            num0 = m_fma(f, m.kB, num0);
+            K0 = m_fma(fy, m.kB, K0);
+        }
+    }
+    const R iden = m_rcp(den);
+    // the return
+    double Ad[3][3], sc;
+    StretchLog<double> ed;
+    if constexpr (sizeof(R) == 8) {
+        ed = e;
+    } else {
+        unpack_A<R, DIM, NMAT, SOLID>(o, Ad);
+        stretch_log<double, DIM>(Ad, ed);
+    }
+    const double G = m_widen(Gn * iden), sigY = m_widen(Sn * iden);
+    double deps;
+    if (g.any_jc) {
+        // Johnson-Cook: the rate is that of a return at the rate-free
+        // yield stress over the step (one explicit predictor)
+        deps = plastic_return_y<DIM>(ed, Ad, G, [&](double svm, double nd, double J2) {
+            R w[L::NVAR];
+#pragma unroll
+            for (int l = 0; l < NMAT - 1; l++) w[L::IPHI + l] = phi[l];
+#pragma unroll
+            for (int l = 0; l < NMAT; l++) {
+                w[L::IAR + l] = rhol[l];
+                const R ar = o[L::IAR + l];
+                if constexpr (SOLID == 2) w[L::IH + l] = ar != R(0) ? o[L::IH + l] * m_rcp(ar) : R(0);
+            }
+            w[L::IE] = m_fma(numJ, e.J2, num0) * iden;
+            double y0, y1;
+            jc_mixture_yield<R, DIM, NMAT, SOLID>(g, w, J2, y0, y1);
+            if (!(svm > y0 && dt > 0.0)) return y0;
+            const double rate = sqrt(2.0 / 3.0) * (1.0 - y0 / svm) * nd / dt;
+            return rate > 1.0 ? y0 + y1 * log(rate) : y0;
+        }, sc);
+    } else {
+        deps = plastic_return_y<DIM>(ed, Ad, G, [sigY](double, double, double) { return sigY; }, sc);
+    }
+#pragma unroll
+    for (int k = 0; k < L::NV; k++) o[L::IV + k] = m_store<R>(Ad[v_row(DIM, k)][v_col(DIM, k)]);
+    if constexpr (SOLID == 2) {
+        // the strain removed by the return, added to every material with a yield stress
+#pragma unroll
+        for (int l = 0; l < NMAT; l++)
+            if ((matc<R>(g, l).sigY > R(0) || g.mat[l].jc) && deps > 0.0)
+                o[L::IH + l] = (R)((double)o[L::IH + l] + (double)o[L::IAR + l] * deps);
+    }
+    // wave speed of the state after the return
+    const R s2 = (R)sc, J2 = s2 * s2 * e.J2;
+    const R p = m_fma(numJ, J2, num0) * iden;
+    const R Yn = m_fma(p, K1, m_fma(J2, KJ, -K0));
+    c = NMAT == 1 ? m_sqrt_ratio(Yn * matc<R>(g, 0).Gam, rhos) : m_sqrt_ratio(Yn, rhos * den);
+    R sum = R(0);
+#pragma unroll
+    for (int d = 0; d < DIM; d++) sum += (m_abs(u[d]) + c) * gridc<R>(g).inv_dx[d];
+    return sum;
 }
 
 }  // namespace dfv

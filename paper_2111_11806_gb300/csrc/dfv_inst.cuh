@@ -11,10 +11,10 @@ namespace dfv {
 template <class R, int DIM, int NMAT, int SOLID>
 struct Impl {
     using L = Lay<DIM, NMAT, SOLID>;
-    // tile sizes that are built: in FP32 the large one only (a CTA's time is
+    // tile sizes that are built: in 2-D FP32 the large one only (a CTA's time is
     // then a chain of dependent work, not the SM's FP64 pipe, and the order of
     // the pressure-force sum, which goes by tiles, stays)
-    static constexpr int NV = DIM <= 2 && sizeof(R) == 8 ? 2 : 1;
+    static constexpr int NV = DIM == 1 || (DIM == 2 && sizeof(R) == 8) ? 2 : 1;
 
     template <int V>
     static dim3 tile_grid(const GridP &g)
@@ -157,9 +157,10 @@ struct Impl {
         return n;
     }
 
-    // next: the seeding before stage 1 reads its box from ctl->rnext
+    // next: the seeding before stage 1 reads its box from ctl->rnext;
+    // flags: bit 0 the pressure force is wanted, bit 1 the body is at rest
     static cudaError_t stage(int s, const GridP &g, const void *in, const void *un, void *out, Ctl *ctl,
-                             double *partials, int want_force, int next, cudaStream_t st)
+                             double *partials, int flags, int next, cudaStream_t st)
     {
         StageArgs a;
         a.in = in;
@@ -167,7 +168,8 @@ struct Impl {
         a.out = out;
         a.ctl = ctl;
         a.partials = partials;
-        a.want_force = want_force;
+        a.want_force = flags & 1;
+        a.rest = flags >> 1 & 1;
         a.early = 0;   // set with the tile size
         a.next = next;
         if (s == 1) return stage_s<1>(g, a, st);

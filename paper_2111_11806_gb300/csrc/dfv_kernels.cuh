@@ -242,6 +242,7 @@ __device__ __forceinline__ void finalize_block(Ctl *ctl, const double *partials,
     constexpr int NWORD = (int)(sizeof(Ctl) / sizeof(unsigned long long));
     for (int k = threadIdx.x; k < NWORD; k += THREADS)
         reinterpret_cast<unsigned long long *>(&sc)[k] = reinterpret_cast<const unsigned long long *>(ctl)[k];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double red[4] = {0.0, 0.0, 0.0, 0.0};
     // tiles of a stage-3 launch fold their maximum into ctl->smax_acc instead
     // of a partial (nb_cfl = 0 then): read it and leave it at 0
@@ -249,14 +250,28 @@ __device__ __forceinline__ void finalize_block(Ctl *ctl, const double *partials,
     if (mode & 1)
         for (long long b = threadIdx.x; b < nb_cfl; b += THREADS) red[0] = fmax(red[0], partials[4 * b]);
     if (mode & 2) {
+#pragma unroll 4
         for (long long b = threadIdx.x; b < nb_force; b += THREADS) {
             red[1] += partials[4 * b + 1];
             red[2] += partials[4 * b + 2];
-            red[3] += partials[4 * b + 3];
+            if (dim > 2) red[3] += partials[4 * b + 3];
         }
-        block_reduce4<THREADS>(red, sred);
-    } else {
+        // warps, then the warps' sums in one warp, in a fixed order
+        for (int k = 1; k <= dim; k++) {
+            for (int o = 16; o > 0; o >>= 1) red[k] += __shfl_down_sync(0xffffffffu, red[k], o);
+            if (lane == 0) sred[k * 32 + warp] = red[k];
+        }
+    }
+    if (nb_cfl > 0) {
         red[0] = block_max<THREADS, double>(red[0], sred);
+    }
+    __syncthreads();
+    if ((mode & 2) && warp == 0) {
+        constexpr int NW = THREADS / 32;
+        for (int k = 1; k <= dim; k++) {
+            red[k] = lane < NW ? sred[k * 32 + lane] : 0.0;
+            for (int o = 16; o > 0; o >>= 1) red[k] += __shfl_down_sync(0xffffffffu, red[k], o);
+        }
     }
     __syncthreads();     // the shared copy is complete
     if (threadIdx.x != 0) return;
@@ -329,13 +344,18 @@ static __global__ void __launch_bounds__(32) k_finalize_lite(Ctl *ctl, int mode,
     finalize_warp(ctl, mode, dim, dxs, true);
 }
 
-static __global__ void __launch_bounds__(1024) k_finalize(Ctl *ctl, const double *partials, long long nb_cfl,
+// 256 threads: the sums of a dynamic body's force go through one SM's FP64
+// pipe, and shuffles of more warps cost more of it than they save in loads
+// (2048 tiles: 24 us with 1024 threads and a serial last sum).
+constexpr int FINALIZE_THREADS = 256;
+
+static __global__ void __launch_bounds__(FINALIZE_THREADS) k_finalize(Ctl *ctl, const double *partials, long long nb_cfl,
                                                    long long nb_force, int mode, int dim, double dx0, double dx1,
                                                    double dx2)
 {
     pdl_enter();
     __shared__ double sred[4 * 32];
-    finalize_block<1024>(ctl, partials, nb_cfl, nb_force, mode, dim, dx0, dx1, dx2, sred);
+    finalize_block<FINALIZE_THREADS>(ctl, partials, nb_cfl, nb_force, mode, dim, dx0, dx1, dx2, sred);
 }
 
 // --------------------------------------------------------------- seeding
@@ -529,6 +549,11 @@ constexpr int SEED_G = 8;
 // arithmetic against another).
 #define PROBE_SNAP 1e-3
 
+// a/b: in FP64 a times the given 1/b, a division being a chain of some ten
+// dependent operations of the FP64 pipe in a kernel that waits for little else
+__device__ __forceinline__ double seed_div(double a, double, double ib) { return a * ib; }
+__device__ __forceinline__ float seed_div(float a, float b, float) { return a / b; }
+
 template <class R, int DIM>
 __device__ __forceinline__ void probe_point(const GridC<R> &gc, const int ijk[3], const R nv[3], int step, int base[3],
                                             R fr[3])
@@ -542,7 +567,7 @@ __device__ __forceinline__ void probe_point(const GridC<R> &gc, const int ijk[3]
 #pragma unroll
     for (int d = 0; d < DIM; d++) {
         const R xp = gc.lo[d] + ((R)ijk[d] + R(0.5)) * gc.dx[d] + sd * nv[d];
-        const R fi = (xp - gc.lo[d]) / gc.dx[d] - R(0.5);
+        const R fi = seed_div(xp - gc.lo[d], gc.dx[d], gc.inv_dx[d]) - R(0.5);
         R fl = floor(fi);
         R f = fi - fl;
         if (f < R(PROBE_SNAP)) {
@@ -581,7 +606,7 @@ __device__ __forceinline__ bool seed_band_test(const R *U, const GridP &g, const
     gn = R(0);
     if (!(rc > R(0.5))) return false;
 #pragma unroll
-    for (int d = 0; d < DIM; d++) gr[d] = (rn[d][1] - rn[d][0]) / (R(2) * gc.dx[d]);
+    for (int d = 0; d < DIM; d++) gr[d] = seed_div(rn[d][1] - rn[d][0], R(2) * gc.dx[d], R(0.5) * gc.inv_dx[d]);
     gn = m_sqrt(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
     return gn * gc.dxmin > R(1e-10);
 }
@@ -598,7 +623,8 @@ __device__ __forceinline__ bool seed_compute(const R *U, const Ctl *ctl, const G
     const int lane = threadIdx.x & 31, sub = lane & (SEED_G - 1), gbase = lane & ~(SEED_G - 1);
     const unsigned gm = ((1u << SEED_G) - 1u) << gbase;
     {
-        R nv[3] = {-gr[0] / gn, -gr[1] / gn, -gr[2] / gn};
+        const R ign = sizeof(R) == 8 ? m_rcp(gn) : R(0);
+        R nv[3] = {-seed_div(gr[0], gn, ign), -seed_div(gr[1], gn, ign), -seed_div(gr[2], gn, ign)};
         if constexpr (DIM == 2 && (OPT & 1)) {
             double blk[9], n2[2];
 #pragma unroll
@@ -929,6 +955,8 @@ struct StageArgs {
     Ctl *ctl;
     double *partials;   // 4 doubles per block
     int want_force;
+    int rest;           // the body is at rest throughout (known to the host: a load of its velocity would
+                        // stand before the tile's own loads)
     int early;          // stage 1 after the seeding launch: of the first `early` tiles (the first wave
                         // of CTAs), those that read no cell of the seeding box load and compute their
                         // faces before waiting for it
@@ -1076,7 +1104,7 @@ __device__ __forceinline__ void face_pass(const GridP &g, R *sQ, R vr, const R *
 // cell, from the face fluxes in sF (no barrier).
 template <class R, int DIM, int NMAT, int SOLID, int V, int D>
 __device__ __forceinline__ void accum_pass(const GridP &g, const R *sW, const R *sF, bool own, int lx, int ly, int lz,
-                                           Acc<R> *Dacc)
+                                           bool rest, Acc<R> *Dacc)
 {
     using L = Lay<DIM, NMAT, SOLID>;
     using B = Box<DIM, V>;
@@ -1090,6 +1118,16 @@ __device__ __forceinline__ void accum_pass(const GridP &g, const R *sW, const R 
         const R dus = sF[L::NVAR * B::MAXF + fr] - sF[L::NVAR * B::MAXF + fl];
 #pragma unroll
         for (int v = 0; v < L::NVAR; v++) {
+            if (sizeof(R) == 8) {
+                // FP64: a resting body has no r flux; a divergence without
+                // other terms is added in one operation
+                if (v == L::IR && rest) continue;
+                const bool plain = !((v >= L::IPHI && v < L::IPHI + NMAT - 1) || (SOLID && v >= L::IV && v < L::IV + L::NV));
+                if (plain) {
+                    Dacc[v].hi = m_fma(sF[v * B::MAXF + fr] - sF[v * B::MAXF + fl], inv, Dacc[v].hi);
+                    continue;
+                }
+            }
             const R div = (sF[v * B::MAXF + fr] - sF[v * B::MAXF + fl]) * inv;
             R snc = R(0);
             if (v >= L::IPHI && v < L::IPHI + NMAT - 1) snc = sW[v * B::N + bcell] * dus * inv;
@@ -1105,16 +1143,6 @@ __device__ __forceinline__ void accum_pass(const GridP &g, const R *sW, const R 
             else Dacc[v].add(div - snc);
         }
     }
-}
-
-// whether the body rests (read from L2 before the seeding launch is waited for)
-template <class R, int DIM>
-__device__ __forceinline__ bool ctl_rest(const Ctl *c, bool early)
-{
-    bool rest = true;
-#pragma unroll
-    for (int d = 0; d < DIM; d++) rest = rest && (early ? ctl_v_cg<R>(c, d) : ctl_v<R>(c, d)) == R(0);
-    return rest;
 }
 
 // One tile of one SSP-RK3 stage, executed by a whole CTA: (tbx, tby, tbz) is
@@ -1154,7 +1182,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
                           (DIM < 3 || (oz >= B::HZ && oz + TL::TZ + B::HZ <= g.n[2]));
     // without a fraction to reconstruct (one material, the body at rest) the
     // outermost halo cells are read by nobody
-    const bool h2 = NMAT == 1 && ctl_rest<R, DIM>(a.ctl, early);
+    const bool h2 = NMAT == 1 && a.rest;
     const int hw = h2 ? 2 : 3, px = TL::TX + 2 * hw;
     const int n1 = px * TL::TY * TL::TZ, n2 = n1 + (DIM >= 2 ? 2 * hw * TL::TX * TL::TZ : 0),
               n3 = n2 + (DIM >= 3 ? 2 * hw * TL::TX * TL::TY : 0);
@@ -1218,7 +1246,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
     // finalize, the only kind that launch runs, leaves it unchanged)
     R vr[3];
 #pragma unroll
-    for (int d = 0; d < 3; d++) vr[d] = early ? ctl_v_cg<R>(a.ctl, d) : ctl_v<R>(a.ctl, d);
+    for (int d = 0; d < 3; d++) vr[d] = a.rest ? R(0) : (early ? ctl_v_cg<R>(a.ctl, d) : ctl_v<R>(a.ctl, d));
     // the rigid box that stage 3 folds starts empty (the seeding and stage 1,
     // which read it, have finished)
     if (STAGE == 2 && tile_id == 0 && threadIdx.x == 0) ctl_box_reset(a.ctl);
@@ -1237,15 +1265,15 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
         face_pass<R, DIM, NMAT, SOLID, V, 0>(g, sF, vr[0], lo0);
         face_pass<R, DIM, NMAT, SOLID, V, 1>(g, sQ, vr[1], lo1);
         __syncthreads();
-        accum_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, own, lx, ly, lz, Dacc);
-        accum_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, own, lx, ly, lz, Dacc);
+        accum_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, own, lx, ly, lz, a.rest, Dacc);
+        accum_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, own, lx, ly, lz, a.rest, Dacc);
     } else {
         R lo[L::NVAR];
         slope_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, vr[0], lo);
         __syncthreads();
         face_pass<R, DIM, NMAT, SOLID, V, 0>(g, sF, vr[0], lo);
         __syncthreads();
-        accum_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, own, lx, ly, lz, Dacc);
+        accum_pass<R, DIM, NMAT, SOLID, V, 0>(g, sW, sF, own, lx, ly, lz, a.rest, Dacc);
         if constexpr (DIM >= 2) {
             // the other face array, or this one once its divergence is formed
             R *sQ = sF + (SM::NSF - 1) * (size_t)L::NF * B::MAXF;
@@ -1254,7 +1282,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
             __syncthreads();
             face_pass<R, DIM, NMAT, SOLID, V, 1>(g, sQ, vr[1], lo);
             __syncthreads();
-            accum_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, own, lx, ly, lz, Dacc);
+            accum_pass<R, DIM, NMAT, SOLID, V, 1>(g, sW, sQ, own, lx, ly, lz, a.rest, Dacc);
         }
         if constexpr (DIM >= 3) {
             if (SM::NSF == 1) __syncthreads();
@@ -1262,7 +1290,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
             __syncthreads();
             face_pass<R, DIM, NMAT, SOLID, V, 2>(g, sF, vr[2], lo);
             __syncthreads();
-            accum_pass<R, DIM, NMAT, SOLID, V, 2>(g, sW, sF, own, lx, ly, lz, Dacc);
+            accum_pass<R, DIM, NMAT, SOLID, V, 2>(g, sW, sF, own, lx, ly, lz, a.rest, Dacc);
         }
     }
 
@@ -1284,38 +1312,28 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
             if (masked && v != L::IR) {
                 o[v] = unv;
             } else {
-                o[v] = rk_combine<R>(STAGE, unv, in[v * P + c], Dacc[v], dt, ca, cb);
+                o[v] = sizeof(R) == 8 && v == L::IR && a.rest
+                           ? (STAGE == 1 ? in[v * P + c] : ca * unv + cb * in[v * P + c])
+                           : rk_combine<R>(STAGE, unv, in[v * P + c], Dacc[v], dt, ca, cb);
             }
         }
-        if (SOLID && STAGE == 3 && !masked) {
-            // plastic relaxation on the new state (mixture G, sigma_Y from its primitives)
-            R w[L::NVAR];
-            cons_to_prim<R, DIM, NMAT, SOLID>(g, o, w);
-            State<R, DIM, NMAT, SOLID> s;
-            state_from_prim<R, DIM, NMAT, SOLID>(g, w, s);
-            double A[3][3];
-            unpack_A<R, DIM, NMAT, SOLID>(o, A);
-            double deps;
-            if (g.any_jc) {
-                // Johnson-Cook: the rate is that of a return at the rate-free
-                // yield stress over the step (one explicit predictor)
-                const double G = (double)s.G, dtd = a.ctl->dt;
-                deps = plastic_return_y<DIM>(A, G, [&](double svm, double nd, double J2) {
-                    const double sy0 = jc_mixture_yield<R, DIM, NMAT, SOLID>(g, w, J2, 0.0);
-                    const double rate = (svm > sy0 && dtd > 0.0) ? sqrt(2.0 / 3.0) * (1.0 - sy0 / svm) * nd / dtd : 0.0;
-                    return jc_mixture_yield<R, DIM, NMAT, SOLID>(g, w, J2, rate);
-                });
-            } else {
-                deps = plastic_return<DIM>(A, (double)s.G, (double)s.sigY);
-            }
+        R cs = R(0);
+        bool sped = false;   // the wave speed came with the plastic return
+        if constexpr (SOLID != 0 && STAGE == 3) {
+            if (!masked && !fp64_closure<R, NMAT>(o + L::IPHI)) {
+                smax_cell = solid_finish<R, DIM, NMAT, SOLID>(g, a.ctl->dt, o, cs);
+                sped = true;
+            } else if (!masked) {
+                // a cell whose closure the FP32 form does in FP64
+                double od[L::NVAR], cd;
 #pragma unroll
-            for (int cc = 0; cc < L::NV; cc++) o[L::IV + cc] = (R)A[v_row(DIM, cc)][v_col(DIM, cc)];
-            if constexpr (SOLID == 2) {
-                // the strain removed by the return, added to every material with a yield stress
+                for (int v = 0; v < L::NVAR; v++) od[v] = (double)o[v];
+                smax_cell = (R)solid_finish<double, DIM, NMAT, SOLID>(g, a.ctl->dt, od, cd);
+                cs = (R)cd;
+                sped = true;
 #pragma unroll
-                for (int l = 0; l < NMAT; l++)
-                    if ((matc<R>(g, l).sigY > R(0) || g.mat[l].jc) && deps > 0.0)
-                        o[L::IH + l] = (R)((double)o[L::IH + l] + (double)o[L::IAR + l] * deps);
+                for (int v = L::IV; v < L::NVAR; v++)
+                    if (v != L::IR) o[v] = (R)od[v];
             }
         }
 #pragma unroll
@@ -1336,8 +1354,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
         if (STAGE == 3) rigid_new = o[L::IR] > R(0.5);
         if (STAGE == 3) {
             // CFL wave speed of the new state, in the compute precision
-            R cs;
-            smax_cell = cell_speed<R, DIM, NMAT, SOLID>(g, o, cs);
+            if (!sped) smax_cell = cell_speed<R, DIM, NMAT, SOLID>(g, o, cs);
             if (!(cs > R(0))) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
         }
     }
@@ -1459,7 +1476,7 @@ __global__ void __launch_bounds__(256) k_prim_to_cons(const double *prim, long l
         for (int v = 0; v < L::NVAR; v++) w[v] = prim[v * ppitch + c];
         prim_to_cons<double, DIM, NMAT, SOLID>(g, w, q);
 #pragma unroll
-        for (int v = 0; v < L::NVAR; v++) U[v * g.pitch + c] = (R)q[v];
+        for (int v = 0; v < L::NVAR; v++) U[v * g.pitch + c] = m_store<R>(q[v]);
     }
 }
 
@@ -1472,7 +1489,7 @@ __global__ void __launch_bounds__(256) k_cons_to_prim(const void *Uv, double *pr
          c += (long long)gridDim.x * blockDim.x) {
         double q[L::NVAR], w[L::NVAR];
 #pragma unroll
-        for (int v = 0; v < L::NVAR; v++) q[v] = (double)U[v * g.pitch + c];
+        for (int v = 0; v < L::NVAR; v++) q[v] = m_widen(U[v * g.pitch + c]);
         cons_to_prim_ct<double, DIM, NMAT, SOLID>(g, q, w);
 #pragma unroll
         for (int v = 0; v < L::NVAR; v++) prim[v * ppitch + c] = w[v];
@@ -1485,7 +1502,7 @@ __global__ void __launch_bounds__(256) k_cons_to_f64(const void *Uv, double *out
     const R *U = reinterpret_cast<const R *>(Uv);
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < g.ncell;
          c += (long long)gridDim.x * blockDim.x)
-        for (int v = 0; v < nvar; v++) outp[v * ppitch + c] = (double)U[v * g.pitch + c];
+        for (int v = 0; v < nvar; v++) outp[v * ppitch + c] = m_widen(U[v * g.pitch + c]);
 }
 
 }  // namespace dfv

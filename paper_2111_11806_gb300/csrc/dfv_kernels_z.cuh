@@ -154,7 +154,7 @@ __device__ __forceinline__ void z_faces(const GridP &g, R *sQ, R vr, const R *lo
 
 // divergence of direction D (0, 1) of the thread's cell (accum_pass)
 template <class R, int NMAT, int D>
-__device__ __forceinline__ void z_accum(const GridP &g, const R *sQ, const R *w, Acc<R> *Dacc)
+__device__ __forceinline__ void z_accum(const GridP &g, const R *sQ, const R *w, bool rest, Acc<R> *Dacc)
 {
     using L = Lay<3, NMAT, 0>;
     using Z = ZGeo<R>;
@@ -164,6 +164,13 @@ __device__ __forceinline__ void z_accum(const GridP &g, const R *sQ, const R *w,
     const R dus = NMAT > 1 ? q[L::NVAR * Z::MAXF + SF] - q[L::NVAR * Z::MAXF] : R(0);
 #pragma unroll
     for (int v = 0; v < L::NVAR; v++) {
+        if (sizeof(R) == 8 && v >= NMAT - 1) {
+            // FP64: as accum_pass
+            if (v == L::IR && rest) continue;
+            const R df = q[v * Z::MAXF + SF] - q[v * Z::MAXF];
+            Dacc[v].hi = D == 0 ? df * inv : m_fma(df, inv, Dacc[v].hi);
+            continue;
+        }
         const R div = (q[v * Z::MAXF + SF] - q[v * Z::MAXF]) * inv;
         const R snc = (v >= L::IPHI && v < L::IPHI + NMAT - 1) ? w[v] * dus * inv : R(0);
         if (D == 0) Dacc[v].set(div - snc);
@@ -224,7 +231,7 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
     const long long P = g.pitch;
     const int ox = blockIdx.x * Z::TX, oy = blockIdx.y * Z::TY;
     const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, g.n[2]);
-    const int hw = NMAT == 1 && ctl_rest<R, 3>(a.ctl, false) ? 2 : 3;
+    const int hw = NMAT == 1 && a.rest ? 2 : 3;
     const bool interior = ox >= hw && ox + Z::TX + hw <= g.n[0] && oy >= hw && oy + Z::TY + hw <= g.n[1];
     const bool own = threadIdx.x < Z::CELLS;
     const int lx = threadIdx.x % Z::TX, ly = threadIdx.x / Z::TX;
@@ -233,7 +240,7 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
     const int cell = own ? (ly + Z::HY) * Z::BX + (lx + Z::HX) : 0;
     R vr[3];
 #pragma unroll
-    for (int d = 0; d < 3; d++) vr[d] = ctl_v<R>(a.ctl, d);
+    for (int d = 0; d < 3; d++) vr[d] = a.rest ? R(0) : ctl_v<R>(a.ctl, d);
     const R dt = ctl_dt<R>(a.ctl);
     const R ca = STAGE == 2 ? R(0.75) : (STAGE == 3 ? R(1.0 / 3.0) : R(0));
     const R cb = STAGE == 2 ? R(0.25) : (STAGE == 3 ? R(2.0 / 3.0) : R(1));
@@ -293,8 +300,8 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
             const long long c = gx + (long long)g.n[0] * (gy + (long long)g.n[1] * z);
             Acc<R> Dacc[L::NVAR];
             // x, then y, then z, in the order of the tiled kernel
-            z_accum<R, NMAT, 0>(g, sQx, w0, Dacc);
-            z_accum<R, NMAT, 1>(g, sQy, w0, Dacc);
+            z_accum<R, NMAT, 0>(g, sQx, w0, a.rest, Dacc);
+            z_accum<R, NMAT, 1>(g, sQy, w0, a.rest, Dacc);
             const R inv = gc.inv_dx[2];
             const R dus = Fhi[L::NVAR] - Flo[L::NVAR];
             R cun[L::NVAR], o[L::NVAR];
@@ -303,6 +310,16 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
             const bool masked = cun[L::IR] > R(0.5);
 #pragma unroll
             for (int v = 0; v < L::NVAR; v++) {
+                if (sizeof(R) == 8 && v >= NMAT - 1) {
+                    if (v == L::IR && a.rest) {
+                        o[v] = STAGE == 1 ? in[v * P + c] : ca * cun[v] + cb * in[v * P + c];
+                        continue;
+                    }
+                    Dacc[v].hi = m_fma(Fhi[v] - Flo[v], inv, Dacc[v].hi);
+                    o[v] = (masked && v != L::IR) ? cun[v]
+                                                  : rk_combine<R>(STAGE, cun[v], in[v * P + c], Dacc[v], dt, ca, cb);
+                    continue;
+                }
                 const R div = (Fhi[v] - Flo[v]) * inv;
                 const R snc = (v >= L::IPHI && v < L::IPHI + NMAT - 1) ? w0[v] * dus * inv : R(0);
                 Dacc[v].add(div - snc);

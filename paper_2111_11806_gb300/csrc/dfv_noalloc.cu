@@ -119,7 +119,7 @@ extern "C" dfv_status dfv_compute_dt_noalloc(int dim, const int n[3], const doub
     k_noalloc_init_ctl<<<1, 1, 0, st>>>(ctl, v0, v1, v2);
     if (cudaGetLastError() != cudaSuccess) return DFV_ERR_CUDA;
     if (ops->cfl(p, cons, partials, (int)nblocks, st) != cudaSuccess) return DFV_ERR_CUDA;
-    dfv::k_finalize<<<1, 1024, 0, st>>>(ctl, partials, nblocks, 0, 1, dim, p.dx[0], p.dx[1], p.dx[2]);
+    dfv::k_finalize<<<1, dfv::FINALIZE_THREADS, 0, st>>>(ctl, partials, nblocks, 0, 1, dim, p.dx[0], p.dx[1], p.dx[2]);
     if (cudaGetLastError() != cudaSuccess) return DFV_ERR_CUDA;
     double smax = 0.0;
     if (cudaMemcpyAsync(&smax, &ctl->smax, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess)
