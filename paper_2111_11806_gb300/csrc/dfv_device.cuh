@@ -1753,6 +1753,34 @@ __device__ __forceinline__ void jc_mixture_yield(const GridP &g, const R *w, dou
 // and sound speed before and after it come from one stretch logarithm and one
 // evaluation of the curves (FP64 form: five and four before).  The
 // decomposition and the return are FP64 in both forms.
+// The return of a cell below yield (s = 1) in 2-D: A becomes the unimodular
+// stretch of A A^T = B itself.  A 2 x 2 block's root is (B + d I)/sqrt(T), d its
+// own root's determinant |det A_2| and T = tr B + 2 d, so that with the scale to
+// determinant one the block is (B + d I) X^(-1/6), X = (d |A_zz|)^2 T^3: some 33
+// operations of the FP64 pipe in place of 95 by way of the logarithm.  The
+// sixth root starts in FP32 and takes one third-order step; false (nothing
+// written) where X leaves FP32's middle range.
+__device__ __forceinline__ bool elastic_stretch(double A[3][3])
+{
+    const double b00 = fma(A[0][0], A[0][0], A[0][1] * A[0][1]);
+    const double b11 = fma(A[1][1], A[1][1], A[1][0] * A[1][0]);
+    const double b01 = fma(A[0][0], A[1][0], A[0][1] * A[1][1]);
+    const double d = m_abs(fma(A[0][0], A[1][1], -(A[0][1] * A[1][0])));
+    const double T = fma(2.0, d, b00 + b11), m = d * m_abs(A[2][2]);
+    const double X = (m * m) * (T * T * T);
+    const float xf = m_narrow(X);
+    if (!(xf > 1e-25f && xf < 1e25f)) return false;
+    const double y = m_widen(exp2f(log2f(xf) * (-1.f / 6.f)));
+    const double y2 = y * y, e = fma(-X, y2 * y2 * y2, 1.0);
+    const double q = fma(y * e, fma(e, 7.0 / 72.0, 1.0 / 6.0), y);
+    A[2][2] = m_rcp(d * (q * q) * T);
+    A[0][0] = (b00 + d) * q;
+    A[1][1] = (b11 + d) * q;
+    A[0][1] = A[1][0] = b01 * q;
+    A[0][2] = A[2][0] = A[1][2] = A[2][1] = 0.0;
+    return true;
+}
+
 template <class R, int DIM, int NMAT, int SOLID>
 __device__ __forceinline__ R solid_finish(const GridP &g, double dt, R *o, R &c)
 {
@@ -1807,17 +1835,22 @@ __device__ __forceinline__ R solid_finish(const GridP &g, double dt, R *o, R &c)
     }
     const R iden = m_rcp(den);
     // the return
-    double Ad[3][3], sc;
+    double Ad[3][3], sc = 1.0, deps = 0.0;
     StretchLog<double> ed;
+    bool elastic = false;
     if constexpr (sizeof(R) == 8) {
         ed = e;
     } else {
         unpack_A<R, DIM, NMAT, SOLID>(o, Ad);
-        stretch_log<double, DIM>(Ad, ed);
+        // below yield by more than the error of the FP32 stretch (1e-7 against
+        // yield strains of 1e-4 and more)
+        if (DIM == 2 && !g.any_jc && R(2.4494897) * Gn * m_sqrt(e.J2) <= R(0.99) * Sn && e.J2 < R(0.25))
+            elastic = elastic_stretch(Ad);
+        if (!elastic) stretch_log<double, DIM>(Ad, ed);
     }
     const double G = m_widen(Gn * iden), sigY = m_widen(Sn * iden);
-    double deps;
-    if (g.any_jc) {
+    if (elastic) {
+    } else if (g.any_jc) {
         // Johnson-Cook: the rate is that of a return at the rate-free
         // yield stress over the step (one explicit predictor)
         deps = plastic_return_y<DIM>(ed, Ad, G, [&](double svm, double nd, double J2) {
