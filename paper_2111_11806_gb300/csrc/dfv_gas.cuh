@@ -78,6 +78,16 @@ __device__ __forceinline__ float gas_rsqrt(float x)
     return r;
 }
 
+// the halves of four values, for the packed FP32 units
+__device__ __forceinline__ float2 gasw_lo(const float4 &v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 gasw_hi(const float4 &v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float4 gasw_cat(const float2 &l, const float2 &h) { return make_float4(l.x, l.y, h.x, h.y); }
+
+__device__ __forceinline__ float4 gasw_sub(const float4 &p, const float4 &q)
+{
+    return gasw_cat(gas_sub2(gasw_lo(p), gasw_lo(q)), gas_sub2(gasw_hi(p), gasw_hi(q)));
+}
+
 // Conserved (rho, rho u, rho v, rho E) -> primitive (rho, u, v, p) of the gas
 // (a: any argument block with the gas constants Gam, invGam, pref0).
 template <class A>

@@ -110,7 +110,8 @@ struct __align__(128) Gas3Smem {
     float4 fya[Gas3T::FYS][Gas3T::TX];
     float fye[Gas3T::FYS][Gas3T::TX];
     // per column: the carried top z-face value and bottom z-face flux
-    float zcarry[10][Gas3T::CELLS];
+    float4 zqa[Gas3T::CELLS], zfa[Gas3T::CELLS];
+    float zqp[Gas3T::CELLS], zfe[Gas3T::CELLS];
     double red[32];
 };
 
@@ -346,60 +347,90 @@ __device__ __forceinline__ void gas3_places(const Gas3Args &a, Gas3Plane &f, int
     }
 }
 
+// (rho, u, v, w) and p, or the fluxes of (rho, rho u, rho v, rho w) and rho E:
+// the four by twos on the packed FP32 units
+struct Gas3S {
+    float4 a;
+    float p;
+};
+
 // primitives of the column's own cell in a ring slot
-__device__ __forceinline__ void gas3_own(const Gas3Smem &S, int slot, int px, int py, float w[5])
+__device__ __forceinline__ Gas3S gas3_own(const Gas3Smem &S, int slot, int px, int py)
 {
-    const float4 a4 = S.pa[slot][py][px];
-    w[0] = a4.x;
-    w[1] = a4.y;
-    w[2] = a4.z;
-    w[3] = a4.w;
-    w[4] = S.pp[slot][py][px];
+    return {S.pa[slot][py][px], S.pp[slot][py][px]};
 }
 
 // primitives of the own column's cell at plane z, loaded and converted
 // directly (the planes below the chunk, needed for its first z slopes only)
-__device__ __forceinline__ void gas3_column(const Gas3Args &a, int gx, int gy, int z, float w[5])
+__device__ __forceinline__ Gas3S gas3_column(const Gas3Args &a, int gx, int gy, int z)
 {
     bool fz = false, fx = false, fy = false;
     const int gz = gas3_map(z, a.n2, a.wall[2][0], a.wall[2][1], &fz);
     const int cx = gas3_map(gx, a.n0, 0, 0, &fx), cy = gas3_map(gy, a.n1, 0, 0, &fy);
     const long long c = cx + (long long)a.n0 * (cy + (long long)a.n1 * gz);
-    float q[5];
+    float q[5], w[5];
 #pragma unroll
     for (int v = 0; v < 5; v++) q[v] = a.in[c + v * a.pitch];
     gas3_prim(a, q, fz ? 4u : 0u, w);
+    return {make_float4(w[0], w[1], w[2], w[3]), w[4]};
 }
 
-__device__ __forceinline__ void gas3_slope(const float m[5], const float c[5], const float p[5], float lo[5],
-                                           float hi[5])
+// half the limited slope of four values
+__device__ __forceinline__ float4 gas3_half(const float4 &m, const float4 &c, const float4 &p)
 {
-#pragma unroll
-    for (int v = 0; v < 5; v++) {
-        const float h = gas_half_slope(c[v] - m[v], p[v] - c[v]);
-        lo[v] = c[v] - h;
-        hi[v] = c[v] + h;
+    const float4 d = gasw_sub(c, m), e = gasw_sub(p, c);
+    return gasw_cat(gas_half_slope2(gasw_lo(d), gasw_lo(e)), gas_half_slope2(gasw_hi(d), gasw_hi(e)));
+}
+__device__ __forceinline__ float4 gas3_add(const float4 &x, const float4 &y)
+{
+    return gasw_cat(__fadd2_rn(gasw_lo(x), gasw_lo(y)), __fadd2_rn(gasw_hi(x), gasw_hi(y)));
+}
+
+// face values of cell c from its neighbours m and p: lo towards m, hi towards p
+__device__ __forceinline__ void gas3_slope(const Gas3S &m, const Gas3S &c, const Gas3S &p, Gas3S &lo, Gas3S &hi)
+{
+    const float4 h = gas3_half(m.a, c.a, p.a);
+    const float hp = gas_half_slope(c.p - m.p, p.p - c.p);
+    lo.a = gasw_sub(c.a, h);
+    hi.a = gas3_add(c.a, h);
+    lo.p = c.p - hp;
+    hi.p = c.p + hp;
+}
+
+// the same in x and y at once (the two pressures as a pair)
+__device__ __forceinline__ void gas3_slope_xy(const Gas3S &xm, const Gas3S &xp, const Gas3S &ym, const Gas3S &yp,
+                                              const Gas3S &c, Gas3S &xlo, Gas3S &xhi, Gas3S &ylo, Gas3S &yhi)
+{
+    const float4 hx = gas3_half(xm.a, c.a, xp.a), hy = gas3_half(ym.a, c.a, yp.a);
+    xlo.a = gasw_sub(c.a, hx);
+    xhi.a = gas3_add(c.a, hx);
+    ylo.a = gasw_sub(c.a, hy);
+    yhi.a = gas3_add(c.a, hy);
+    const float2 cp = gas_f2(c.p, c.p);
+    const float2 h = gas_half_slope2(gas_sub2(cp, gas_f2(xm.p, ym.p)), gas_sub2(gas_f2(xp.p, yp.p), cp));
+    const float2 lo = gas_sub2(cp, h), hi = __fadd2_rn(cp, h);
+    xlo.p = lo.x;
+    ylo.p = lo.y;
+    xhi.p = hi.x;
+    yhi.p = hi.y;
+}
+
+// HLLC flux of a face normal to direction D (0, 1, 2)
+template <int D>
+__device__ __forceinline__ Gas3S gas3_face(const Gas3Args &a, const Gas3S &l, const Gas3S &r)
+{
+    float L[5] = {l.a.x, l.a.y, l.a.z, l.a.w, l.p}, R[5] = {r.a.x, r.a.y, r.a.z, r.a.w, r.p}, F[5];
+    if (D == 1) {
+        L[1] = l.a.z, L[2] = l.a.w, L[3] = l.a.y;
+        R[1] = r.a.z, R[2] = r.a.w, R[3] = r.a.y;
+    } else if (D == 2) {
+        L[1] = l.a.w, L[2] = l.a.y, L[3] = l.a.z;
+        R[1] = r.a.w, R[2] = r.a.y, R[3] = r.a.z;
     }
-}
-
-// a face state in the order (rho, normal velocity, tangential 1, 2, p) for direction d
-__device__ __forceinline__ void gas3_orient(const float w[5], int d, float o[5])
-{
-    o[0] = w[0];
-    o[1] = w[1 + d];
-    o[2] = w[1 + (d + 1) % 3];
-    o[3] = w[1 + (d + 2) % 3];
-    o[4] = w[4];
-}
-
-// flux in the order of orient back to (rho, rho u, rho v, rho w, rho E)
-__device__ __forceinline__ void gas3_unorient(const float F[5], int d, float o[5])
-{
-    o[0] = F[0];
-    o[1 + d] = F[1];
-    o[1 + (d + 1) % 3] = F[2];
-    o[1 + (d + 2) % 3] = F[3];
-    o[4] = F[4];
+    gas_hllc3(a, L, R, F);
+    return {D == 0 ? make_float4(F[0], F[1], F[2], F[3])
+                   : (D == 1 ? make_float4(F[0], F[3], F[1], F[2]) : make_float4(F[0], F[2], F[3], F[1])),
+            F[4]};
 }
 
 // A tensor copy that did not complete in the bounded wait: report it, and
@@ -410,6 +441,15 @@ __device__ __forceinline__ void gas3_fail(const Gas3Args &a, Gas3Smem &S, const 
         atomicOr(&a.ctl->err, (unsigned)ERR_TIMEOUT);
         (void)mbar_wait(&S.mbar, (f.phase - 1u) & 1u);
     }
+}
+
+// a column's carried top z-face value and bottom z-face flux
+__device__ __forceinline__ void gas3_carry(Gas3Smem &S, int tid, const Gas3S &q, const Gas3S &F)
+{
+    S.zqa[tid] = q.a;
+    S.zqp[tid] = q.p;
+    S.zfa[tid] = F.a;
+    S.zfe[tid] = F.p;
 }
 
 // TMA: the plane boxes come by tensor copies through `map` (over the stage
@@ -467,23 +507,13 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
     }
     gas3_fetch<TMA>(a, &map, S, fp, ox, oy, z0 + 2, interior);
     if (own) {
-        float wm2[5], wm1[5], w0[5], w1[5], lo[5], hi[5], hiM[5], A[5], B[5], F[5];
-        gas3_column(a, gx, gy, z0 - 2, wm2);
-        gas3_column(a, gx, gy, z0 - 1, wm1);
-        gas3_own(S, z0 % T::RING, px, py, w0);
-        gas3_own(S, (z0 + 1) % T::RING, px, py, w1);
-        gas3_slope(wm2, wm1, w0, lo, hiM);   // plane z0-1: its top-face value hiM
+        const Gas3S wm2 = gas3_column(a, gx, gy, z0 - 2), wm1 = gas3_column(a, gx, gy, z0 - 1);
+        const Gas3S w0 = gas3_own(S, z0 % T::RING, px, py), w1 = gas3_own(S, (z0 + 1) % T::RING, px, py);
+        Gas3S lo, hi, hm;
+        gas3_slope(wm2, wm1, w0, lo, hm);    // plane z0-1: its top-face value hm
         gas3_slope(wm1, w0, w1, lo, hi);     // plane z0: bottom-face value lo, top-face value hi
-        gas3_orient(hiM, 2, A);
-        gas3_orient(lo, 2, B);
-        gas_hllc3(a, A, B, F);
-        float Fzlo[5];
-        gas3_unorient(F, 2, Fzlo);           // the bottom z face of plane z0
-#pragma unroll
-        for (int v = 0; v < 5; v++) {
-            S.zcarry[v][tid] = hi[v];
-            S.zcarry[5 + v][tid] = Fzlo[v];
-        }
+        const Gas3S F = gas3_face<2>(a, hm, lo);   // the bottom z face of plane z0
+        gas3_carry(S, tid, hi, F);
     }
 
     float smax_cell = 0.f;
@@ -510,24 +540,17 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
         }
 
         // 2. slopes: x and y of plane z (face values to shared memory), z of plane z+1
-        float qRx[5], qRy[5], qRz1[5], qLz1[5];
+        Gas3S qRx, qRy, qRz1, qLz1;
         if (own) {
-            float wc[5], ww[5], we[5], ws[5], wn[5], hi[5];
-            gas3_own(S, sz, px, py, wc);
-            gas3_own(S, sz, px - 1, py, ww);
-            gas3_own(S, sz, px + 1, py, we);
-            gas3_own(S, sz, px, py - 1, ws);
-            gas3_own(S, sz, px, py + 1, wn);
-            gas3_slope(ww, wc, we, qRx, hi);
-            S.fvxa[cj][ci + 1] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-            S.fvxp[cj][ci + 1] = hi[4];
-            gas3_slope(ws, wc, wn, qRy, hi);
-            S.fvya[cj + 1][ci] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-            S.fvyp[cj + 1][ci] = hi[4];
-            float w1[5], w2[5];
-            gas3_own(S, s1, px, py, w1);
-            gas3_own(S, s2, px, py, w2);
-            gas3_slope(wc, w1, w2, qRz1, qLz1);
+            const Gas3S wc = gas3_own(S, sz, px, py);
+            Gas3S hx, hy;
+            gas3_slope_xy(gas3_own(S, sz, px - 1, py), gas3_own(S, sz, px + 1, py), gas3_own(S, sz, px, py - 1),
+                          gas3_own(S, sz, px, py + 1), wc, qRx, hx, qRy, hy);
+            S.fvxa[cj][ci + 1] = hx.a;
+            S.fvxp[cj][ci + 1] = hx.p;
+            S.fvya[cj + 1][ci] = hy.a;
+            S.fvyp[cj + 1][ci] = hy.p;
+            gas3_slope(wc, gas3_own(S, s1, px, py), gas3_own(S, s2, px, py), qRz1, qLz1);
         } else {
             // the extra warp: lanes 0-7 the right-face values of column -1,
             // lanes 8-15 the left-face values of column TX; every lane the
@@ -536,86 +559,47 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
             const bool west = l < T::TY, east = !west && l < 2 * T::TY;
             const int jh = west ? l : (east ? l - T::TY : 0);
             const int cx = west ? T::H - 1 : T::TX + T::H;
-            float m[5], c0[5], p[5], lo[5], hi[5];
-            gas3_own(S, sz, cx - 1, jh + T::H, m);
-            gas3_own(S, sz, cx, jh + T::H, c0);
-            gas3_own(S, sz, cx + 1, jh + T::H, p);
-            gas3_slope(m, c0, p, lo, hi);
+            Gas3S lo, hi;
+            gas3_slope(gas3_own(S, sz, cx - 1, jh + T::H), gas3_own(S, sz, cx, jh + T::H),
+                       gas3_own(S, sz, cx + 1, jh + T::H), lo, hi);
             if (west) {
-                S.fvxa[jh][0] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-                S.fvxp[jh][0] = hi[4];
+                S.fvxa[jh][0] = hi.a;
+                S.fvxp[jh][0] = hi.p;
             } else if (east) {
-                S.hrxa[jh] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-                S.hrxp[jh] = lo[4];
+                S.hrxa[jh] = lo.a;
+                S.hrxp[jh] = lo.p;
             }
-            gas3_own(S, sz, l + T::H, T::H - 2, m);
-            gas3_own(S, sz, l + T::H, T::H - 1, c0);
-            gas3_own(S, sz, l + T::H, T::H, p);
-            gas3_slope(m, c0, p, lo, hi);
-            S.fvya[0][l] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-            S.fvyp[0][l] = hi[4];
-            gas3_own(S, sz, l + T::H, T::TY + T::H - 1, m);
-            gas3_own(S, sz, l + T::H, T::TY + T::H, c0);
-            gas3_own(S, sz, l + T::H, T::TY + T::H + 1, p);
-            gas3_slope(m, c0, p, lo, hi);
-            S.hrya[l] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-            S.hryp[l] = lo[4];
+            gas3_slope(gas3_own(S, sz, l + T::H, T::H - 2), gas3_own(S, sz, l + T::H, T::H - 1),
+                       gas3_own(S, sz, l + T::H, T::H), lo, hi);
+            S.fvya[0][l] = hi.a;
+            S.fvyp[0][l] = hi.p;
+            gas3_slope(gas3_own(S, sz, l + T::H, T::TY + T::H - 1), gas3_own(S, sz, l + T::H, T::TY + T::H),
+                       gas3_own(S, sz, l + T::H, T::TY + T::H + 1), lo, hi);
+            S.hrya[l] = lo.a;
+            S.hryp[l] = lo.p;
         }
         __syncthreads();
 
         // 3. faces: left x, bottom y, top z of the cell
-        float Fxl[5], Fyl[5], Fzhi[5];
+        Gas3S Fxl, Fyl, Fzhi;
         if (own) {
-            float A[5], B[5], F[5], Lw[5];
-            {
-                const float4 l4 = S.fvxa[cj][ci];
-                const float Lv[5] = {l4.x, l4.y, l4.z, l4.w, S.fvxp[cj][ci]};
-                gas3_orient(Lv, 0, A);
-                gas3_orient(qRx, 0, B);
-                gas_hllc3(a, A, B, F);
-                gas3_unorient(F, 0, Fxl);
-            }
-            {
-                const float4 l4 = S.fvya[cj][ci];
-                const float Lv[5] = {l4.x, l4.y, l4.z, l4.w, S.fvyp[cj][ci]};
-                gas3_orient(Lv, 1, A);
-                gas3_orient(qRy, 1, B);
-                gas_hllc3(a, A, B, F);
-                gas3_unorient(F, 1, Fyl);
-            }
-#pragma unroll
-            for (int v = 0; v < 5; v++) Lw[v] = S.zcarry[v][tid];
-            gas3_orient(Lw, 2, A);
-            gas3_orient(qRz1, 2, B);
-            gas_hllc3(a, A, B, F);
-            gas3_unorient(F, 2, Fzhi);
-            S.fxa[cj][ci] = make_float4(Fxl[0], Fxl[1], Fxl[2], Fxl[3]);
-            S.fxe[cj][ci] = Fxl[4];
-            S.fya[cj][ci] = make_float4(Fyl[0], Fyl[1], Fyl[2], Fyl[3]);
-            S.fye[cj][ci] = Fyl[4];
+            Fxl = gas3_face<0>(a, {S.fvxa[cj][ci], S.fvxp[cj][ci]}, qRx);
+            Fyl = gas3_face<1>(a, {S.fvya[cj][ci], S.fvyp[cj][ci]}, qRy);
+            Fzhi = gas3_face<2>(a, {S.zqa[tid], S.zqp[tid]}, qRz1);
+            S.fxa[cj][ci] = Fxl.a;
+            S.fxe[cj][ci] = Fxl.p;
+            S.fya[cj][ci] = Fyl.a;
+            S.fye[cj][ci] = Fyl.p;
         } else {
             const int l = tid - T::CELLS, jh = l < T::TY ? l : 0;
-            float A[5], B[5], F[5], o[5];
             if (l < T::TY) {
-                const float4 l4 = S.fvxa[jh][T::TX], r4 = S.hrxa[jh];
-                const float Lv[5] = {l4.x, l4.y, l4.z, l4.w, S.fvxp[jh][T::TX]};
-                const float Rv[5] = {r4.x, r4.y, r4.z, r4.w, S.hrxp[jh]};
-                gas3_orient(Lv, 0, A);
-                gas3_orient(Rv, 0, B);
-                gas_hllc3(a, A, B, F);
-                gas3_unorient(F, 0, o);
-                S.fxa[jh][T::TX] = make_float4(o[0], o[1], o[2], o[3]);
-                S.fxe[jh][T::TX] = o[4];
+                const Gas3S F = gas3_face<0>(a, {S.fvxa[jh][T::TX], S.fvxp[jh][T::TX]}, {S.hrxa[jh], S.hrxp[jh]});
+                S.fxa[jh][T::TX] = F.a;
+                S.fxe[jh][T::TX] = F.p;
             }
-            const float4 l4 = S.fvya[T::TY][l], r4 = S.hrya[l];
-            const float Lv[5] = {l4.x, l4.y, l4.z, l4.w, S.fvyp[T::TY][l]};
-            const float Rv[5] = {r4.x, r4.y, r4.z, r4.w, S.hryp[l]};
-            gas3_orient(Lv, 1, A);
-            gas3_orient(Rv, 1, B);
-            gas_hllc3(a, A, B, F);
-            gas3_unorient(F, 1, o);
-            S.fya[T::TY][l] = make_float4(o[0], o[1], o[2], o[3]);
-            S.fye[T::TY][l] = o[4];
+            const Gas3S F = gas3_face<1>(a, {S.fvya[T::TY][l], S.fvyp[T::TY][l]}, {S.hrya[l], S.hryp[l]});
+            S.fya[T::TY][l] = F.a;
+            S.fye[T::TY][l] = F.p;
         }
         __syncthreads();
 
@@ -630,17 +614,29 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
                 cin[v] = (a.in + v * a.pitch)[c];
                 cun[v] = (a.un + v * a.pitch)[c];
             }
-            const float4 e4 = S.fxa[cj][ci + 1], n4 = S.fya[cj + 1][ci];
-            const float Fxr[5] = {e4.x, e4.y, e4.z, e4.w, S.fxe[cj][ci + 1]};
-            const float Fyr[5] = {n4.x, n4.y, n4.z, n4.w, S.fye[cj + 1][ci]};
             const bool masked = cun[5] > 0.5f;
             float o[6];
+            // D = dFx/dx + dFy/dy + dFz/dz; out = ca un + cb (in - dt D)
+            const float4 dx = gasw_sub(S.fxa[cj][ci + 1], Fxl.a), dy = gasw_sub(S.fya[cj + 1][ci], Fyl.a),
+                         dz = gasw_sub(Fzhi.a, S.zfa[tid]);
+            const float2 ix = gas_f2(a.idx, a.idx), iy = gas_f2(a.idy, a.idy), iz = gas_f2(a.idz, a.idz);
+            const float2 mdt = gas_f2(-dt, -dt), ca2 = gas_f2(ca, ca), cb2 = gas_f2(cb, cb);
 #pragma unroll
-            for (int v = 0; v < 5; v++) {
-                const float D = fmaf(Fzhi[v] - S.zcarry[5 + v][tid], a.idz,
-                                     fmaf(Fyr[v] - Fyl[v], a.idy, (Fxr[v] - Fxl[v]) * a.idx));
-                const float y = fmaf(-dt, D, cin[v]);
-                o[v] = masked ? cun[v] : (STAGE == 1 ? y : fmaf(cb, y, __fmul_rn(ca, cun[v])));
+            for (int h = 0; h < 2; h++) {
+                const float2 D = __ffma2_rn(h ? gasw_hi(dz) : gasw_lo(dz), iz,
+                                            __ffma2_rn(h ? gasw_hi(dy) : gasw_lo(dy), iy,
+                                                       __fmul2_rn(h ? gasw_hi(dx) : gasw_lo(dx), ix)));
+                const float2 y = __ffma2_rn(mdt, D, gas_f2(cin[2 * h], cin[2 * h + 1]));
+                const float2 n = gas_f2(cun[2 * h], cun[2 * h + 1]);
+                const float2 t = STAGE == 1 ? y : __ffma2_rn(cb2, y, __fmul2_rn(ca2, n));
+                o[2 * h] = masked ? n.x : t.x;
+                o[2 * h + 1] = masked ? n.y : t.y;
+            }
+            {
+                const float D = fmaf(Fzhi.p - S.zfe[tid], a.idz,
+                                     fmaf(S.fye[cj + 1][ci] - Fyl.p, a.idy, (S.fxe[cj][ci + 1] - Fxl.p) * a.idx));
+                const float y = fmaf(-dt, D, cin[4]);
+                o[4] = masked ? cun[4] : (STAGE == 1 ? y : fmaf(cb, y, __fmul_rn(ca, cun[4])));
             }
             // r: no flux without a moving body
             o[5] = STAGE == 1 ? cin[5] : fmaf(cb, cin[5], __fmul_rn(ca, cun[5]));
@@ -658,13 +654,7 @@ __global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, co
                 if (!(c2 > 0.f)) atomicOr(&a.ctl->err, (unsigned)ERR_SOUND);
             }
         }
-        if (own) {
-#pragma unroll
-            for (int v = 0; v < 5; v++) {
-                S.zcarry[v][tid] = qLz1[v];
-                S.zcarry[5 + v][tid] = Fzhi[v];
-            }
-        }
+        if (own) gas3_carry(S, tid, qLz1, Fzhi);
     }
     if (STAGE == 3) {
         // the column's rigid cells into the box of the next seeding, the

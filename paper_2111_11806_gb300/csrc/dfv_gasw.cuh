@@ -97,11 +97,6 @@ __device__ __forceinline__ float4 gasw_prim(const A &a, const float c[4], bool f
     return make_float4(w[0], fx ? -w[1] : w[1], fy ? -w[2] : w[2], w[3]);
 }
 
-// the (rho, u) and (v, p) halves of a state, for the packed FP32 units
-__device__ __forceinline__ float2 gasw_lo(const float4 &v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 gasw_hi(const float4 &v) { return make_float2(v.z, v.w); }
-__device__ __forceinline__ float4 gasw_cat(const float2 &l, const float2 &h) { return make_float4(l.x, l.y, h.x, h.y); }
-
 // van Leer face values of cell c from its backward and forward differences
 // db = c - m, df = p - c along one direction: lo at its face towards m, hi
 // at its face towards p
@@ -111,11 +106,6 @@ __device__ __forceinline__ void gasw_faces_d(const float4 &c, const float4 &db, 
     const float2 h0 = gas_half_slope2(gasw_lo(db), gasw_lo(df)), h1 = gas_half_slope2(gasw_hi(db), gasw_hi(df));
     lo = gasw_cat(gas_sub2(gasw_lo(c), h0), gas_sub2(gasw_hi(c), h1));
     hi = gasw_cat(__fadd2_rn(gasw_lo(c), h0), __fadd2_rn(gasw_hi(c), h1));
-}
-
-__device__ __forceinline__ float4 gasw_sub(const float4 &p, const float4 &q)
-{
-    return gasw_cat(gas_sub2(gasw_lo(p), gasw_lo(q)), gas_sub2(gasw_hi(p), gasw_hi(q)));
 }
 
 // the same from the neighbours m and p
