@@ -108,9 +108,12 @@ struct Impl {
         if constexpr (NV == 2)
             if (e == cudaSuccess) e = prepare_v<1>();
         if constexpr (ZM) {
-            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 1>, zsmem);
-            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 2>, zsmem);
-            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 3>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 1, false>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 2, false>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 3, false>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 1, true>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 2, true>, zsmem);
+            if (e == cudaSuccess) e = opt_in(k_stage_z<R, NMAT, 3, true>, zsmem);
         }
         return e;
     }
@@ -129,7 +132,9 @@ struct Impl {
         if constexpr (ZM) {
             if (!(S == 1 && a.want_force)) {
                 const int zc = zchunk(g);
-                return launch_pdl(k_stage_z<R, NMAT, S>, zgrid(g, zc), dim3(ZGeo<R>::THREADS), zsmem, st, a, g, zc);
+                const dim3 b(ZGeo<R>::THREADS);
+                return a.rest ? launch_pdl(k_stage_z<R, NMAT, S, true>, zgrid(g, zc), b, zsmem, st, a, g, zc)
+                              : launch_pdl(k_stage_z<R, NMAT, S, false>, zgrid(g, zc), b, zsmem, st, a, g, zc);
             }
         }
         if constexpr (NV == 2)

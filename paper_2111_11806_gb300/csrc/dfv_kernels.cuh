@@ -1415,13 +1415,16 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
 // Register bound of the 2-D forms: four CTAs per SM for the FP32
 // single-material fluid, three for the other FP32 forms (two for solids of
 // three materials, which would spill), two for the FP64 ones
-// (which would otherwise take up to 138 registers and run one 9-warp CTA per
-// SM); twice as many small tiles.
+// (which would otherwise take up to 168 registers and run one 9-warp CTA per
+// SM); twice as many small tiles, but three of the FP64 solids, which four
+// would spill (copper plate 301 x 299: 2596 us a pass with four, 2540 with
+// three; with large tiles 700 x 700: 9712 us with two CTAs, 10098 with one).
 template <class R, int DIM, int NMAT, int SOLID, int V>
 __host__ __device__ constexpr int stage_min_ctas()
 {
-    return DIM != 2 ? 1
-                    : (sizeof(R) == 4 ? (NMAT == 1 && SOLID == 0 ? 4 : (NMAT == 3 && SOLID ? 2 : 3)) : 2) * (V ? 2 : 1);
+    if (DIM != 2) return 1;
+    if (sizeof(R) == 8 && SOLID) return V ? 3 : 2;
+    return (sizeof(R) == 4 ? (NMAT == 1 && SOLID == 0 ? 4 : (NMAT == 3 && SOLID ? 2 : 3)) : 2) * (V ? 2 : 1);
 }
 
 template <class R, int DIM, int NMAT, int SOLID, int STAGE, int V>

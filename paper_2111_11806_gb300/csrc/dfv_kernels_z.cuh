@@ -211,10 +211,15 @@ __device__ __forceinline__ void z_slope_z(const GridP &g, const R *in, const R *
     }
 }
 
-// Two CTAs per SM: the ring and the face arrays take 106 KB in FP64 (53 KB in
-// FP32, three CTAs).
-template <class R, int NMAT, int STAGE>
-__global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_stage_z(StageArgs a, GridP g, int zc)
+// REST: the body is at rest (no r to reconstruct).  Two CTAs per SM in FP64
+// (ring and face arrays 106 KB), three in FP32; a moving body's FP64 kernel
+// takes the registers of one CTA instead, since with the BVD choice of r it
+// would spill 600 bytes a thread.  Measured in FP64 over two steps: sphere
+// 52 x 70 x 59 moving 7172 us with two CTAs, 4500 with one; 97 x 90 x 101 at
+// rest 7236 with one, 6668 with two, 6385 since REST is known at compile time.
+template <class R, int NMAT, int STAGE, bool REST>
+__global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? (REST ? 2 : 1) : 3)
+    k_stage_z(StageArgs a, GridP g, int zc)
 {
     pdl_enter();
     using L = Lay<3, NMAT, 0>;
@@ -231,7 +236,7 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
     const long long P = g.pitch;
     const int ox = blockIdx.x * Z::TX, oy = blockIdx.y * Z::TY;
     const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, g.n[2]);
-    const int hw = NMAT == 1 && a.rest ? 2 : 3;
+    constexpr int hw = NMAT == 1 && REST ? 2 : 3;
     const bool interior = ox >= hw && ox + Z::TX + hw <= g.n[0] && oy >= hw && oy + Z::TY + hw <= g.n[1];
     const bool own = threadIdx.x < Z::CELLS;
     const int lx = threadIdx.x % Z::TX, ly = threadIdx.x / Z::TX;
@@ -240,7 +245,7 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
     const int cell = own ? (ly + Z::HY) * Z::BX + (lx + Z::HX) : 0;
     R vr[3];
 #pragma unroll
-    for (int d = 0; d < 3; d++) vr[d] = a.rest ? R(0) : ctl_v<R>(a.ctl, d);
+    for (int d = 0; d < 3; d++) vr[d] = REST ? R(0) : ctl_v<R>(a.ctl, d);
     const R dt = ctl_dt<R>(a.ctl);
     const R ca = STAGE == 2 ? R(0.75) : (STAGE == 3 ? R(1.0 / 3.0) : R(0));
     const R cb = STAGE == 2 ? R(0.25) : (STAGE == 3 ? R(2.0 / 3.0) : R(1));
@@ -300,8 +305,8 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
             const long long c = gx + (long long)g.n[0] * (gy + (long long)g.n[1] * z);
             Acc<R> Dacc[L::NVAR];
             // x, then y, then z, in the order of the tiled kernel
-            z_accum<R, NMAT, 0>(g, sQx, w0, a.rest, Dacc);
-            z_accum<R, NMAT, 1>(g, sQy, w0, a.rest, Dacc);
+            z_accum<R, NMAT, 0>(g, sQx, w0, REST, Dacc);
+            z_accum<R, NMAT, 1>(g, sQy, w0, REST, Dacc);
             const R inv = gc.inv_dx[2];
             const R dus = Fhi[L::NVAR] - Flo[L::NVAR];
             R cun[L::NVAR], o[L::NVAR];
@@ -311,7 +316,7 @@ __global__ void __launch_bounds__(ZGeo<R>::THREADS, sizeof(R) == 8 ? 2 : 3) k_st
 #pragma unroll
             for (int v = 0; v < L::NVAR; v++) {
                 if (sizeof(R) == 8 && v >= NMAT - 1) {
-                    if (v == L::IR && a.rest) {
+                    if (v == L::IR && REST) {
                         o[v] = STAGE == 1 ? in[v * P + c] : ca * cun[v] + cb * in[v * P + c];
                         continue;
                     }
