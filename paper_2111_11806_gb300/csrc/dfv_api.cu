@@ -514,7 +514,7 @@ dfv_status dfv_create_grid(int dim, const int n[3], const double lo[3], const do
         memset(&I, 0, sizeof(I));
         I.n0 = p.n[0];
         I.n1 = p.n[1];
-        I.rows = opt->gas_rows > 0 ? opt->gas_rows : dfv::gasw_rows((long long)p.n[0] * p.n[1]);
+        I.rows = opt->gas_rows > 0 ? opt->gas_rows : dfv::gasw_rows(p.n[0], p.n[1]);
         I.strips = dfv::gasw_strips(p.n[0]);
         I.nitems = I.strips * ((p.n[1] + I.rows - 1) / I.rows);
         I.off = 0;

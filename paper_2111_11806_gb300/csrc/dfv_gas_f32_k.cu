@@ -2,6 +2,7 @@
 // (dfv_gasw.cuh) and 3-D (dfv_gas3.cuh), and the TMA tensor maps the 3-D
 // kernel reads its plane boxes through.  Built with the fast single-precision
 // divide and square root and flush-to-zero, like the other FP32 kernels.
+#include <algorithm>
 #include <cstring>
 
 #include <cudaTypedefs.h>
@@ -58,15 +59,49 @@ cudaError_t gasw_stage(int stage, const GaswArgs &a, int grid, cudaStream_t st)
 
 int gasw_rows(long long cells)
 {
-    // measured on the cylinders and the 256-ellipse batch: 4-row chunks
-    // below 2^19 cells (512^2: 5.7e9 against 5.2e9 cell-updates/s at 8
-    // rows), then 8, growing to at most 32 while at least four items remain
-    // per resident warp (152 SMs x 20 warps); 64-row chunks were 2 % slower
-    // than 32 on the batch
+    // 4-row chunks below 2^19 cells, then 8, growing to at most 32 while at
+    // least four items remain per resident warp (152 SMs x 20 warps); 64-row
+    // chunks were 2 % slower than 32 on the 256-ellipse batch.  The estimate for
+    // one grid below gained 4 % on some batches and lost 5 % on others: grids of
+    // several sizes do not end their waves together.
     const long long target = 4LL * 152 * GaswT::MIN_CTAS * GaswT::WARPS;
     int rows = cells < (1LL << 19) ? 4 : 8;
     while (rows < 32 && cells / ((long long)GaswT::OWN * rows * 2) >= target) rows *= 2;
     return rows;
+}
+
+int gasw_rows(int n0, int n1)
+{
+    // The length of the least estimated time l (rows + 2): two rows for a
+    // chunk's prologue, l a row's time with the CTAs of the SM that has the most.
+    // In one wave (five are resident) l is about the same from three CTAs on and
+    // less when one or two leave each warp waiting by itself; every whole wave
+    // adds its time, and a last one that begins costs two CTAs more than it has
+    // (half a percent over a whole wave is lost in the spread of its ends).
+    // Fitted to lengths 1 .. 64 on 22 grids of 64^2 .. 3000 x 2000 cells: within
+    // 4 % of the best length's time on each.  us a step with the lengths by the
+    // number of cells alone and with these: 64^2 22.6, 16.4; 320^2 28.6, 24.7;
+    // 640^2 42.6, 38.3; 1200 x 800 70.0, 67.4; 2048^2 248, 231.
+    double least = 1e300;
+    int best = 1;
+    for (int r = 1; r <= 64; r++) {
+        const long long items = (long long)gasw_strips(n0) * ((n1 + r - 1) / r);
+        const long long ctas = (items + GaswT::WARPS - 1) / GaswT::WARPS;
+        long long per = (ctas + 151) / 152;
+        double l;
+        if (per <= GaswT::MIN_CTAS) {
+            l = std::min((double)per + 3.5, 6.0);
+        } else {
+            per = std::max<long long>(GaswT::MIN_CTAS + 1, (ctas * 199 / 200 + 151) / 152);
+            const long long rest = per % GaswT::MIN_CTAS;
+            l = 6.0 * (double)(per / GaswT::MIN_CTAS) + (rest ? (double)rest + 2.0 : 0.0);
+        }
+        if (l * (r + 2) < least) {
+            least = l * (r + 2);
+            best = r;
+        }
+    }
+    return best;
 }
 
 cudaError_t gas3_prepare()

@@ -346,9 +346,11 @@ __global__ void __launch_bounds__(GaswT::THREADS, STAGE == 1 ? 6 : GaswT::MIN_CT
 // Host side (dfv_gas_f32_k.cu).
 int gasw_max_ctas_per_sm();   // resident CTAs per SM of the stage kernels
 cudaError_t gasw_stage(int stage, const GaswArgs &a, int grid, cudaStream_t st);
-// Rows per chunk for grids of `cells` cells in all: long chunks (few repeated
-// halo rows) while there are enough work items to keep every warp busy.
+// Rows per chunk for a batch of `cells` cells in all and for one grid: long
+// chunks (few repeated halo rows) while there are enough work items to keep
+// every warp busy.
 int gasw_rows(long long cells);
+int gasw_rows(int n0, int n1);
 // Strips (28 columns) and items of one instance.
 inline int gasw_strips(int n0) { return (n0 + GaswT::OWN - 1) / GaswT::OWN; }
 

@@ -115,6 +115,23 @@ def test_seeding_of_small_and_large_boxes(n, radius):
     assert np.all(err <= 1e-12), err
 
 
+@pytest.mark.parametrize("n", [(5, 4), (29, 64), (230, 210), (900, 420)])
+def test_gas_rows_chosen_by_size_give_the_same_bits(n):
+    """The chunk length that the size chooses (1, 2 or 5 rows; 4 in the batch)
+    against 8 rows."""
+    wl = W.cylinder_2d(n[0], ny=n[1])
+    ref = B.Grid.from_workload(wl, precision=B.DFV_FP32, gas_rows=8)
+    t = ref.run(4, 0.6)
+    g = B.Grid.from_workload(wl, precision=B.DFV_FP32)
+    assert g.run(4, 0.6) == t
+    np.testing.assert_array_equal(g.cons(), ref.cons())
+    b = B.Batch([wl, wl])
+    b.set_all_fields()
+    b.run(4, 0.6)
+    for i in range(2):
+        np.testing.assert_array_equal(b.get_fields(i), ref.cons())
+
+
 def test_gas_planes_of_4_gib_take_64_bit_offsets():
     """An FP32 2-D gas whose five planes take 4 GiB: its first and last cells
     (a seeded disc among these) against the general kernel on the same grid,
