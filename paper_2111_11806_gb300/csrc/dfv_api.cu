@@ -56,6 +56,7 @@ struct dfv_grid {
     // the material, the options and the body allow it (gas_on)
     bool gas_ready = false;
     bool gas3_ready = false;   // the 3-D gas kernel is prepared (FP32 3-D single-material fluid grid)
+    int gas3_zc = 1;           // ... its planes per CTA
     bool gas3_tma = false;     // ... with the tensor maps of its plane boxes over U, U1, U3
     CUtensorMap gas3_map[3];
     bool body_moving = false;
@@ -306,7 +307,7 @@ dfv_status launch_stage(dfv_grid *g, int s, const void *in, const void *un, void
         a.idz = (float)g->g.inv_dx[2];
         for (int d = 0; d < 3; d++)
             for (int k = 0; k < 2; k++) a.wall[d][k] = g->g.wall[d][k];
-        a.zc = dfv::Gas3T::ZCHUNK;
+        a.zc = g->gas3_zc;
         a.Gam = g->g.mc_f[0].Gam;
         a.invGam = g->g.mc_f[0].invGam;
         a.pref0 = g->g.mc_f[0].pref0;
@@ -501,6 +502,7 @@ dfv_status dfv_create_grid(int dim, const int n[3], const double lo[3], const do
             return DFV_ERR_CUDA;
         }
         g->gas3_ready = true;
+        g->gas3_zc = dfv::gas3_planes(p.n[0], p.n[1], p.n[2]);
         const void *bases[3] = {g->U, g->U1, g->U3};
         g->gas3_tma = true;
         for (int k = 0; k < 3 && g->gas3_tma; k++)

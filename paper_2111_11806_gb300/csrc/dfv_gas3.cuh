@@ -77,9 +77,10 @@ struct Gas3T {
     static constexpr int RING = 3;
     static constexpr int NP = 6;                             // rho, rho u, rho v, rho w, rho E, r
     static constexpr int FXS = TX + 1, FYS = TY + 1;
-    // planes per CTA (256^3 sphere, cell-updates/s at 16 / 24 / 32 / 48 / 64
-    // planes: 8.59 / 8.64 / 8.40 / 8.52 / 8.04e9)
+    // planes per CTA of large grids (256^3 sphere, us a step at 16 / 24 / 32 /
+    // 48 / 64 planes: 1602 / 1590 / 1621 / 1589 / 1611); gas3_planes otherwise
     static constexpr int ZCHUNK = 24;
+    static constexpr int CTAS = 3;   // resident per SM
     // the TMA box of a plane: x from ox-4 (a 16-byte boundary) to ox+35, y
     // from oy-2 to oy+9, the five conserved planes rho .. rho E
     static constexpr int BX = TX + 8, BY = PY, BV = 5;
@@ -455,7 +456,7 @@ __device__ __forceinline__ void gas3_carry(Gas3Smem &S, int tid, const Gas3S &q,
 // TMA: the plane boxes come by tensor copies through `map` (over the stage
 // input's first five planes); else by per-thread asynchronous copies.
 template <int STAGE, bool TMA>
-__global__ void __launch_bounds__(Gas3T::THREADS, 3) k_gas3_stage(Gas3Args a, const __grid_constant__ CUtensorMap map)
+__global__ void __launch_bounds__(Gas3T::THREADS, Gas3T::CTAS) k_gas3_stage(Gas3Args a, const __grid_constant__ CUtensorMap map)
 {
     pdl_enter();
     using T = Gas3T;
@@ -695,6 +696,7 @@ cudaError_t gas3_prepare();
 // floats at base, row stride n0, plane stride n0 n1, variable stride pitch.
 // False when the grid does not allow it (rows or planes not a multiple of 16
 // bytes, a misaligned base); the kernel then copies per thread.
+int gas3_planes(int n0, int n1, int n2);   // planes per CTA
 bool gas3_encode_map(CUtensorMap *map, const void *base, int n0, int n1, int n2, long long pitch);
 // map: the stage input's tensor map, or nullptr for the per-thread copies.
 cudaError_t gas3_stage(int stage, const Gas3Args &a, const CUtensorMap *map, cudaStream_t st);

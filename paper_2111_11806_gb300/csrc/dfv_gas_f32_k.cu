@@ -116,6 +116,33 @@ cudaError_t gas3_prepare()
     return e;
 }
 
+int gas3_planes(int n0, int n1, int n2)
+{
+    // The number of the least estimated time l (planes + 2), two planes for a
+    // chunk's prologue, l a plane's time with the CTAs of the SM that has the
+    // most: nearly the same for one to the three that are resident, a whole
+    // wave's for each wave, and one CTA more than it has for a last one that
+    // begins.  Large grids keep ZCHUNK, as does a grid that would gain less than
+    // 10 % (the estimate's own spread).  Fitted to 2 .. 256 planes on 17 grids:
+    // us a step at 24 planes and at these, 40^3 167, 49; 64^3 173, 63;
+    // 58 x 155 x 86 289, 135; 97 x 90 x 101 452, 269; 128^3 312, 275.
+    const long long cols = (long long)((n0 + Gas3T::TX - 1) / Gas3T::TX) * ((n1 + Gas3T::TY - 1) / Gas3T::TY);
+    auto time = [&](int z) {
+        const long long per = (cols * ((n2 + z - 1) / z) + 151) / 152;
+        const long long full = per / Gas3T::CTAS, rest = per % Gas3T::CTAS;
+        const double l = per == 1 ? 2.4 : per == 2 ? 2.8 : 3.0 * (double)full + (rest ? (double)rest + 1.0 : 0.0);
+        return l * (z + 2);
+    };
+    int best = Gas3T::ZCHUNK;
+    double least = time(best) / 1.1;
+    for (int z = n2 < 2 ? 1 : 2; z <= n2 && z <= 64; z++)
+        if (time(z) < least) {
+            least = time(z);
+            best = z;
+        }
+    return best;
+}
+
 bool gas3_encode_map(CUtensorMap *map, const void *base, int n0, int n1, int n2, long long pitch)
 {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
