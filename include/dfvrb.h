@@ -298,10 +298,10 @@ dfv_status dfv_batch_get_fields(dfv_batch *b, int i, double *out, int which, int
 /* The same for every instance in one call (Sec. 4 setup of many independent
  * problems): prim[i] / out[i] (count pointers, caller-owned, host or device
  * as on_device says) hold instance i's nvar FP64 planes of n[0] n[1] values.
- * The copies and conversions of all instances are issued back to back on the
- * batch's stream and the call returns when they are done (host buffers may
- * then be reused); page-locked host buffers are converted in place, without
- * the staging copy, as for dfv_set_fields. DFV_ERR_ARG for a null pointer (nothing is copied) or,
+ * The call returns when everything is copied and converted (host buffers may
+ * then be reused). Device and page-locked host buffers are converted in place,
+ * 256 instances a launch; where an instance's buffer is pageable, copies and
+ * conversions go instance by instance through the staging area. DFV_ERR_ARG for a null pointer (nothing is copied) or,
  * when reading, an instance whose fields were never set. */
 dfv_status dfv_batch_set_all_fields(dfv_batch *b, const double *const *prim, int on_device);
 dfv_status dfv_batch_get_all_fields(dfv_batch *b, double *const *out, int which, int on_device);

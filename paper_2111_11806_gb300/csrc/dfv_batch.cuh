@@ -15,7 +15,7 @@ struct BatchInst {
     long long off;      // element offset of its planes in the state arrays
     long long part0;    // its first slot in the partials array (4 doubles each)
     int tiles_x, tiles_y, ntiles, rest;   // rest: its body does not move
-    Ctl *ctl;           // its control block (dt, t, smax, ticket, error word)
+    Ctl *ctl;           // its control block (dt, t, smax, error word)
 };
 
 struct BatchArgs {
@@ -26,8 +26,7 @@ struct BatchArgs {
     const int2 *items;       // (instance, tile) in the order of the schedule
     long long nitems;
     double *partials;
-    int final_mode;          // finalize mode: by each instance's last tile (CFL phase) or
-                             // by the finalize phase after stage 3
+    int final_mode;          // mode of the finalize phase (after stage 3 or a CFL reduction)
     unsigned int *queue;     // dynamic schedule: next item counter (nullptr: static round-robin)
 };
 

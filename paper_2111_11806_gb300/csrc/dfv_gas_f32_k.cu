@@ -124,8 +124,8 @@ int gas3_planes(int n0, int n1, int n2)
     // wave's for each wave, and one CTA more than it has for a last one that
     // begins.  Large grids keep ZCHUNK, as does a grid that would gain less than
     // 10 % (the estimate's own spread).  Fitted to 2 .. 256 planes on 17 grids:
-    // us a step at 24 planes and at these, 40^3 167, 49; 64^3 173, 63;
-    // 58 x 155 x 86 289, 135; 97 x 90 x 101 452, 269; 128^3 312, 275.
+    // us a step at 24 planes and at these, 40^3 167, 49; 64^3 173, 61;
+    // 58 x 155 x 86 289, 135; 97 x 90 x 101 452, 266; 128^3 312, 260.
     const long long cols = (long long)((n0 + Gas3T::TX - 1) / Gas3T::TX) * ((n1 + Gas3T::TY - 1) / Gas3T::TY);
     auto time = [&](int z) {
         const long long per = (cols * ((n2 + z - 1) / z) + 151) / 152;
