@@ -34,6 +34,8 @@ struct dfv_grid {
     size_t ws_bytes = 0;
     Ctl *ctl = nullptr;
     double *partials = nullptr;
+    double *force = nullptr;   // the stage blocks' force partials: in partials, or where small tiles are
+                               // more than it holds in the staging area (32 bytes a tile: no step uses it)
     void *U = nullptr, *U1 = nullptr, *U3 = nullptr;
     double *staging = nullptr;
     long long nb_stage = 0, nb_cfl = 0;
@@ -95,9 +97,8 @@ struct Layout {
 
 long long stage_blocks(int dim, const int n[3])
 {
-    // the smallest tile of dfv_kernels.cuh per dimension: an upper bound on the
-    // number of stage blocks of either precision
-    const int tx = 32, ty = dim == 1 ? 1 : 4, tz = dim == 3 ? 2 : 1;
+    // the large tile of dfv_kernels.cuh per dimension
+    const int tx = dim == 1 ? 256 : 32, ty = dim == 1 ? 1 : (dim == 2 ? 8 : 4), tz = dim == 3 ? 2 : 1;
     const long long bx = (n[0] + tx - 1) / tx;
     const long long by = dim >= 2 ? (n[1] + ty - 1) / ty : 1;
     const long long bz = dim >= 3 ? (n[2] + tz - 1) / tz : 1;
@@ -225,8 +226,9 @@ dfv_status finalize(dfv_grid *g, int mode, long long nb_max)
                "k_finalize_lite");
         return DFV_OK;
     }
-    DFV_CU(g, dfv::launch_pdl(dfv::k_finalize, dim3(1), dim3(dfv::FINALIZE_THREADS), 0, g->stream, g->ctl, (const double *)g->partials,
-                              nb_max, g->nb_stage, mode, g->dim, g->g.dx[0], g->g.dx[1], g->g.dx[2]),
+    DFV_CU(g, dfv::launch_pdl(dfv::k_finalize, dim3(1), dim3(dfv::FINALIZE_THREADS), 0, g->stream, g->ctl,
+                              (const double *)(mode & 2 ? g->force : g->partials), nb_max, g->nb_stage, mode, g->dim,
+                              g->g.dx[0], g->g.dx[1], g->g.dx[2]),
            "k_finalize");
     return DFV_OK;
 }
@@ -335,7 +337,7 @@ dfv_status launch_stage(dfv_grid *g, int s, const void *in, const void *un, void
         return DFV_OK;
     }
     const int rest = g->dynamic || g->body_moving ? 0 : 2;
-    DFV_CU(g, g->ops->stage(s, g->g, in, un, out, g->ctl, g->partials, (want_force ? 1 : 0) | rest, next, g->stream),
+    DFV_CU(g, g->ops->stage(s, g->g, in, un, out, g->ctl, g->force, (want_force ? 1 : 0) | rest, next, g->stream),
            "k_stage");
     return DFV_OK;
 }
@@ -488,6 +490,7 @@ dfv_status dfv_create_grid(int dim, const int n[3], const double lo[3], const do
     {
         const dim3 sg = ops->stage_grid(p);
         g->nb_stage = (long long)sg.x * sg.y * sg.z;
+        g->force = g->nb_stage <= std::max(L.nb_stage, L.nb_cfl) ? g->partials : g->staging;
     }
 
     cudaError_t e = ops->prepare();
