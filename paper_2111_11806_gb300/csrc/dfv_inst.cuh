@@ -59,19 +59,28 @@ struct Impl {
     static constexpr size_t zsmem = ZSmem<R, NMAT>::bytes;
 
     // Planes per CTA: the chunk count that gives the SM with the most CTAs the
-    // fewest planes, a chunk's prologue (two more planes of conversions, one
-    // more z slope and face) counted as a plane and a half; among equals the fewest.
-    static int zchunk(const GridP &g)
+    // least time, a chunk's prologue (two more planes of conversions, one more z
+    // slope and face) counted as a plane and a half; among equals the fewest.
+    // tail: the time of a last wave that has fewer CTAs than are resident, in
+    // full waves' CTAs: an FP64 CTA by itself leaves the pipe a third of its
+    // slots, an FP32 one waits most of the time (and a launch of about one CTA
+    // an SM may come two to an SM, as it starts while the one before it ends).
+    // us over two steps (FP64, at rest) and three (FP32, moving) with every CTA
+    // counted alike and with tails: 96^3 9928, 5218 and 1778, 917; 64^3 3561,
+    // 1984 and 746, 475; 97 x 90 x 101 6404, 6401 and 2378, 1181.
+    static int zchunk(const GridP &g, bool rest)
     {
         using Z = ZGeo<R>;
+        const int res = sizeof(R) == 8 ? (rest ? 2 : 1) : 3;
+        const double tail[3] = {0.0, sizeof(R) == 8 ? 1.35 : 2.4, 2.8};
         const long long cols = (long long)((g.n[0] + Z::TX - 1) / Z::TX) * ((g.n[1] + Z::TY - 1) / Z::TY);
-        long long best = -1;
+        double best = -1.0;
         int zbest = g.n[2];
         for (int k = 1; k <= g.n[2] && k <= 64; k++) {
             const int zc = (g.n[2] + k - 1) / k;
             const long long ctas = cols * ((g.n[2] + zc - 1) / zc), per = (ctas + 151) / 152;
-            const long long cost = per * (2 * zc + 3);
-            if (best < 0 || cost < best) {
+            const double cost = ((double)(per / res * res) + tail[per % res]) * (2 * zc + 3);
+            if (best < 0.0 || cost < best) {
                 best = cost;
                 zbest = zc;
             }
@@ -131,7 +140,7 @@ struct Impl {
     {
         if constexpr (ZM) {
             if (!(S == 1 && a.want_force)) {
-                const int zc = zchunk(g);
+                const int zc = zchunk(g, a.rest);
                 const dim3 b(ZGeo<R>::THREADS);
                 return a.rest ? launch_pdl(k_stage_z<R, NMAT, S, true>, zgrid(g, zc), b, zsmem, st, a, g, zc)
                               : launch_pdl(k_stage_z<R, NMAT, S, false>, zgrid(g, zc), b, zsmem, st, a, g, zc);
