@@ -131,6 +131,7 @@ struct Impl {
     static cudaError_t stage_v(const GridP &g, StageArgs a, cudaStream_t st)
     {
         a.early = S == 1 ? first_wave<V>() : 0;
+        a.late = late<V>(g);
         return launch_pdl(k_stage<R, DIM, NMAT, SOLID, S, V>, tile_grid<V>(g), dim3(Tile<DIM, V>::THREADS), smem<V>, st,
                           a, g);
     }
@@ -171,6 +172,22 @@ struct Impl {
         return n;
     }
 
+    // Whether the next launch has to wait for the end of this one.  Started at
+    // once, its CTAs take the slots that are free while this one's still run:
+    // two to an SM that this one left empty, none to others.  That doubles a
+    // stage's time where few CTAs share an SM, not where half of the SMs hold
+    // them all or most slots are taken anyway, nor in FP32 1-D, whose stages
+    // are shorter than the start that is then waited for.  us of five steps with
+    // the next launch at once and late: cylinder 150 x 140 FP64 832, 636; 200 x
+    // 190 953, 817; two-fluid 220 x 120 FP64 (four) 1466, 1197, 300 x 170 FP32
+    // 394, 374; 260 x 250 (567 tiles of 608 slots) 904, 912 without the bound.
+    template <int V>
+    static bool late(const GridP &g)
+    {
+        const long long t = tiles<V>(g);
+        return (DIM > 1 || sizeof(R) == 8) && 2 * t > 152 && 4 * t <= 3LL * first_wave<V>();
+    }
+
     // next: the seeding before stage 1 reads its box from ctl->rnext;
     // flags: bit 0 the pressure force is wanted, bit 1 the body is at rest
     static cudaError_t stage(int s, const GridP &g, const void *in, const void *un, void *out, Ctl *ctl,
@@ -186,6 +203,7 @@ struct Impl {
         a.rest = flags >> 1 & 1;
         a.early = 0;   // set with the tile size
         a.next = next;
+        a.late = 0;    // likewise
         if (s == 1) return stage_s<1>(g, a, st);
         if (s == 2) return stage_s<2>(g, a, st);
         return stage_s<3>(g, a, st);

@@ -961,6 +961,7 @@ struct StageArgs {
                         // of CTAs), those that read no cell of the seeding box load and compute their
                         // faces before waiting for it
     int next;           // ... the seeding box is ctl->rnext (its finalize runs in the seeding launch)
+    int late;           // the next launch starts when this one ends
 };
 
 // Whether a tile's loaded cells (the tile and its halo of 3, after boundary
@@ -1432,8 +1433,8 @@ __global__ void __launch_bounds__(Tile<DIM, V>::THREADS, stage_min_ctas<R, DIM, 
     k_stage(StageArgs a, GridP g)
 {
     // stage 1 after the seeding waits inside stage_tile (early tiles late)
-    if (STAGE == 1 && a.early > 0) pdl_release();
-    else pdl_enter();
+    if (!(STAGE == 1 && a.early > 0)) pdl_wait();
+    if (!a.late) pdl_release();
     const long long tile = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
     const long long nt = (long long)gridDim.x * gridDim.y * gridDim.z;
     stage_tile<R, DIM, NMAT, SOLID, STAGE, V>(g, a, blockIdx.x, blockIdx.y, blockIdx.z, tile, nt);
