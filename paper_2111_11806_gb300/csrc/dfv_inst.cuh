@@ -269,21 +269,21 @@ struct Impl {
 };
 
 // Tables of one (precision, dimension, materials): fluids, solids and solids
-// with plastic-strain planes (3-D solids are not built).
+// with plastic-strain planes.  Not built are 3-D solids and the 3-D FP64
+// three-material fluid, whose tile exceeds a CTA's shared memory; every other
+// form is, and a tile that grows beyond it fails the build.
 template <class R, int DIM, int NMAT>
 const Ops *select_ops_nmat(int solid)
 {
-    // a stage tile must fit the 227 KB of shared memory a CTA may have (the
-    // 3-D FP64 three-material fluid does not: not built)
-    constexpr size_t lim = 227u * 1024u;
-    if constexpr (StageSmem<R, DIM, NMAT, 0, 0>::bytes <= lim) {
+    if constexpr (!(sizeof(R) == 8 && DIM == 3 && NMAT == 3)) {
+        static_assert(StageSmem<R, DIM, NMAT, 0, 0>::bytes <= SMEM_CTA, "a fluid's tile fits a CTA");
         if (!solid) return Impl<R, DIM, NMAT, 0>::ops();
     }
     if constexpr (DIM <= 2) {
-        if constexpr (StageSmem<R, DIM, NMAT, 1, 0>::bytes <= lim)
-            if (solid == 1) return Impl<R, DIM, NMAT, 1>::ops();
-        if constexpr (StageSmem<R, DIM, NMAT, 2, 0>::bytes <= lim)
-            if (solid == 2) return Impl<R, DIM, NMAT, 2>::ops();
+        static_assert(StageSmem<R, DIM, NMAT, 1, 0>::bytes <= SMEM_CTA, "a solid's tile fits a CTA");
+        static_assert(StageSmem<R, DIM, NMAT, 2, 0>::bytes <= SMEM_CTA, "a tile with plastic strains fits a CTA");
+        if (solid == 1) return Impl<R, DIM, NMAT, 1>::ops();
+        if (solid == 2) return Impl<R, DIM, NMAT, 2>::ops();
     }
     return nullptr;
 }

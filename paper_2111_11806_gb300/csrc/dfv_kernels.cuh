@@ -61,15 +61,27 @@ struct Box {
     __host__ __device__ static constexpr int stride(int d) { return d == 0 ? 1 : (d == 1 ? BX : BX * BY); }
 };
 
+// the shared memory that a CTA may have
+constexpr size_t SMEM_CTA = 227u * 1024u;
+
+// shared memory of a tile with nsf face arrays
 template <class R, int DIM, int NMAT, int SOLID, int V>
-struct StageSmem {
+__host__ __device__ constexpr size_t stage_smem(int nsf)
+{
     using L = Lay<DIM, NMAT, SOLID>;
     using B = Box<DIM, V>;
+    const size_t floats = (size_t)L::NVAR * B::N + (size_t)nsf * L::NF * B::MAXF;
+    return ((sizeof(R) * floats + 7) & ~(size_t)7) + 4 * 32 * sizeof(double);
+}
+
+template <class R, int DIM, int NMAT, int SOLID, int V>
+struct StageSmem {
     // fluids keep one face array per direction or two in turn, which saves
-    // barriers (solids one: their larger face records would cost occupancy)
-    static constexpr int NSF = (DIM >= 2 && SOLID == 0) ? 2 : 1;
-    static constexpr size_t floats = (size_t)L::NVAR * B::N + (size_t)NSF * L::NF * B::MAXF;
-    static constexpr size_t bytes = ((sizeof(R) * floats + 7) & ~(size_t)7) + 4 * 32 * sizeof(double);
+    // barriers, where two fit (a 3-D FP64 fluid of two materials takes 251 KB
+    // with two, 223 KB with one); solids keep one: their larger face records
+    // would cost occupancy
+    static constexpr int NSF = DIM >= 2 && SOLID == 0 && stage_smem<R, DIM, NMAT, SOLID, V>(2) <= SMEM_CTA ? 2 : 1;
+    static constexpr size_t bytes = stage_smem<R, DIM, NMAT, SOLID, V>(NSF);
 };
 
 // ---------------------------------------------------- compensated sums
@@ -1160,7 +1172,7 @@ __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, i
     using SM = StageSmem<R, DIM, NMAT, SOLID, V>;
     R *sW = reinterpret_cast<R *>(smem_raw);
     R *sF = sW + (size_t)L::NVAR * B::N;
-    double *sred = reinterpret_cast<double *>(smem_raw + ((sizeof(R) * SM::floats + 7) & ~(size_t)7));
+    double *sred = reinterpret_cast<double *>(smem_raw + SM::bytes - 4 * 32 * sizeof(double));
 
     const R *in = reinterpret_cast<const R *>(a.in);
     const R *un = reinterpret_cast<const R *>(a.un);
