@@ -438,6 +438,16 @@ __device__ __forceinline__ float m_rcp(float x)
 __device__ __forceinline__ float m_div(float a, float b) { return __fmul_rn(a, m_rcp(b)); }
 __device__ __forceinline__ double m_div(double a, double b) { return a * m_rcp(b); }
 
+// a/b for a b of any size: the partial density of a material that spreads
+// through cells it was absent from falls by orders of magnitude a cell, down
+// through the subnormals, whose reciprocal overflows
+__device__ __forceinline__ double m_quot(double a, double b)
+{
+    if ((__double2hiint(b) & 0x7fffffff) < 0x00400000) return a / b;   // |b| < 2^-1019
+    return m_div(a, b);
+}
+__device__ __forceinline__ float m_quot(float a, float b) { return m_div(a, b); }
+
 // comparisons on the bits, with those of the ordinary operators: false for a
 // NaN, zero of either sign equal to zero
 __device__ __forceinline__ unsigned long long m_bits(double x) { return (unsigned long long)__double_as_longlong(x); }
@@ -1089,7 +1099,7 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
     // history: specific eps_l = (phi rho eps)_l / (phi rho)_l, 0 without mass
     if constexpr (SOLID == 2) {
 #pragma unroll
-        for (int l = 0; l < NMAT; l++) w[L::IH + l] = ar[l] != T(0) ? q[L::IH + l] * m_rcp(ar[l]) : T(0);
+        for (int l = 0; l < NMAT; l++) w[L::IH + l] = ar[l] != T(0) ? m_quot(q[L::IH + l], ar[l]) : T(0);
     }
 }
 
@@ -1861,7 +1871,7 @@ __device__ __forceinline__ R solid_finish(const GridP &g, double dt, R *o, R &c)
             for (int l = 0; l < NMAT; l++) {
                 w[L::IAR + l] = rhol[l];
                 const R ar = o[L::IAR + l];
-                if constexpr (SOLID == 2) w[L::IH + l] = ar != R(0) ? o[L::IH + l] * m_rcp(ar) : R(0);
+                if constexpr (SOLID == 2) w[L::IH + l] = ar != R(0) ? m_quot(o[L::IH + l], ar) : R(0);
             }
             w[L::IE] = m_fma(numJ, e.J2, num0) * iden;
             double y0, y1;
