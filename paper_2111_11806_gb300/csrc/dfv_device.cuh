@@ -418,13 +418,18 @@ __device__ __forceinline__ double m_store<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float m_store<float>(double x) { return m_narrow(x); }
 
-// 1/x: y (1 + e + e^2), e = 1 - x y
+// 1/x: y (1 + e + e^2), e = 1 - x y; to one unit in the last place for
+// 2^-1022 <= |x| <= 2^1022.  Where the start is 0 or infinite it is the result:
+// infinity for 0 and the subnormals (from 2^-1024 on 1/x would still be a
+// number, see m_quot), 0 for infinity and |x| > 2^1022.
 __device__ __forceinline__ double m_rcp(double x)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    const double r = fma(y, fma(e, e, e), y);
+    const bool edge = ((__double2hiint(y) + 0x00100000) & 0x7fe00000) == 0;   // exponent 0 or all ones
+    return __longlong_as_double(edge ? __double_as_longlong(y) : __double_as_longlong(r));
 }
 __device__ __forceinline__ float m_rcp(float x)
 {
@@ -491,7 +496,8 @@ __device__ __forceinline__ double m_max(double a, double b)
 }
 __device__ __forceinline__ float m_max(float a, float b) { return fmaxf(a, b); }
 
-// sqrt(x): x/sqrt(x), the reciprocal root with the third-order step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2
+// sqrt(x): x/sqrt(x), the reciprocal root with the third-order step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2;
+// to one unit in the last place for every x >= 0
 __device__ __forceinline__ double m_sqrt(double x)
 {
     if (m_pos(x) && m_less(x, 1e-290)) return sqrt(x);   // the start flushes subnormals to 0
@@ -500,20 +506,21 @@ __device__ __forceinline__ double m_sqrt(double x)
     const double c = x * y;
     const double e = fma(-c, y, 1.0);
     const double r = fma(c, e * fma(e, 0.375, 0.5), c);
-    return m_sel(m_zero(x), 0.0, r);
+    return m_sel(m_zero(x) || m_bits(x) == M_INF, x, r);
 }
 
-// sqrt(a/b), b > 0: a / sqrt(a b) with the reciprocal root's start y and its
-// third-order step y (1 + e/2 + 3 e^2/8), e = 1 - a b y^2
+// sqrt(a/b): a / sqrt(a b) with the reciprocal root's start y and its
+// third-order step y (1 + e/2 + 3 e^2/8), e = 1 - a b y^2; to two units in the
+// last place.  Products outside 2^-959 .. 2^993 (and a = 0) take the quotient.
 __device__ __forceinline__ double m_sqrt_ratio(double a, double b)
 {
     const double x = a * b;
+    if ((unsigned)(__double2hiint(x) & 0x7fffffff) - 0x04000000u >= 0x7a000000u) return m_sqrt(m_div(a, b));
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-(x * y), y, 1.0);
     const double c = a * y;
-    const double r = fma(c, e * fma(e, 0.375, 0.5), c);
-    return m_sel(m_zero(x), 0.0, r);
+    return fma(c, e * fma(e, 0.375, 0.5), c);
 }
 __device__ __forceinline__ float m_sqrt_ratio(float a, float b) { return sqrtf(a * m_rcp(b)); }
 
