@@ -106,17 +106,18 @@ __device__ __forceinline__ void gas_prim(const A &a, float r, float mu, float mv
 
 // The wave speeds of a face between (rL, unL, pL) and (rR, unR, pR): Davis'
 // S_L, S_R, the contact S*, and of each side d = S_K - u_K and rho d.  The
-// sound speed is k/sqrt(k rho) with k = rho c^2 = (Gam + 1) p - p_ref: one
-// special function a side.  The contact numerator's products are rounded one
-// by one (a wall face between mirror-image states gets S* = 0 exactly).
+// sound speed is sqrt(k)/sqrt(rho) with k = rho c^2 = (Gam + 1) p - p_ref, so
+// that k and rho alone have to be within FP32's range, not k rho, whose root
+// would be one special function a side less.  The contact numerator's products
+// are rounded one by one (a wall face between mirror-image states gets S* = 0
+// exactly).
 template <class A>
 __device__ __forceinline__ void gas_waves(const A &a, float rL, float unL, float pL, float rR, float unR, float pR,
                                           float &SL, float &SR, float &Ss, float2 &d2, float2 &m2)
 {
     const float2 r2 = gas_f2(rL, rR), un2 = gas_f2(unL, unR);
     const float2 k2 = __ffma2_rn(gas_f2(a.Gam, a.Gam), gas_f2(pL, pR), gas_sub2(gas_f2(pL, pR), gas_f2(a.pref0, a.pref0)));
-    const float2 x2 = __fmul2_rn(k2, r2);
-    const float2 c2 = __fmul2_rn(k2, gas_f2(gas_rsqrt(x2.x), gas_rsqrt(x2.y)));
+    const float2 c2 = __fmul2_rn(gas_f2(sqrtf(k2.x), sqrtf(k2.y)), gas_f2(gas_rsqrt(rL), gas_rsqrt(rR)));
     const float2 lo = gas_sub2(un2, c2), hi = __fadd2_rn(un2, c2);
     SL = fminf(lo.x, lo.y);
     SR = fmaxf(hi.x, hi.y);
