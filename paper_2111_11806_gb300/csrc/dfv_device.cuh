@@ -1620,9 +1620,9 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
 
 // -------------------------------------------------------- plastic return
 
-// cosh(y) and sinh(y)/y of y^2 (>= 0), FP64: their series to 2^-53 below
+// cosh(y) - 1 and sinh(y)/y of y^2 (>= 0), FP64: their series to 2^-53 below
 // y^2 = 0.02 (elastic metals: y is half the yield strain), exp above.
-__device__ __forceinline__ void cosh_sinhc(double y2, double &ch, double &sh)
+__device__ __forceinline__ void coshm1_sinhc(double y2, double &ch, double &sh)
 {
     if (m_less(y2, 0.02)) {
         double c = 1.0 / 3628800.0;                      // 1/10!
@@ -1630,7 +1630,7 @@ __device__ __forceinline__ void cosh_sinhc(double y2, double &ch, double &sh)
         c = fma(c, y2, 1.0 / 720.0);
         c = fma(c, y2, 1.0 / 24.0);
         c = fma(c, y2, 0.5);
-        ch = fma(c, y2, 1.0);
+        ch = c * y2;
         double s = 1.0 / 39916800.0;                     // 1/11!
         s = fma(s, y2, 1.0 / 362880.0);
         s = fma(s, y2, 1.0 / 5040.0);
@@ -1640,26 +1640,23 @@ __device__ __forceinline__ void cosh_sinhc(double y2, double &ch, double &sh)
         return;
     }
     const double y = sqrt(y2), e = exp(y), i = 1.0 / e;
-    ch = 0.5 * (e + i);
+    ch = fma(0.5, e + i, -1.0);
     sh = 0.5 * (e - i) / y;
 }
 
-// exp(x): its series to 2^-53 for |x| < 0.0625, exp otherwise
-__device__ __forceinline__ double exp_near0(double x)
+// exp(x) - 1 for |x| < 0.0625: its series to 2^-53
+__device__ __forceinline__ double expm1_near0(double x)
 {
-    if (m_less(m_abs(x), 0.0625)) {
-        double e = 1.0 / 362880.0;                       // 1/9!
-        e = fma(e, x, 1.0 / 40320.0);
-        e = fma(e, x, 1.0 / 5040.0);
-        e = fma(e, x, 1.0 / 720.0);
-        e = fma(e, x, 1.0 / 120.0);
-        e = fma(e, x, 1.0 / 24.0);
-        e = fma(e, x, 1.0 / 6.0);
-        e = fma(e, x, 0.5);
-        e = fma(e, x, 1.0);
-        return fma(e, x, 1.0);
-    }
-    return exp(x);
+    double e = 1.0 / 362880.0;                           // 1/9!
+    e = fma(e, x, 1.0 / 40320.0);
+    e = fma(e, x, 1.0 / 5040.0);
+    e = fma(e, x, 1.0 / 720.0);
+    e = fma(e, x, 1.0 / 120.0);
+    e = fma(e, x, 1.0 / 24.0);
+    e = fma(e, x, 1.0 / 6.0);
+    e = fma(e, x, 0.5);
+    e = fma(e, x, 1.0);
+    return e * x;
 }
 
 // Perfect plasticity by instantaneous radial return, in FP64: the stored A is
@@ -1697,16 +1694,26 @@ __device__ __forceinline__ double plastic_return_y(const StretchLog<double> &e, 
         A[2][2] = exp(sc * e.d2);
         A[0][1] = A[1][0] = 0.0;
     } else {
-        const double h = 0.5 * sc;
-        double ch, sh;
-        cosh_sinhc(h * h * e.k2, ch, sh);
-        const double m = exp_near0(-h * e.d2);
-        const double q = m * sh * (h * e.q);     // sinh(s k/2)/|(half, b01)|, times the mean stretch
-        ch *= m;
-        A[0][0] = fma(q, e.half, ch);
-        A[1][1] = fma(-q, e.half, ch);
+        const double h = 0.5 * sc, x = -h * e.d2;
+        double ch, sh, q;
+        coshm1_sinhc(h * h * e.k2, ch, sh);
+        // q: sinh(s k/2)/|(half, b01)|, times the mean stretch e^x
+        if (m_less(m_abs(x), 0.03125)) {
+            // stretches near 1 by what they differ from it, each rounded once
+            const double m = expm1_near0(x), s = fma(ch, m, ch + m);   // e^x cosh - 1
+            q = (1.0 + m) * sh * (h * e.q);
+            A[0][0] = 1.0 + fma(q, e.half, s);
+            A[1][1] = 1.0 + fma(-q, e.half, s);
+            A[2][2] = 1.0 + expm1_near0(-2.0 * x);
+        } else {
+            const double m = exp(x);
+            q = m * sh * (h * e.q);
+            ch = fma(ch, m, m);
+            A[0][0] = fma(q, e.half, ch);
+            A[1][1] = fma(-q, e.half, ch);
+            A[2][2] = exp(-2.0 * x);
+        }
         A[0][1] = A[1][0] = q * e.b01;
-        A[2][2] = m_rcp(m * m);
     }
     A[0][2] = A[2][0] = A[1][2] = A[2][1] = 0.0;
     return deps;

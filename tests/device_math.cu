@@ -8,7 +8,7 @@ using namespace dfv;
 
 namespace {
 
-enum { RCP, DIV, QUOT, SQRT, SQRT_RATIO, ARTANH, COSH, SINHC, EXP0, WIDEN, NARROW, MIN, MAX, PRED, LESS, POWER };
+enum { RCP, DIV, QUOT, SQRT, SQRT_RATIO, ARTANH, COSH, SINHC, EXPM1, WIDEN, NARROW, MIN, MAX, PRED, LESS, POWER };
 
 __global__ void k_eval(int id, const double *a, const double *b, double *out, int n)
 {
@@ -23,9 +23,9 @@ __global__ void k_eval(int id, const double *a, const double *b, double *out, in
     case SQRT: r = m_sqrt(x); break;
     case SQRT_RATIO: r = m_sqrt_ratio(x, y); break;
     case ARTANH: r = artanh_ratio(x); break;
-    case COSH: cosh_sinhc(x, r, s); break;
-    case SINHC: cosh_sinhc(x, s, r); break;
-    case EXP0: r = exp_near0(x); break;
+    case COSH: coshm1_sinhc(x, r, s); r += 1.0; break;
+    case SINHC: coshm1_sinhc(x, s, r); break;
+    case EXPM1: r = expm1_near0(x); break;
     case WIDEN: r = m_widen(__uint_as_float((unsigned)__double_as_longlong(x))); break;
     case NARROW: r = __longlong_as_double((long long)__float_as_uint(m_narrow(x))); break;
     case MIN: r = m_min(x, y); break;
