@@ -1770,13 +1770,6 @@ __device__ __forceinline__ void jc_mixture_yield(const GridP &g, const R *w, dou
     y1 = n1 * i;
 }
 
-// End of a step for a cell of a solid's grid (Sec. 2.1.1): the plastic return
-// of the new conserved state o, and the wave speed of the state it leaves
-// (cell_speed).  The reference curves are linear in J^2 (p_ref and rho e_ref
-// by G J^2), and the return scales J^2 by s^2, so that pressure, shear modulus
-// and sound speed before and after it come from one stretch logarithm and one
-// evaluation of the curves (FP64 form: five and four before).  The
-// decomposition and the return are FP64 in both forms.
 // The return of a cell below yield (s = 1) in 2-D: A becomes the unimodular
 // stretch of A A^T = B itself.  A 2 x 2 block's root is (B + d I)/sqrt(T), d its
 // own root's determinant |det A_2| and T = tr B + 2 d, so that with the scale to
@@ -1805,6 +1798,14 @@ __device__ __forceinline__ bool elastic_stretch(double A[3][3])
     return true;
 }
 
+// End of a step for a cell of a solid's grid (Sec. 2.1.1): the plastic return
+// of the new conserved state o, and the wave speed of the state it leaves
+// (cell_speed).  The reference curves are linear in J^2 (p_ref and rho e_ref
+// by G J^2), and the return scales J^2 by s^2, so that pressure, shear modulus
+// and sound speed before and after it come from one stretch logarithm and one
+// evaluation of the curves (FP64 form: five and four before).  Decomposition
+// and return are FP64 in both forms; the FP32 form first asks its own stretch
+// logarithm whether the cell is clearly below yield, where the return is a root.
 template <class R, int DIM, int NMAT, int SOLID>
 __device__ __forceinline__ R solid_finish(const GridP &g, double dt, R *o, R &c)
 {
@@ -1866,9 +1867,10 @@ __device__ __forceinline__ R solid_finish(const GridP &g, double dt, R *o, R &c)
         ed = e;
     } else {
         unpack_A<R, DIM, NMAT, SOLID>(o, Ad);
-        // below yield by more than the error of the FP32 stretch (1e-7 against
-        // yield strains of 1e-4 and more)
-        if (DIM == 2 && !g.any_jc && R(2.4494897) * Gn * m_sqrt(e.J2) <= R(0.99) * Sn && e.J2 < R(0.25))
+        // below yield by more than the error of the FP32 stretch: 1 % and 5e-7, twice
+        // what the roundings of A A^T's terms leave of |dev H| (2e-7 in all), so that
+        // a yield strain of that size takes the FP64 decomposition in every cell
+        if (DIM == 2 && !g.any_jc && R(2.4494897) * Gn * (m_sqrt(e.J2) + R(5e-7)) <= R(0.99) * Sn && e.J2 < R(0.25))
             elastic = elastic_stretch(Ad);
         if (!elastic) stretch_log<double, DIM>(Ad, ed);
     }

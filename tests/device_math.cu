@@ -1,5 +1,7 @@
 // Host entry of the device arithmetic of dfv_device.cuh, function by function,
 // for test_gpu_device_math.py (built there with the library's own flags).
+#include <cstring>
+
 #include <cuda_runtime.h>
 
 #include "dfv_device.cuh"
@@ -37,6 +39,23 @@ __global__ void k_eval(int id, const double *a, const double *b, double *out, in
     out[i] = r;
 }
 
+// the end of a step for a solid's cell at rest, FP32 with a strain plane: A in
+// and out, rho times the strain that the return adds
+__global__ void k_finish(GridP g, float *A, float *strain, int n)
+{
+    using L = Lay<2, 1, 2>;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float o[L::NVAR], c;
+    for (int v = 0; v < L::NVAR; v++) o[v] = 0.f;
+    o[L::IAR] = (float)g.mat[0].rho0;
+    o[L::IE] = 1e5f;
+    for (int k = 0; k < L::NV; k++) o[L::IV + k] = A[(size_t)k * n + i];
+    solid_finish<float, 2, 1, 2>(g, 1e-9, o, c);
+    for (int k = 0; k < L::NV; k++) A[(size_t)k * n + i] = o[L::IV + k];
+    strain[i] = o[L::IH];
+}
+
 }  // namespace
 
 extern "C" int dm_eval(int id, const double *a, const double *b, double *out, int n)
@@ -51,6 +70,35 @@ extern "C" int dm_eval(int id, const double *a, const double *b, double *out, in
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(out, d + 2 * (size_t)n, bytes, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return (int)e;
+}
+
+extern "C" int dm_finish(double rho0, double K0, double G0, double sigY, float *A, float *strain, int n)
+{
+    GridP g;
+    memset(&g, 0, sizeof(g));
+    g.dim = 2;
+    for (int d = 0; d < 3; d++) g.dx[d] = g.inv_dx[d] = 1.0;
+    g.mat[0].kind = 2;
+    g.mat[0].rho0 = rho0;
+    g.mat[0].K0 = K0;
+    g.mat[0].G0 = G0;
+    g.mat[0].alpha = g.mat[0].beta = 1.0;
+    g.mat[0].Gamma0 = 2.0;
+    g.mat[0].sigY = sigY;
+    apply_options(g, 1, 1.6, 0, 0, 0, 0);
+    finish_params(g);
+    float *d = nullptr;
+    const size_t bytes = sizeof(float) * (size_t)n;
+    cudaError_t e = cudaMalloc(&d, 6 * bytes);
+    if (e == cudaSuccess) e = cudaMemcpy(d, A, 5 * bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_finish<<<(n + 255) / 256, 256>>>(g, d, d + 5 * (size_t)n, n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(A, d, 5 * bytes, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(strain, d + 5 * (size_t)n, bytes, cudaMemcpyDeviceToHost);
     cudaFree(d);
     return (int)e;
 }

@@ -25,8 +25,8 @@ pytestmark = pytest.mark.gpu
 
 U = 2.0 ** -53
 HERE = os.path.dirname(os.path.abspath(__file__))
-NAMES = ["rcp", "div", "quot", "sqrt", "sqrt_ratio", "artanh", "cosh", "sinhc", "expm1", "widen", "narrow", "min", "max",
-         "pred", "less", "power"]
+NAMES = ["rcp", "div", "quot", "sqrt", "sqrt_ratio", "artanh", "cosh", "sinhc", "expm1", "widen", "narrow", "min",
+         "max", "pred", "less", "power"]
 INF, NAN = np.inf, np.nan
 TINY, HUGE = np.finfo(float).tiny, np.finfo(float).max
 EDGES = np.array([0.0, 5e-324, 1e-310, TINY, 1e-300, 1e-290, 1e-160, 1.0 - U, 1.0, 1.0 + 2 * U, 3.0, 1e160, 1e300,
@@ -34,12 +34,16 @@ EDGES = np.array([0.0, 5e-324, 1e-310, TINY, 1e-300, 1e-290, 1e-160, 1.0 - U, 1.
 
 
 @pytest.fixture(scope="module")
-def dev(tmp_path_factory):
+def lib(tmp_path_factory):
     from paper_2111_11806_gb300 import _build
     so = str(tmp_path_factory.mktemp("device_math") / "libdevice_math.so")
     subprocess.check_call([_build.nvcc()] + _build.ARCH + _build.FLAGS
                           + ["-I" + _build.CSRC, "-shared", "-o", so, os.path.join(HERE, "device_math.cu"), "-lcudart"])
-    lib = ctypes.CDLL(so)
+    return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def dev(lib):
     dp = ctypes.POINTER(ctypes.c_double)
 
     def call(name, a, b=None):
@@ -160,3 +164,32 @@ def test_comparisons_give_the_values_of_the_operators(dev):
         for name, fn in (("min", np.fmin), ("max", np.fmax)):
             got, want = dev(name, a, b), fn(a, b)
             assert np.all((got == want) | (np.isnan(got) & np.isnan(want)))
+
+
+@pytest.mark.parametrize("yield_strain", [1e-3, 1e-5, 4e-7])
+def test_fp32_cells_beyond_a_small_yield_strain_yield(lib, yield_strain):
+    """Stretches of 0.8 to 1.3 times the yield strain, exact in FP32, in the FP32
+    form: the plastic strain is that of the FP64 return (its factor 1 - s by the
+    FP32 rounding of G, 1e-7; allowed 1e-6 of |dev H|), none below yield."""
+    n, G0, rho0 = 20000, 26e9, 2700.0
+    rng = np.random.default_rng(14)
+    d = rng.standard_normal((5, n))
+    d[4] = -(d[0] + d[3])
+    d *= yield_strain * rng.uniform(0.8, 1.3, n) / np.sqrt(d[0] ** 2 + d[3] ** 2 + d[4] ** 2 + (d[1] + d[2]) ** 2 / 2)
+    A = np.ascontiguousarray(d + np.array([1, 0, 0, 1, 1])[:, None], dtype=np.float32)
+    a = A.astype(np.longdouble)
+    # |dev ln V| by the eigenvalues of the in-plane block of A A^T less 1
+    b00 = (a[0] - 1) * (a[0] + 1) + a[1] ** 2
+    b11 = (a[3] - 1) * (a[3] + 1) + a[2] ** 2
+    b01 = a[0] * a[2] + a[1] * a[3]
+    mid, rad = (b00 + b11) / 2, np.sqrt(((b00 - b11) / 2) ** 2 + b01 ** 2)
+    h = np.array([np.log1p(mid + rad), np.log1p(mid - rad), np.log1p((a[4] - 1) * (a[4] + 1))]) / 2
+    norm = np.sqrt(((h - h.mean(axis=0)) ** 2).sum(axis=0))
+    sig_y = np.sqrt(6.0) * G0 * yield_strain
+    want = np.sqrt(np.longdouble(2) / 3) * np.maximum(norm - yield_strain, 0)
+    strain = np.empty(n, dtype=np.float32)
+    fp = ctypes.POINTER(ctypes.c_float)
+    lib.dm_finish.argtypes = [ctypes.c_double] * 4 + [fp, fp, ctypes.c_int]
+    assert lib.dm_finish(rho0, 76e9, G0, sig_y, A.ctypes.data_as(fp), strain.ctypes.data_as(fp), n) == 0
+    assert np.any(want > 0) and np.any(want == 0)
+    assert np.all(np.abs(strain / rho0 - want) <= 1e-6 * norm)
