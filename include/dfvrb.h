@@ -298,11 +298,14 @@ dfv_status dfv_batch_get_fields(dfv_batch *b, int i, double *out, int which, int
 /* The same for every instance in one call (Sec. 4 setup of many independent
  * problems): prim[i] / out[i] (count pointers, caller-owned, host or device
  * as on_device says) hold instance i's nvar FP64 planes of n[0] n[1] values.
- * The call returns when everything is copied and converted (host buffers may
- * then be reused). Device and page-locked host buffers are converted in place,
- * 256 instances a launch; where an instance's buffer is pageable, copies and
- * conversions go instance by instance through the staging area. DFV_ERR_ARG for a null pointer (nothing is copied) or,
- * when reading, an instance whose fields were never set. */
+ * With host buffers the call returns when everything is copied and converted
+ * (they may then be reused); with on_device it is only enqueued on the batch's
+ * stream, and the buffers have to stay valid, and be ordered against other
+ * streams by the caller, until that stream has passed it. Device and page-locked
+ * host buffers are converted in place, 256 instances a launch; where an
+ * instance's buffer is pageable, copies and conversions go instance by instance
+ * through the staging area. DFV_ERR_ARG for a null pointer (nothing is copied)
+ * or, when reading, an instance whose fields were never set. */
 dfv_status dfv_batch_set_all_fields(dfv_batch *b, const double *const *prim, int on_device);
 dfv_status dfv_batch_get_all_fields(dfv_batch *b, double *const *out, int which, int on_device);
 /* `steps` steps of every instance, each with its own dt = cfl / (its CFL
