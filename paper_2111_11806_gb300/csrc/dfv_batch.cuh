@@ -13,7 +13,6 @@ namespace dfv {
 struct BatchInst {
     GridP g;            // the instance's grid and materials (pitch: its own)
     long long off;      // element offset of its planes in the state arrays
-    long long part0;    // its first slot in the partials array (4 doubles each)
     int tiles_x, tiles_y, ntiles, rest;   // rest: its body does not move
     Ctl *ctl;           // its control block (dt, t, smax, error word)
 };
@@ -25,7 +24,6 @@ struct BatchArgs {
     const BatchInst *inst;
     const int2 *items;       // (instance, tile) in the order of the schedule
     long long nitems;
-    double *partials;
     int final_mode;          // mode of the finalize phase (after stage 3 or a CFL reduction)
     unsigned int *queue;     // dynamic schedule: next item counter (nullptr: static round-robin)
 };
@@ -77,12 +75,13 @@ __global__ void __launch_bounds__(Tile<2, 0>::THREADS, (sizeof(R) == 4 && NMAT =
         a.un = reinterpret_cast<const R *>(b.un) + I.off;
         a.out = reinterpret_cast<R *>(b.out) + I.off;
         a.ctl = I.ctl;
-        a.partials = b.partials + 4 * I.part0;
+        a.partials = nullptr;   // no force is wanted
         a.want_force = 0;
         a.rest = I.rest;
         a.early = 0;
         a.next = 0;
-        stage_tile<R, 2, NMAT, 0, STAGE, 0>(I.g, a, w.y % I.tiles_x, w.y / I.tiles_x, 0, w.y, I.ntiles);
+        a.late = 0;
+        stage_tile<R, 2, NMAT, 0, STAGE, 0>(I.g, a, w.y % I.tiles_x, w.y / I.tiles_x, 0, w.y);
     }
 }
 
@@ -158,8 +157,7 @@ __global__ void __launch_bounds__(THREADS) k_batch_finalize(BatchArgs b)
     pdl_enter();
     __shared__ double sred[4 * 32];
     const BatchInst &I = b.inst[blockIdx.x];
-    finalize_block<THREADS>(I.ctl, b.partials + 4 * I.part0, 0, 0, b.final_mode, 2, I.g.dx[0], I.g.dx[1],
-                            I.g.dx[2], sred);
+    finalize_block<THREADS>(I.ctl, nullptr, 0, 0, b.final_mode, 2, I.g.dx[0], I.g.dx[1], I.g.dx[2], sred);
     // the stages of this step are complete: reset the dynamic-schedule counters
     if (blockIdx.x == 0 && threadIdx.x == 0 && b.queue)
         for (int k = 1; k <= 3; k++) b.queue[k] = 0u;

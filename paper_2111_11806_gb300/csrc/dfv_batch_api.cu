@@ -28,12 +28,12 @@ namespace {
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Plan {
-    size_t off_inst, off_items0, off_items1, off_ctl, off_ctlbak, off_part, off_queue, off_vbody;
+    size_t off_inst, off_items0, off_items1, off_ctl, off_ctlbak, off_queue, off_vbody;
     size_t off_ginst, off_gitems0, off_gitems1;   // the gas stage kernel's records
     size_t off_U, off_U1, off_U3, off_Ubak, off_stage, total;
-    long long elems, nitems, max_cells, ntiles_total, gas_nitems;
+    long long elems, nitems, max_cells, gas_nitems;
     int gas_rows;
-    std::vector<long long> inst_off, inst_part0;
+    std::vector<long long> inst_off;
     std::vector<int> tiles_x, tiles_y;
 };
 
@@ -50,7 +50,6 @@ bool plan_batch(int count, const dfv_instance_desc *desc, int precision, int nma
     P.nitems = 0;
     P.max_cells = 0;
     P.inst_off.resize(count);
-    P.inst_part0.resize(count);
     P.tiles_x.resize(count);
     P.tiles_y.resize(count);
     for (int i = 0; i < count; i++) {
@@ -61,7 +60,6 @@ bool plan_batch(int count, const dfv_instance_desc *desc, int precision, int nma
         P.elems += nvar * pitch;
         P.tiles_x[i] = (desc[i].n[0] + BatchTile::TX - 1) / BatchTile::TX;
         P.tiles_y[i] = (desc[i].n[1] + BatchTile::TY - 1) / BatchTile::TY;
-        P.inst_part0[i] = P.nitems;
         P.nitems += (long long)P.tiles_x[i] * P.tiles_y[i];
         P.max_cells = std::max(P.max_cells, nc);
     }
@@ -72,7 +70,6 @@ bool plan_batch(int count, const dfv_instance_desc *desc, int precision, int nma
     P.gas_nitems = 0;
     for (int i = 0; i < count; i++)
         P.gas_nitems += (long long)dfv::gasw_strips(desc[i].n[0]) * ((desc[i].n[1] + P.gas_rows - 1) / P.gas_rows);
-    P.ntiles_total = P.nitems;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
@@ -84,7 +81,6 @@ bool plan_batch(int count, const dfv_instance_desc *desc, int precision, int nma
     P.off_items1 = take(sizeof(int2) * P.nitems);
     P.off_ctl = take(256 * (size_t)count);
     P.off_ctlbak = take(256 * (size_t)count);
-    P.off_part = take(sizeof(double) * 4 * P.nitems);
     P.off_queue = take(sizeof(unsigned int) * 8);
     P.off_vbody = take(sizeof(double) * 3 * count);
     P.off_ginst = take(sizeof(dfv::GasInst) * count);
@@ -121,7 +117,7 @@ struct dfv_batch {
     BatchInst *d_inst = nullptr;
     int2 *d_items[2] = {nullptr, nullptr};
     Ctl *d_ctl = nullptr, *d_ctl_bak = nullptr;
-    double *d_part = nullptr, *d_vbody = nullptr, *staging = nullptr;
+    double *d_vbody = nullptr, *staging = nullptr;
     unsigned int *d_queue = nullptr;
     void *U = nullptr, *U1 = nullptr, *U3 = nullptr, *Ubak = nullptr;
     int sm_count = 152, ctas_per_sm = 1, max_ctas = 1;
@@ -180,7 +176,6 @@ BatchArgs args(dfv_batch *b, const void *in, const void *un, void *out, int fina
     a.inst = b->d_inst;
     a.items = b->d_items[b->schedule == 0 ? 0 : 1];
     a.nitems = b->plan.nitems;
-    a.partials = b->d_part;
     a.final_mode = final_mode;
     a.queue = nullptr;
     return a;
@@ -360,7 +355,6 @@ dfv_status dfv_batch_create(int dim, int count, const dfv_instance_desc *desc, i
     b->d_items[1] = (int2 *)(b->ws + P.off_items1);
     b->d_ctl = (Ctl *)(b->ws + P.off_ctl);
     b->d_ctl_bak = (Ctl *)(b->ws + P.off_ctlbak);
-    b->d_part = (double *)(b->ws + P.off_part);
     b->d_queue = (unsigned int *)(b->ws + P.off_queue);
     if (cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned int) * 8, b->stream) != cudaSuccess) {
         delete b;
@@ -401,7 +395,6 @@ dfv_status dfv_batch_create(int dim, int count, const dfv_instance_desc *desc, i
         dfv::apply_options(p, opt->use_thinc, opt->thinc_beta, opt->hllc_lm, opt->seed_variant,
                        opt->normal_method, opt->probe_mode);
         I.off = P.inst_off[i];
-        I.part0 = P.inst_part0[i];
         I.tiles_x = P.tiles_x[i];
         I.tiles_y = P.tiles_y[i];
         I.ntiles = P.tiles_x[i] * P.tiles_y[i];

@@ -227,7 +227,7 @@ struct Ctl {
     int auto_dt;              // 1: the finalize kernel sets the next dt from cfl
     unsigned int err;         // bit 0: rho<=0/NaN in an update, bit 1: c^2<=0/NaN
     int steps;
-    unsigned int ticket;      // not used (its place in the block stays)
+    unsigned int pad;
     float dtf, vf[3];         // dt and v in single precision, kept equal to (float)dt, (float)v
     int rbox_valid;           // 1: rbox bounds every cell with r > 0.5 of the stored state
     int rbox[6];              // inclusive cell-index box lo x, y, z, hi x, y, z (empty: lo > hi)

@@ -105,8 +105,10 @@ struct Impl {
     static cudaError_t prepare_v()
     {
         cudaError_t e = opt_in(k_stage<R, DIM, NMAT, SOLID, 1, V>, smem<V>);
-        if (e == cudaSuccess) e = opt_in(k_stage<R, DIM, NMAT, SOLID, 2, V>, smem<V>);
-        if (e == cudaSuccess) e = opt_in(k_stage<R, DIM, NMAT, SOLID, 3, V>, smem<V>);
+        if constexpr (!ZM) {
+            if (e == cudaSuccess) e = opt_in(k_stage<R, DIM, NMAT, SOLID, 2, V>, smem<V>);
+            if (e == cudaSuccess) e = opt_in(k_stage<R, DIM, NMAT, SOLID, 3, V>, smem<V>);
+        }
         // the first-wave size is looked up here, outside any stream capture
         if (e == cudaSuccess) (void)first_wave<V>();
         return e;
@@ -137,19 +139,26 @@ struct Impl {
     }
 
     template <int S>
+    static cudaError_t march(const GridP &g, const StageArgs &a, cudaStream_t st)
+    {
+        const int zc = zchunk(g, a.rest);
+        const dim3 b(ZGeo<R>::THREADS);
+        return a.rest ? launch_pdl(k_stage_z<R, NMAT, S, true>, zgrid(g, zc), b, zsmem, st, a, g, zc)
+                      : launch_pdl(k_stage_z<R, NMAT, S, false>, zgrid(g, zc), b, zsmem, st, a, g, zc);
+    }
+
+    template <int S>
     static cudaError_t stage_s(const GridP &g, const StageArgs &a, cudaStream_t st)
     {
-        if constexpr (ZM) {
-            if (!(S == 1 && a.want_force)) {
-                const int zc = zchunk(g, a.rest);
-                const dim3 b(ZGeo<R>::THREADS);
-                return a.rest ? launch_pdl(k_stage_z<R, NMAT, S, true>, zgrid(g, zc), b, zsmem, st, a, g, zc)
-                              : launch_pdl(k_stage_z<R, NMAT, S, false>, zgrid(g, zc), b, zsmem, st, a, g, zc);
-            }
+        if constexpr (ZM && S != 1) {
+            return march<S>(g, a, st);
+        } else {
+            if constexpr (ZM)
+                if (!a.want_force) return march<S>(g, a, st);
+            if constexpr (NV == 2)
+                if (small_tiles(g)) return stage_v<S, 1>(g, a, st);
+            return stage_v<S, 0>(g, a, st);
         }
-        if constexpr (NV == 2)
-            if (small_tiles(g)) return stage_v<S, 1>(g, a, st);
-        return stage_v<S, 0>(g, a, st);
     }
 
     // CTAs of the stage-1 kernel resident at once on the device (the first

@@ -11,7 +11,8 @@
 //   k_finalize  one block: deterministic sums of the per-block partials,
 //               body update, next dt (k_finalize_lite: one warp, no partials)
 //   k_prim_to_cons / k_cons_to_prim / k_cons_to_f64   field conversion
-// The 3-D FP32 single-material stages march along z instead (dfv_kernels_z.cuh).
+// The 3-D single-material stages march along z instead (dfv_kernels_z.cuh), but
+// for the stage 1 that sums the pressure force.
 #pragma once
 
 #include "dfv_device.cuh"
@@ -23,7 +24,7 @@ namespace dfv {
 // Tile of one CTA: TX x TY x TZ cells, one thread each, and as many extra
 // threads as a sweep has pencils at most, which do their closing faces.  V
 // selects the size: 0 the large one, whose halo costs least, 1 the small one,
-// for FP64 grids of few large tiles (small_tiles says when).
+// for 1-D grids and FP64 2-D grids of few large tiles (small_tiles says when).
 template <int DIM, int V>
 struct Tile;
 template <>
@@ -1159,11 +1160,11 @@ __device__ __forceinline__ void accum_pass(const GridP &g, const R *sW, const R 
 }
 
 // One tile of one SSP-RK3 stage, executed by a whole CTA: (tbx, tby, tbz) is
-// the tile position in tile units, tile_id its index among the ntiles tiles of
-// the grid (partials slot; the last of them to finish runs the finalize).
+// the tile position in tile units, tile_id its index among the tiles of the
+// grid (its slot of the force partials).
 template <class R, int DIM, int NMAT, int SOLID, int STAGE, int V>
 __device__ __forceinline__ void stage_tile(const GridP &g, const StageArgs &a, int tbx, int tby, int tbz,
-                                           long long tile_id, long long ntiles)
+                                           long long tile_id)
 {
     using L = Lay<DIM, NMAT, SOLID>;
     using B = Box<DIM, V>;
@@ -1448,8 +1449,7 @@ __global__ void __launch_bounds__(Tile<DIM, V>::THREADS, stage_min_ctas<R, DIM, 
     if (!(STAGE == 1 && a.early > 0)) pdl_wait();
     if (!a.late) pdl_release();
     const long long tile = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-    const long long nt = (long long)gridDim.x * gridDim.y * gridDim.z;
-    stage_tile<R, DIM, NMAT, SOLID, STAGE, V>(g, a, blockIdx.x, blockIdx.y, blockIdx.z, tile, nt);
+    stage_tile<R, DIM, NMAT, SOLID, STAGE, V>(g, a, blockIdx.x, blockIdx.y, blockIdx.z, tile);
 }
 
 // ------------------------------------------------------------------ CFL
