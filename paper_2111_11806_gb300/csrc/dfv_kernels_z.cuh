@@ -214,7 +214,8 @@ __device__ __forceinline__ void z_slope_z(const GridP &g, const R *in, const R *
 // REST: the body is at rest (no r to reconstruct).  Two CTAs per SM in FP64
 // (ring and face arrays 106 KB), three in FP32; a moving body's FP64 kernel
 // takes the registers of one CTA instead, since with the BVD choice of r it
-// would spill 600 bytes a thread.  Measured in FP64 over two steps: sphere
+// would spill 600 bytes a thread (105 in stage 3 as it is, 300 at rest, of the
+// 168 and 96 registers that the CTAs leave).  Measured in FP64 over two steps: sphere
 // 52 x 70 x 59 moving 7172 us with two CTAs, 4500 with one; 97 x 90 x 101 at
 // rest 7236 with one, 6668 with two, 6385 since REST is known at compile time.
 template <class R, int NMAT, int STAGE, bool REST>

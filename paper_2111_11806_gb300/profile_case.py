@@ -17,7 +17,7 @@ if ROOT not in sys.path:
 
 def main(argv=None):
     ap = argparse.ArgumentParser()
-    ap.add_argument("--workload", default="cylinder", choices=["cylinder", "dynamic", "impact", "sphere"])
+    ap.add_argument("--workload", default="cylinder", choices=["cylinder", "dynamic", "impact", "copper", "sphere"])
     ap.add_argument("--n", type=int, default=4096)
     ap.add_argument("--precision", default="fp32", choices=["fp32", "fp64"])
     ap.add_argument("--steps", type=int, default=3)
@@ -30,7 +30,8 @@ def main(argv=None):
     from paper_2111_11806_gb300 import binding as B
     B.load()
     make = {"cylinder": lambda n: W.cylinder_2d(n), "dynamic": lambda n: W.dynamic_body_2d(n, n // 2),
-            "impact": lambda n: W.impact_2d(n), "sphere": lambda n: W.sphere_3d(n)}[args.workload]
+            "impact": lambda n: W.impact_2d(n),
+            "copper": lambda n: W.with_history(W.impact_2d(n, solid_material=W.COPPER)), "sphere": lambda n: W.sphere_3d(n)}[args.workload]
     wl = make(args.n)
     prec = B.DFV_FP32 if args.precision == "fp32" else B.DFV_FP64
     stream = torch.cuda.Stream()
