@@ -470,6 +470,7 @@ __device__ __forceinline__ bool m_over1(double x)                               
 }
 __device__ __forceinline__ bool m_over1(float x) { return x > 1.f; }
 __device__ __forceinline__ bool m_nan(double x) { return (__double2hiint(x) & 0x7fffffff) >= 0x7ff80000; }  // quiet NaN
+__device__ __forceinline__ bool m_nan(float x) { return x != x; }
 // whether a < b, neither a NaN; the bits of doubles, negative ones with their magnitude inverted, order like them
 __device__ __forceinline__ long long m_key(double x)
 {
@@ -1319,7 +1320,9 @@ __device__ __forceinline__ void recon_cell(const GridP &g, const T *s, bool frac
     thinc<T>(g, s[2], s[3], s[4], tCm, tCp);
     const T tbvBM = m_abs(Ap - Bm) + m_abs(Bp - Cm);
     const T tbvBT = m_abs(tAp - tBm) + m_abs(tBp - tCm);
-    if (m_less(tbvBT, tbvBM)) {
+    // (at a steepness from about 19 on tanh beta is 1 in FP64 and a profile's end value can be 0/0: the variation is
+    // then a NaN, and MUSCL's values stand)
+    if (!m_nan(tbvBT) && m_less(tbvBT, tbvBM)) {
         lo = tBm;
         hi = tBp;
     }
