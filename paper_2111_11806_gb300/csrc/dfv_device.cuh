@@ -419,15 +419,27 @@ template <>
 __device__ __forceinline__ float m_store<float>(double x) { return m_narrow(x); }
 
 // 1/x: y (1 + e + e^2), e = 1 - x y; to one unit in the last place for
-// 2^-1022 <= |x| <= 2^1022.  Where the start is 0 or infinite it is the result:
-// infinity for 0 and the subnormals (from 2^-1024 on 1/x would still be a
-// number, see m_quot), 0 for infinity and |x| > 2^1022.
+// 2^-1022 <= |x| <= 2^1022.  m_rcp: where the start is 0 or infinite it is the
+// result: infinity for 0 and the subnormals (from 2^-1024 on 1/x would still be
+// a number, see m_quot), 0 for infinity and |x| > 2^1022.  m_rcp_normal: NaN
+// there, for a cell's density and the differences of a face's wave speeds, from
+// which a 0 makes no state either way (1-D grids, where few warps wait for each
+// other's chains, 2113 us a pass of tube 400 against 2176 with m_rcp).
+__device__ __forceinline__ double m_rcp_step(double x, double &y)
+{
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double m_rcp_normal(double x)
+{
+    double y;
+    return m_rcp_step(x, y);
+}
 __device__ __forceinline__ double m_rcp(double x)
 {
     double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    const double r = fma(y, fma(e, e, e), y);
+    const double r = m_rcp_step(x, y);
     const bool edge = ((__double2hiint(y) + 0x00100000) & 0x7fe00000) == 0;   // exponent 0 or all ones
     return __longlong_as_double(edge ? __double_as_longlong(y) : __double_as_longlong(r));
 }
@@ -437,6 +449,7 @@ __device__ __forceinline__ float m_rcp(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+__device__ __forceinline__ float m_rcp_normal(float x) { return m_rcp(x); }
 
 // a/b (FP32: the product with the approximate reciprocal, rounded on its own --
 // what the fast division gives over the normal range, without its range fix-up)
@@ -1051,7 +1064,7 @@ __device__ __forceinline__ void cons_to_prim_ct(const GridP &g, const T *q, T *w
         return;
     }
     T u[DIM], mu = T(0);
-    const T irho = m_rcp(rho);
+    const T irho = m_rcp_normal(rho);
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
         u[a] = q[L::IMOM + a] * irho;
@@ -1500,7 +1513,7 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
     const T dL = SL - uL, dR = SR - uR;
     const T mL = mul_rn(sl.rho, dL), mR = mul_rn(sr.rho, dR);
     const T num = add_rn(add_rn(TR - TL, mul_rn(mL, uL)), -mul_rn(mR, uR));
-    const T Ss = num * m_rcp(mL - mR);
+    const T Ss = num * m_rcp_normal(mL - mR);
     // regions: left of S_L, left star, right star, right of S_R
     const bool all_left = m_ge0(SL);
     const bool left = all_left || m_ge0(Ss);
@@ -1558,7 +1571,7 @@ __device__ __forceinline__ void riemann(const GridP &g, const T *wL, const T *wR
     // cS: transport velocity of the upwind side's contents (rho* S*/rho_K, or u_K)
     T cS, Tf, EF;
     if (star) {
-        const T iD = m_rcp(SK - Ss);
+        const T iD = m_rcp_normal(SK - Ss);
         cS = dK * iD * Ss;
         Tf = m_fma(mK, Ss - uK, TK);
         const T Es = m_fma(dK, EK, m_fma(Tf, Ss, -(TK * uK))) * iD;
